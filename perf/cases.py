@@ -340,7 +340,9 @@ def tolerance(case):
     """Codes and scales of the inputs are defined bit by bit.  A 16-bit output
     is the rounding of an fp32 sum: it is within half a unit of the last place
     of the exact product (relative 2-norm 1.7e-3 for bf16, 2.1e-4 for fp16),
-    and two orders of summation differ in a few roundings."""
+    and two orders of summation differ in a few roundings (against the exact
+    product rounded to bf16, 1e-5 of one layer's outputs and 3e-4 of two
+    chained layers' measured different)."""
     kind = case["kind"]
     if kind in ("quantize", "weight"):
         return "exact"
@@ -349,7 +351,7 @@ def tolerance(case):
     if kind in ("translator", "stack"):
         # the second layer's input codes may differ where a rounding of the
         # first layer's output does
-        return {"rel": 1.5e-2, "max": 0.5, "differ": 1e-2}
+        return {"rel": 7e-3, "max": 0.1, "differ": 2e-3}
     return {"rel": 6e-3, "max": 3e-2, "differ": 1e-3}
 
 
