@@ -333,6 +333,21 @@ __device__ __forceinline__ void mma_nvfp4_pair(uint32_t d_tmem, uint64_t a_desc,
       : "memory");
 }
 
+// Same with K = 96 per instruction (six scales per row; idesc_nvfp4_k96): the
+// same 128 cycles at N = 256 as K = 64.
+__device__ __forceinline__ void mma_nvfp4_k96_pair(uint32_t d_tmem, uint64_t a_desc,
+                                                   uint64_t b_desc, uint32_t idesc,
+                                                   uint32_t sfa_tmem, uint32_t sfb_tmem,
+                                                   uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::mxf4nvf4.block_scale.block16"
+      " [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem)
+      : "memory");
+}
+
 __device__ __forceinline__ void mma_fp8_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                              uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -415,6 +430,19 @@ __device__ __forceinline__ void mma_nvfp4(uint32_t d_tmem, uint64_t a_desc, uint
       : "memory");
 }
 
+// Same with K = 96 per instruction (idesc_nvfp4_k96).
+__device__ __forceinline__ void mma_nvfp4_k96(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                              uint32_t idesc, uint32_t sfa_tmem,
+                                              uint32_t sfb_tmem, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::mxf4nvf4.block_scale.block16"
+      " [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem)
+      : "memory");
+}
+
 // D[tmem] (+)= A[smem] * B[smem]^T with E4M3 operands, K = 32 per instruction.
 __device__ __forceinline__ void mma_fp8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                         uint32_t idesc, uint32_t accumulate) {
@@ -444,6 +472,12 @@ __host__ __device__ constexpr uint32_t idesc_nvfp4(int n, int m = 128) {
          | ((uint32_t)(n >> 3) << 17)   // N / 8
          | (0u << 23)                   // scale type: UE4M3
          | ((uint32_t)(m >> 4) << 24);  // M / 16
+}
+
+// The same with K = 96 (sm_103a): six scales per row and operand, read from
+// byte sf_id (0 or 2) of the scale column group given and from the next group.
+__host__ __device__ constexpr uint32_t idesc_nvfp4_k96(int n, int m, int sf_id) {
+  return idesc_nvfp4(n, m) | (1u << 31) | ((uint32_t)sf_id << 29) | ((uint32_t)sf_id << 4);
 }
 
 // Instruction descriptor, kind::f8f6f4: E4M3 A and B, fp32 accumulator.

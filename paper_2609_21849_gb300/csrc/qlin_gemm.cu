@@ -111,8 +111,13 @@ struct Cfg {
   static constexpr int kStagesRaw = (kSmemBudget - kOutBytes) / kStageBytes;
   static constexpr int kStages = kStagesRaw > 8 ? 8 : kStagesRaw;
   static constexpr int kNumAcc = (kFp4 && kBN == 256) ? 1 : 2;
-  static constexpr int kSfColsPerStep = kFp4 ? 4 + 4 * kSfbAtoms : 0;
+  // Scale columns of one stage: A's (4 per 64 elements of K), then W's (4 per
+  // 64 elements and 128-row atom), each operand's groups of 64 elements side
+  // by side, because a K = 96 MMA reads two neighbouring groups.
+  static constexpr int kSfaCols = 4, kSfbCols = 4 * kSfbAtoms;
+  static constexpr int kSfColsPerStep = kFp4 ? kSfaCols + kSfbCols : 0;
   static constexpr int kSfColBase = kNumAcc * kBN;
+  static constexpr bool kK96 = kFp4 && kBN >= 128;
   static constexpr int kTmemCols =
       pow2_at_least(kSfColBase + kStages * kStepsPerStage * kSfColsPerStep);
   static constexpr int kBarrierBytes = 512;
@@ -414,15 +419,17 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           const uint64_t adesc0 = sdesc_k128(sA), bdesc0 = sdesc_k128(sB);
           const uint32_t sfa0 = tmem_base + (uint32_t)(C::kSfColBase + stage * kStepsPerStage *
                                                                            C::kSfColsPerStep);
+          const uint32_t sfb0 = sfa0 + (uint32_t)(kStepsPerStage * C::kSfaCols) + sfb_off;
           auto issue = [&](int j, uint32_t accumulate) {
             const uint64_t adesc = adesc0 + (uint64_t)(2 * j);
             const uint64_t bdesc = bdesc0 + (uint64_t)(2 * j);
             if (kFp4) {
-              const uint32_t sfa_t = sfa0 + (uint32_t)(j * C::kSfColsPerStep);
+              const uint32_t sfa_t = sfa0 + (uint32_t)(j * C::kSfaCols);
+              const uint32_t sfb_t = sfb0 + (uint32_t)(j * C::kSfbCols);
               if (kPair)
-                mma_nvfp4_pair(d_tmem, adesc, bdesc, idesc, sfa_t, sfa_t + 4, accumulate);
+                mma_nvfp4_pair(d_tmem, adesc, bdesc, idesc, sfa_t, sfb_t, accumulate);
               else
-                mma_nvfp4(d_tmem, adesc, bdesc, idesc, sfa_t, sfa_t + 4 + sfb_off, accumulate);
+                mma_nvfp4(d_tmem, adesc, bdesc, idesc, sfa_t, sfb_t, accumulate);
             } else if (kBf16) {
               if (kPair)
                 mma_bf16_pair(d_tmem, adesc, bdesc, idesc, accumulate);
@@ -435,11 +442,32 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
                 mma_fp8(d_tmem, adesc, bdesc, idesc, accumulate);
             }
           };
+          // NVFP4: elements 96 h .. 96 h + 95 of the stage (48 bytes in) in one
+          // K = 96 MMA; its six scales start at group 0 byte 0 (h = 0) or
+          // group 1 byte 2 (h = 1)
+          auto issue96 = [&](int h, uint32_t accumulate) {
+            if constexpr (C::kK96) {
+              const uint64_t adesc = adesc0 + (uint64_t)(3 * h), bdesc = bdesc0 + (uint64_t)(3 * h);
+              const uint32_t sfa_t = sfa0 + (uint32_t)(h * C::kSfaCols);
+              const uint32_t sfb_t = sfb0 + (uint32_t)(h * C::kSfbCols);
+              const uint32_t id = idesc_nvfp4_k96(kBN, kMmaM, 2 * h);
+              if (kPair)
+                mma_nvfp4_k96_pair(d_tmem, adesc, bdesc, id, sfa_t, sfb_t, accumulate);
+              else
+                mma_nvfp4_k96(d_tmem, adesc, bdesc, id, sfa_t, sfb_t, accumulate);
+            }
+          };
           // Full stages issue their MMAs unrolled, with no branch between
           // them: a runtime step loop around the MMA issue costs ~100 cycles
           // a stage (measured), a fifth of the stage's tensor work.  Only a
           // partial last stage (K % 256 != 0) takes the loop.
-          if (nsteps == kStepsPerStage) {
+          if (C::kK96 && nsteps >= 3) {
+            // K = 256 as 96 + 96 + 64, K = 192 as 96 + 96: an MMA of K = 96
+            // takes the time of one of K = 64
+            issue96(0, kb > 0 ? 1u : 0u);
+            issue96(1, 1u);
+            if (nsteps == kStepsPerStage) issue(3, 1u);
+          } else if (nsteps == kStepsPerStage) {
             issue(0, kb > 0 ? 1u : 0u);
 #pragma unroll
             for (int jj = 1; jj < kStepsPerStage; ++jj) issue(jj, 1u);
@@ -521,9 +549,10 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           constexpr int kShare = kStepsPerStage / C::kCpWarps;
           const int j_end = min(nsteps, (sw + 1) * kShare);
           for (int j = sw * kShare; j < j_end; ++j) {
-            const uint32_t sfa_t = tmem_base + (uint32_t)(C::kSfColBase +
-                                                          (stage * kStepsPerStage + j) *
-                                                              C::kSfColsPerStep);
+            const uint32_t sf0 = tmem_base + (uint32_t)(C::kSfColBase +
+                                                        stage * kStepsPerStage * C::kSfColsPerStep);
+            const uint32_t sfa_t = sf0 + (uint32_t)(j * C::kSfaCols);
+            const uint32_t sfb_t = sf0 + (uint32_t)(kStepsPerStage * C::kSfaCols + j * C::kSfbCols);
             if (kPair)
               tc_cp_scales_pair(sfa_t, sdesc_scales(sSFA + j * 512));
             else
@@ -532,9 +561,9 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
             for (int r = 0; r < C::kSfbAtoms; ++r) {
               const uint32_t src = sSFB + r * kStepsPerStage * 512 + j * 512;
               if (kPair)
-                tc_cp_scales_pair(sfa_t + 4 + 4 * r, sdesc_scales(src));
+                tc_cp_scales_pair(sfb_t + 4 * r, sdesc_scales(src));
               else
-                tc_cp_scales(sfa_t + 4 + 4 * r, sdesc_scales(src));
+                tc_cp_scales(sfb_t + 4 * r, sdesc_scales(src));
             }
           }
           // the stage is ready for its MMAs once these copies and its
