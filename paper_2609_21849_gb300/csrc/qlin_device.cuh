@@ -121,6 +121,33 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   }
 }
 
+// One lane of a converged warp (elect.sync): true in that lane.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(r));
+  return r != 0u;
+}
+
+// mbar_wait by every lane of a converged warp, which leaves together.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtl& ctl) {
+  const uint32_t a = smem_u32(bar);
+  if (__all_sync(0xFFFFFFFFu, mbar_try_wait(a, parity))) return true;
+  const uint64_t t0 = global_timer_ns();
+  for (uint32_t i = 1;; ++i) {
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait(a, parity))) return true;
+    if ((i & 63u) == 0u) {
+      bool stop = *ctl.abort != 0;
+      if (!stop && global_timer_ns() - t0 > ctl.timeout_ns) {
+        *ctl.abort = 1;
+        atomicExch(ctl.err, kErrTimeout);
+        stop = true;
+      }
+      if (__any_sync(0xFFFFFFFFu, stop)) return false;
+    }
+  }
+}
+
 // ------------------------------------------------------------------ TMA ---
 
 // 2-D tiled load global -> shared, completion counted on `bar` in bytes.
@@ -513,6 +540,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr)
       : "memory");
+}
+
+// Store four consecutive TMEM columns of this thread's lane.
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint4 v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr),
+               "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+
+__device__ __forceinline__ void tmem_st_wait() {
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void tmem_ld_wait() {

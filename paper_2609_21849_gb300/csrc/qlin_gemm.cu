@@ -50,12 +50,6 @@ constexpr int kEpiWarps = 8;
 // Build-time layout choices (the defaults measured fastest): scale-copy warps
 // of NVFP4 pair tiles, a warp of its own for their scale boxes, and row boxes
 // per operand tile and stage.
-#ifndef QLIN_PAIR_CP_WARPS
-#define QLIN_PAIR_CP_WARPS 4
-#endif
-#ifndef QLIN_SPLIT_SCALE_ISSUE
-#define QLIN_SPLIT_SCALE_ISSUE 1
-#endif
 #ifndef QLIN_TMA_SPLIT
 #define QLIN_TMA_SPLIT 2
 #endif
@@ -70,7 +64,10 @@ constexpr int kEpiWarps = 8;
 #ifndef QLIN_GROUP_M
 #define QLIN_GROUP_M 0
 #endif
-constexpr int kSmemBudget = 232448 - 2048;  // opt-in shared memory minus barriers/alignment
+#ifndef QLIN_SF_SLOTS
+#define QLIN_SF_SLOTS 5
+#endif
+constexpr int kSmemBudget = 232448 - 1536;  // opt-in shared memory minus barriers/alignment
 constexpr int kSplit = QLIN_TMA_SPLIT;      // row boxes per operand tile and stage
 
 constexpr int pow2_at_least(int x) {
@@ -83,23 +80,20 @@ constexpr int pow2_at_least(int x) {
 // holds its own 128 rows of A and its own half of the W tile.
 template <bool kFp4, int kBN, bool kPair = false>
 struct Cfg {
-  // warps: 0 producer, 1 MMA, then the scale-copy warps, then the epilogue
-  // (an epilogue warp w reads TMEM lanes 32 (w % 4) and up, so any eight
-  // consecutive warps cover the accumulator).  NVFP4 pair tiles need 12
-  // scale copies per stage, shared between the scale-copy warps.
-  static constexpr int kCpWarps = (kFp4 && kPair) ? QLIN_PAIR_CP_WARPS : 2;
-  static_assert(kStepsPerStage % kCpWarps == 0, "each scale-copy warp takes whole MMA steps");
-  // NVFP4 pair tiles: a warp of its own issues the scale boxes, so the
-  // operand boxes' instruction has two lanes instead of four
-  static constexpr int kScaleWarp = (kFp4 && kPair && QLIN_SPLIT_SCALE_ISSUE) ? 2 + kCpWarps : -1;
-  static constexpr int kEpiWarp0 = 2 + kCpWarps + (kScaleWarp >= 0 ? 1 : 0);
+  // warps: 0 producer, 1 MMA, NVFP4: four scale warps, pairs: the scale
+  // producer, then the epilogue (an epilogue or scale warp w reaches TMEM
+  // lanes 32 (w % 4) and up, so any four or eight consecutive warps cover
+  // every lane).
+  static constexpr int kSfWarps = kFp4 ? 4 : 0;
+  static constexpr bool kSfCopy = kFp4 && kPair;   // scales by TMA and tcgen05.cp
+  static_assert(!kSfCopy || kStepsPerStage % kSfWarps == 0, "whole MMA steps per copy warp");
+  static constexpr int kSfProducer = kSfCopy ? 2 + kSfWarps : -1;
+  static constexpr int kEpiWarp0 = 2 + kSfWarps + (kSfCopy ? 1 : 0);
   static constexpr int kThreads = (kEpiWarp0 + kEpiWarps) * 32;
   static constexpr int kSfbAtoms = kFp4 ? (kBN + 127) / 128 : 0;
   static constexpr int kABytes = kBM * kRowBytes;
   static constexpr int kBBytes = (kPair ? kBN / 2 : kBN) * kRowBytes;
-  static constexpr int kSfaBytes = kFp4 ? kStepsPerStage * 512 : 0;
-  static constexpr int kSfbBytes = kFp4 ? kSfbAtoms * kStepsPerStage * 512 : 0;
-  static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;
+  static constexpr int kStageBytes = kABytes + kBBytes;
   // Pair tiles store y straight from registers (each thread its row's 64
   // bytes per 32 columns): for FP8 / 16-bit tiles the staging's shared memory
   // holds a seventh pipeline stage, and for NVFP4 tiles the operand loads
@@ -108,7 +102,10 @@ struct Cfg {
   // boxes (2 KB each) stage TMA stores.
   static constexpr bool kDirectStore = kPair && kBN == 256 && (!kFp4 || QLIN_FP4_DIRECT_STORE);
   static constexpr int kOutBytes = kDirectStore ? 0 : kEpiWarps * 2 * 2048;
-  static constexpr int kStagesRaw = (kSmemBudget - kOutBytes) / kStageBytes;
+  static constexpr int kSfSmemSlots = kSfCopy ? QLIN_SF_SLOTS : 0;
+  static constexpr int kSfSlotBytes = (1 + kSfbAtoms) * kStepsPerStage * 512;
+  static constexpr int kSfBytes = kSfSmemSlots * kSfSlotBytes;
+  static constexpr int kStagesRaw = (kSmemBudget - kOutBytes - kSfBytes) / kStageBytes;
   static constexpr int kStages = kStagesRaw > 8 ? 8 : kStagesRaw;
   static constexpr int kNumAcc = (kFp4 && kBN == 256) ? 1 : 2;
   // Scale columns of one stage: A's (4 per 64 elements of K), then W's (4 per
@@ -118,10 +115,17 @@ struct Cfg {
   static constexpr int kSfColsPerStep = kFp4 ? kSfaCols + kSfbCols : 0;
   static constexpr int kSfColBase = kNumAcc * kBN;
   static constexpr bool kK96 = kFp4 && kBN >= 128;
+  // Scale slots in TMEM: a ring of its own, at most as long as the operand
+  // ring (the scale warps' wait for a slot relies on that).
+  static constexpr int kSfColsPerSlot = kStepsPerStage * kSfColsPerStep;
+  static constexpr int kSfSlotsRaw = kFp4 ? (512 - kSfColBase) / kSfColsPerSlot : 1;
+  static constexpr int kSfSlots =
+      kSfCopy ? kSfSmemSlots : kSfSlotsRaw < kStages ? kSfSlotsRaw : kStages;
+  static_assert(!kFp4 || (kSfSlots <= kSfSlotsRaw && kSfSlots <= kStages), "scale slots");
   static constexpr int kTmemCols =
-      pow2_at_least(kSfColBase + kStages * kStepsPerStage * kSfColsPerStep);
+      pow2_at_least(kSfColBase + kSfSlots * kSfColsPerSlot);
   static constexpr int kBarrierBytes = 512;
-  static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kOutBytes + kBarrierBytes;
+  static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kOutBytes + kSfBytes + kBarrierBytes;
   static_assert(kStageBytes % 1024 == 0, "stages must keep 1024-byte alignment");
   static_assert(kTmemCols <= 512, "TMEM budget");
   static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -183,6 +187,14 @@ __device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity, uint6
   }
 }
 
+__device__ __forceinline__ uint4 ld_global_v4(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ void st_global_v4(void* p, uint32_t a, uint32_t b, uint32_t c,
                                              uint32_t d) {
   asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(a), "r"(b), "r"(c),
@@ -228,40 +240,46 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* out_stage = smem + C::kStages * C::kStageBytes;   // epilogue staging boxes
-  uint64_t* full = reinterpret_cast<uint64_t*>(out_stage + C::kOutBytes);
+  uint8_t* sf_ring = out_stage + C::kOutBytes;               // block scales (kSfCopy)
+  uint64_t* full = reinterpret_cast<uint64_t*>(sf_ring + C::kSfBytes);
   uint64_t* empty = full + C::kStages;
-  uint64_t* sf_full = empty + C::kStages;   // NVFP4: the stage's scale bytes landed
-  uint64_t* tmem_full = sf_full + C::kStages;
+  uint64_t* sf_full = empty + C::kStages;       // kSfCopy: a slot's scale bytes landed
+  uint64_t* tmem_full = sf_full + C::kSfSmemSlots;
   uint64_t* tmem_empty = tmem_full + 2;
   uint64_t* mma_done = tmem_empty + 2;
-  uint64_t* sf_done = mma_done + 1;   // one barrier per scale-copy warp
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sf_done + C::kCpWarps);
+  uint64_t* sf_done = mma_done + 1;             // kSfCopy: one per scale warp
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sf_done + C::kSfWarps);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5;
+  // The roles below run whole warps in step, with one elected lane issuing: a
+  // warp index (and rank) that the compiler knows to be the same in all lanes
+  // keeps the addresses, descriptors and coordinates of tcgen05 and TMA
+  // instructions in uniform registers, where those instructions take them.
+  const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31;
-  const int rank = kPair ? (int)cluster_ctarank() : 0;
+  const int rank = kPair ? __shfl_sync(0xFFFFFFFFu, (int)cluster_ctarank(), 0) : 0;
   const bool leader = rank == 0;   // a pair's MMA / scale-copy CTA
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
-      // NVFP4: the scale-copy warps' commits (one per warp) also arrive on
-      // full, so the MMA issuer waits on one barrier per stage
-      mbar_init(&full[s], kFp4 ? 1 + C::kCpWarps : 1);
+      // NVFP4: the scale warps also arrive on full, so the MMA issuer waits
+      // on one barrier per stage
+      mbar_init(&full[s], 1 + C::kSfWarps);
       mbar_init(&empty[s], 1);
+    }
+    for (int s = 0; s < C::kSfSmemSlots; ++s) {
       mbar_init(&sf_full[s], 1);
     }
+    for (int w = 0; w < C::kSfWarps; ++w) mbar_init(&sf_done[w], 1);
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tmem_full[a], 1);
       mbar_init(&tmem_empty[a], kCM * kEpiWarps);   // every epilogue warp of the cluster
     }
     mbar_init(mma_done, 1);
-    for (int w = 0; w < C::kCpWarps; ++w) mbar_init(&sf_done[w], 1);
     *abort_flag = 0;
     mbar_fence_init();
   }
-  if (warp == 0 && lane < (kFp4 ? 4 : 2))
-    prefetch_tmap(lane == 0 ? &tmap_a : lane == 1 ? &tmap_b : lane == 2 ? &tmap_sfa : &tmap_sfb);
+  if (warp == 0 && lane < 2) prefetch_tmap(lane == 0 ? &tmap_a : &tmap_b);
   if (warp == 1) {
     if (kPair)
       tmem_alloc_pair(tmem_slot, C::kTmemCols);
@@ -274,7 +292,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   else
     __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot, 0);
   const WaitCtl ctl{abort_flag, p.err, p.timeout_ns};
   // the prologue above overlaps the previous kernel; global data only below
   grid_dep_wait();
@@ -290,111 +308,80 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   const int num_kb = (int)((k_bytes + kRowBytes - 1) / kRowBytes);
   const int k_steps = (int)(k_bytes / 32);
 
-  if (warp == 0 || warp == C::kScaleWarp) {
+  if (warp == 0) {
     // ------------------------------------------------------ TMA producer ---
-    // One 4-D tensor copy per lane (0: A tile, 1: W tile, 2: A scale atoms,
-    // 3: W scale atoms), all four issued as ONE instruction: a TMA copy holds
-    // its issuing thread for hundreds of cycles, so issuing them one by one
-    // would starve the tensor cores.  Out-of-range boxes (rows past M or N, K
-    // atoms past the end) are zero-filled and still count their full bytes,
-    // so every stage expects the same byte counts.
-    // Each operand tile is split into kSplit row boxes, one lane each, so
-    // more copies run at once (lanes [0, kSplit): A parts, [kSplit, 2 kSplit):
-    // W parts, then A scales, W scales): an SM's tensor copies fill shared
-    // memory at ~15 B/cycle per issuing lane, up to ~72 B/cycle with six or
-    // more lanes at once (measured), and a copy's rows split in two keep the
-    // stage's bytes in more streams (4608 x 12288 x 3072 NVFP4: 64.5 -> 63.0
-    // us; four boxes measured slower).
-    // With a scale-issue warp, warp 0 takes the operand lanes and that warp
-    // the two scale lanes; pl numbers the producer lanes across both.
-    constexpr int kOpLanes = 2 * kSplit;
-    const int pl = warp == 0 ? lane : kOpLanes + lane;
-    const int nlanes = warp != 0 ? 2 : (kFp4 && C::kScaleWarp < 0) ? kOpLanes + 2 : kOpLanes;
-    if (lane < nlanes) {
-      const bool is_scale = pl >= kOpLanes;
-      const int part = pl % kSplit;
-      const CUtensorMap* map = pl < kSplit      ? &tmap_a
-                               : pl < kOpLanes  ? &tmap_b
-                               : pl == kOpLanes ? &tmap_sfa
-                                                : &tmap_sfb;
-      uint64_t* bars = is_scale ? sf_full : full;
-      // barrier each copy completes on: this CTA's, or in a pair CTA 0's
-      const uint32_t bar0 = kPair ? mapa_shared(bars, 0) : smem_u32(bars);
-      int stage = 0;
-      uint32_t phase = 0;
-      int issued = 0;
-      for (int ct = cid; ct < num_ctiles; ct += ncl) {
-        int mg, nb;
-        tile_coords(ct, groups_m, tiles_n, &mg, &nb);
-        const int mb = mg * kCM + rank;
-        bool ok = true;
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, ctl)) {
-            ok = false;
-            break;
-          }
-          uint8_t* sA = smem + stage * C::kStageBytes;
-          uint8_t* sB = sA + C::kABytes;
-          uint8_t* sSF = sB + C::kBBytes;   // the stage's scale atoms: A's, then W's
-          if (leader && pl == 0)
-            mbar_arrive_expect_tx(&full[stage], kCM * (C::kABytes + C::kBBytes));
-          if (kFp4 && leader && pl == kOpLanes)
-            mbar_arrive_expect_tx(&sf_full[stage], kCM * (C::kSfaBytes + C::kSfbBytes));
-          __syncwarp((1u << nlanes) - 1u);
-          uint8_t* dst;
-          int32_t c0, c1, c2, c3;
-          constexpr int kARows = kBM / kSplit, kBRowsPart = kBN / kCM / kSplit;
-          if (pl < kSplit) {                // A: part of this CTA's M tile
-            dst = sA + part * kARows * kRowBytes;
-            c0 = kb * kRowBytes; c1 = mb * kBM + part * kARows; c2 = 0; c3 = 0;
-          } else if (pl < kOpLanes) {       // W: part of this CTA's rows of the N tile
-            dst = sB + part * kBRowsPart * kRowBytes;
-            c0 = kb * kRowBytes; c1 = nb * kBN + rank * (kBN / kCM) + part * kBRowsPart;
-            c2 = 0; c3 = 0;
-          } else if (pl == kOpLanes) {      // A scale atoms of this stage
-            dst = sSF; c0 = kb * kStepsPerStage * 64; c1 = mb; c2 = 0; c3 = 0;
-          } else {                          // W scale atoms (all atom rows of the N tile)
-            dst = sSF + C::kSfaBytes; c0 = kb * kStepsPerStage * 64;
-            c1 = (nb * kBN) >> 7; c2 = 0; c3 = 0;   // first 128-row atom of the N tile
-          }
-          const uint32_t bar = bar0 + (uint32_t)(stage * 8);
-          if (kPair)
-            tma_load_4d_pair(dst, map, bar, c0, c1, c2, c3);
-          else
-            tma_load_4d(dst, map, bar, c0, c1, c2, c3);
-          ++issued;
-          if (++stage == C::kStages) {
-            stage = 0;
-            phase ^= 1u;
+    // One elected lane issues a stage's A and W boxes (kSplit row boxes each).
+    // Out-of-range boxes (rows past M or N, K bytes past the end) are
+    // zero-filled and still count their full bytes, so every stage expects the
+    // same byte counts.
+    constexpr int kARows = kBM / kSplit, kWRows = kBN / kCM / kSplit;
+    // barrier the copies complete on: this CTA's, or in a pair the leader's
+    const uint32_t bar0 = kPair ? __shfl_sync(0xFFFFFFFFu, mapa_shared(full, 0), 0) : smem_u32(full);
+    int stage = 0;
+    uint32_t phase = 0;
+    int issued = 0;
+    bool ok = true;
+    for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
+      int mg, nb;
+      tile_coords(ct, groups_m, tiles_n, &mg, &nb);
+      const int a_row = (mg * kCM + rank) * kBM;
+      const int w_row = nb * kBN + rank * (kBN / kCM);
+      for (int kb = 0; kb < num_kb; ++kb) {
+        if (!mbar_wait_warp(&empty[stage], phase ^ 1u, ctl)) {
+          ok = false;
+          break;
+        }
+        uint8_t* const sA = smem + stage * C::kStageBytes;
+        const uint32_t bar = bar0 + (uint32_t)(stage * 8);
+        if (elect_one()) {
+          if (leader) mbar_arrive_expect_tx(&full[stage], kCM * (C::kABytes + C::kBBytes));
+#pragma unroll
+          for (int b = 0; b < kSplit; ++b) {
+            if (kPair) {
+              tma_load_4d_pair(sA + b * kARows * kRowBytes, &tmap_a, bar, kb * kRowBytes,
+                               a_row + b * kARows, 0, 0);
+              tma_load_4d_pair(sA + C::kABytes + b * kWRows * kRowBytes, &tmap_b, bar,
+                               kb * kRowBytes, w_row + b * kWRows, 0, 0);
+            } else {
+              tma_load_4d(sA + b * kARows * kRowBytes, &tmap_a, bar, kb * kRowBytes,
+                          a_row + b * kARows, 0, 0);
+              tma_load_4d(sA + C::kABytes + b * kWRows * kRowBytes, &tmap_b, bar, kb * kRowBytes,
+                          w_row + b * kWRows, 0, 0);
+            }
           }
         }
-        if (!ok) break;
+        ++issued;
+        if (++stage == C::kStages) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
-      // Let the last copies into this CTA land before it exits (the barriers
-      // that count them live in CTA 0; its producer drains them).
-      if (leader && (pl == 0 || (kFp4 && pl == kOpLanes))) {
-        const int n_drain = min(issued, C::kStages);
-        for (int i = 0; i < n_drain; ++i) {
-          if (--stage < 0) {
-            stage = C::kStages - 1;
-            phase ^= 1u;
-          }
-          mbar_drain(&bars[stage], phase, p.timeout_ns, p.err);
+    }
+    // Let the last copies into this CTA land before it exits (the barriers
+    // that count them live in CTA 0; its producer drains them).
+    if (leader && lane == 0) {
+      const int n_drain = min(issued, C::kStages);
+      for (int i = 0; i < n_drain; ++i) {
+        if (--stage < 0) {
+          stage = C::kStages - 1;
+          phase ^= 1u;
         }
+        mbar_drain(&full[stage], phase, p.timeout_ns, p.err);
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer ---
-    if (lane == 0 && leader) {
+    if (leader) {
       constexpr int kMmaM = kPair ? 256 : 128;
       const uint32_t idesc = kFp4    ? idesc_nvfp4(kBN, kMmaM)
                              : kBf16 ? (p.fp16 ? idesc_fp16(kBN, kMmaM) : idesc_bf16(kBN, kMmaM))
                                      : idesc_fp8(kBN, kMmaM);
       // A stage is ready for its MMAs once its operands have landed and, for
       // NVFP4, its scales are in TMEM (one barrier counts both).
-      auto wait_ready = [&](int st, uint32_t ph) { return mbar_wait(&full[st], ph, ctl); };
+      auto wait_ready = [&](int st, uint32_t ph) { return mbar_wait_warp(&full[st], ph, ctl); };
       int stage = 0;
       uint32_t phase = 0;
+      int slot = 0;   // scale slot of the stage
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
@@ -405,7 +392,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
         int mg_, nb_;
         tile_coords(ct, groups_m, tiles_n, &mg_, &nb_);
         const uint32_t sfb_off = kBN < 128 ? 2u * (uint32_t)(nb_ & 1) : 0u;
-        if (!mbar_wait(&tmem_empty[acc], acc_phase ^ 1u, ctl)) break;
+        if (!mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1u, ctl)) break;
         if (!wait_ready(stage, phase)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kBN);
@@ -417,9 +404,10 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           // address field (address / 16, 14 bits; shared addresses stay
           // below 256 KB, so it never carries) advances by 2 j
           const uint64_t adesc0 = sdesc_k128(sA), bdesc0 = sdesc_k128(sB);
-          const uint32_t sfa0 = tmem_base + (uint32_t)(C::kSfColBase + stage * kStepsPerStage *
-                                                                           C::kSfColsPerStep);
+          const uint32_t sfa0 =
+              tmem_base + (uint32_t)(C::kSfColBase + slot * C::kSfColsPerSlot);
           const uint32_t sfb0 = sfa0 + (uint32_t)(kStepsPerStage * C::kSfaCols) + sfb_off;
+          const uint32_t acc0 = kb > 0 ? 1u : 0u;
           auto issue = [&](int j, uint32_t accumulate) {
             const uint64_t adesc = adesc0 + (uint64_t)(2 * j);
             const uint64_t bdesc = bdesc0 + (uint64_t)(2 * j);
@@ -457,39 +445,41 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
                 mma_nvfp4_k96(d_tmem, adesc, bdesc, id, sfa_t, sfb_t, accumulate);
             }
           };
-          // Full stages issue their MMAs unrolled, with no branch between
-          // them: a runtime step loop around the MMA issue costs ~100 cycles
-          // a stage (measured), a fifth of the stage's tensor work.  Only a
+          // The stage is free once its MMAs have read it (both CTAs' halves).
+          auto release = [&] {
+            if (kPair)
+              tc_commit_pair_mc(&empty[stage], kMask);
+            else
+              tc_commit(&empty[stage]);
+          };
+          // Full stages issue their MMAs with no branch between them; only a
           // partial last stage (K % 256 != 0) takes the loop.
-          if (C::kK96 && nsteps >= 3) {
-            // K = 256 as 96 + 96 + 64, K = 192 as 96 + 96: an MMA of K = 96
-            // takes the time of one of K = 64
-            issue96(0, kb > 0 ? 1u : 0u);
-            issue96(1, 1u);
-            if (nsteps == kStepsPerStage) issue(3, 1u);
-          } else if (nsteps == kStepsPerStage) {
-            issue(0, kb > 0 ? 1u : 0u);
+          if (nsteps == kStepsPerStage) {
+            if (elect_one()) {
+              if (C::kK96) {
+                // 256 elements as 96 + 96 + 64: an MMA of K = 96 takes the
+                // time of one of K = 64
+                issue96(0, acc0);
+                issue96(1, 1u);
+                issue(3, 1u);
+              } else {
+                issue(0, acc0);
 #pragma unroll
-            for (int jj = 1; jj < kStepsPerStage; ++jj) issue(jj, 1u);
-          } else {
-            for (int jj = 0; jj < nsteps; ++jj) issue(jj, (jj > 0 || kb > 0) ? 1u : 0u);
+                for (int jj = 1; jj < kStepsPerStage; ++jj) issue(jj, 1u);
+              }
+              release();
+            }
+          } else if (elect_one()) {
+            for (int jj = 0; jj < nsteps; ++jj) issue(jj, jj > 0 ? 1u : acc0);
+            release();
           }
-          // The stage is free once the MMAs have read it (both CTAs' halves).
-          // The release comes right after the stage's last MMA: deferring it
-          // under the next stage's first MMA (to shorten the gap between
-          // issues) measured slower, the load pipeline being the bound.
-          if (kPair)
-            tc_commit_pair_mc(&empty[stage], kMask);
-          else
-            tc_commit(&empty[stage]);
           if (++stage == C::kStages) {
             stage = 0;
             phase ^= 1u;
           }
+          if (++slot == C::kSfSlots) slot = 0;
           // the tile's next stage: one barrier test per stage (the scale
-          // copies arrive on the same barrier as the operands; a second
-          // barrier's test cost ~100 cycles a stage in shared memory this
-          // busy, the MMA queue holding about one instruction)
+          // warps arrive on the same barrier as the operands)
           if (kb + 1 < num_kb) {
             if (!wait_ready(stage, phase)) {
               ok = false;
@@ -499,10 +489,12 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           }
         }
         if (!ok) break;
-        if (kPair)
-          tc_commit_pair_mc(&tmem_full[acc], kMask);   // both CTAs' epilogues
-        else
-          tc_commit(&tmem_full[acc]);
+        if (elect_one()) {
+          if (kPair)
+            tc_commit_pair_mc(&tmem_full[acc], kMask);   // both CTAs' epilogues
+          else
+            tc_commit(&tmem_full[acc]);
+        }
         if (C::kNumAcc == 2) {
           acc ^= 1;
           if (acc == 0) acc_phase ^= 1u;
@@ -511,81 +503,215 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
         }
       }
       // Every MMA / scale copy issued must finish before TMEM is released.
-      if (kPair)
-        tc_commit_pair_mc(mma_done, 1);
-      else
-        tc_commit(mma_done);
-      mbar_drain(mma_done, 0, p.timeout_ns, p.err);
+      if (elect_one()) {
+        if (kPair)
+          tc_commit_pair_mc(mma_done, 1);
+        else
+          tc_commit(mma_done);
+        mbar_drain(mma_done, 0, p.timeout_ns, p.err);
+      }
     }
-  } else if (warp < C::kEpiWarp0) {
-    // --------------------------------------------- NVFP4 scale copies ---
+  } else if (C::kSfCopy && warp == C::kSfProducer) {
+    // ------------------------------------------- scale producer (pairs) ---
+    // The A scale atoms of this CTA's M tile (2 KB a stage) and the W scale
+    // atoms of the whole N tile (4 KB); both complete on the leader.  The scale slots (shared memory and TMEM) are a ring of their
+    // own: a slot is free once the MMAs of the stage that last used it have
+    // completed.  (kSfSlots <= kStages: that stage's next MMAs wait for these
+    // scales, so its barrier cannot be a phase further on.)
+    const uint32_t bar0 = __shfl_sync(0xFFFFFFFFu, mapa_shared(sf_full, 0), 0);
+    int slot = 0, issued = 0, estage = 0;
+    uint32_t phase = 0, ephase = 0;
+    bool ok = true;
+    for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
+      int mg, nb;
+      tile_coords(ct, groups_m, tiles_n, &mg, &nb);
+      const int a_row = mg * kCM + rank, w_row = (nb * kBN) >> 7;
+      for (int kb = 0; kb < num_kb; ++kb) {
+        if (issued >= C::kSfSlots) {
+          if (!mbar_wait_warp(&empty[estage], ephase, ctl)) {
+            ok = false;
+            break;
+          }
+          if (++estage == C::kStages) {
+            estage = 0;
+            ephase ^= 1u;
+          }
+        }
+        uint8_t* const dst = sf_ring + slot * C::kSfSlotBytes;
+        const uint32_t bar = bar0 + (uint32_t)(slot * 8);
+        if (elect_one()) {
+          if (leader) mbar_arrive_expect_tx(&sf_full[slot], kCM * C::kSfSlotBytes);
+          tma_load_4d_pair(dst, &tmap_sfa, bar, kb * kStepsPerStage * 64, a_row, 0, 0);
+          tma_load_4d_pair(dst + kStepsPerStage * 512, &tmap_sfb, bar, kb * kStepsPerStage * 64,
+                           w_row, 0, 0);
+        }
+        ++issued;
+        if (++slot == C::kSfSlots) {
+          slot = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+    if (leader && lane == 0) {   // the last copies land before the pair exits
+      const int n_drain = min(issued, C::kSfSlots);
+      for (int i = 0; i < n_drain; ++i) {
+        if (--slot < 0) {
+          slot = C::kSfSlots - 1;
+          phase ^= 1u;
+        }
+        mbar_drain(&sf_full[slot], phase, p.timeout_ns, p.err);
+      }
+    }
+  } else if (C::kSfCopy && warp < C::kEpiWarp0) {
+    // ------------------------------------- NVFP4 scale copies (pairs) ---
     // Block scales move shared -> TMEM from threads of their own (one lane of
-    // each scale-copy warp), beside the MMA stream: a tcgen05.cp occupies its
-    // issuing thread ~80-120 cycles while the MMAs run, and a stage needs 12
-    // (pair tiles), so each warp copies the atoms of an equal share of the
-    // stage's MMA steps.  Copies issued from separate warps overlap (12 take
-    // ~850 cycles from two warps, ~510 from four, with the MMAs running: the
-    // MMAs' rate is unaffected), so pair tiles use four.  (A converged
-    // instruction from several lanes of one warp does not issue one copy per
-    // lane.)  In a pair, CTA 0's copies fill both SMs' TMEM from their own
-    // shared memory.
-    if (kFp4 && lane == 0 && leader) {
+    // each scale warp), beside the MMA stream: a tcgen05.cp occupies its
+    // issuing thread ~80-120 cycles while the MMAs run, and a stage needs 12,
+    // so each warp copies the atoms of an equal share of the stage's 64-element
+    // groups.  Copies issued from separate warps overlap (12 take ~850 cycles
+    // from two warps, ~510 from four, with the MMAs running: the MMAs' rate is
+    // unaffected).  (A converged instruction from several lanes of one warp
+    // does not issue one copy per lane.)  The leader's copies fill both SMs'
+    // TMEM from their own shared memory.
+    if (leader) {
       const int sw = warp - 2;
-      int stage = 0;
+      int stage = 0, slot = 0;
       uint32_t phase = 0;
-      for (int ct = cid; ct < num_ctiles; ct += ncl) {
-        bool ok = true;
+      bool ok = true;
+      for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(&sf_full[stage], phase, ctl)) {
+          if (!mbar_wait_warp(&sf_full[slot], phase, ctl)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sSFA = smem_u32(smem + stage * C::kStageBytes) + C::kABytes + C::kBBytes;
-          const uint32_t sSFB = sSFA + C::kSfaBytes;
+          const uint32_t sSFA = smem_u32(sf_ring + slot * C::kSfSlotBytes);
+          const uint32_t sSFB = sSFA + kStepsPerStage * 512;
+          const uint32_t sf0 = tmem_base + (uint32_t)(C::kSfColBase + slot * C::kSfColsPerSlot);
           const int nsteps = min(kStepsPerStage, k_steps - kb * kStepsPerStage);
-          // each warp copies all atoms (A, then each W atom row) of its share
-          // of the stage's MMA steps
-          constexpr int kShare = kStepsPerStage / C::kCpWarps;
+          constexpr int kShare = C::kSfCopy ? kStepsPerStage / C::kSfWarps : 1;
           const int j_end = min(nsteps, (sw + 1) * kShare);
-          for (int j = sw * kShare; j < j_end; ++j) {
-            const uint32_t sf0 = tmem_base + (uint32_t)(C::kSfColBase +
-                                                        stage * kStepsPerStage * C::kSfColsPerStep);
-            const uint32_t sfa_t = sf0 + (uint32_t)(j * C::kSfaCols);
-            const uint32_t sfb_t = sf0 + (uint32_t)(kStepsPerStage * C::kSfaCols + j * C::kSfbCols);
-            if (kPair)
-              tc_cp_scales_pair(sfa_t, sdesc_scales(sSFA + j * 512));
-            else
-              tc_cp_scales(sfa_t, sdesc_scales(sSFA + j * 512));
+          if (elect_one()) {
+            for (int j = sw * kShare; j < j_end; ++j) {
+              tc_cp_scales_pair(sf0 + (uint32_t)(j * C::kSfaCols), sdesc_scales(sSFA + j * 512));
 #pragma unroll
-            for (int r = 0; r < C::kSfbAtoms; ++r) {
-              const uint32_t src = sSFB + r * kStepsPerStage * 512 + j * 512;
-              if (kPair)
-                tc_cp_scales_pair(sfb_t + 4 * r, sdesc_scales(src));
-              else
-                tc_cp_scales(sfb_t + 4 * r, sdesc_scales(src));
+              for (int r = 0; r < C::kSfbAtoms; ++r)
+                tc_cp_scales_pair(
+                    sf0 + (uint32_t)(kStepsPerStage * C::kSfaCols + j * C::kSfbCols + 4 * r),
+                    sdesc_scales(sSFB + r * kStepsPerStage * 512 + j * 512));
             }
-          }
-          // the stage is ready for its MMAs once these copies and its
-          // operands have landed: both arrive on its full barrier.  (Its
-          // previous phase has completed: the scale boxes of this stage were
-          // issued after the MMAs of the stage that last used it.)
-          if (kPair)
+            // the stage is ready for its MMAs once these copies and its
+            // operands have landed: both arrive on its full barrier
             tc_commit_pair_mc(&full[stage], 1);
-          else
-            tc_commit(&full[stage]);
-          if (++stage == C::kStages) {
-            stage = 0;
+          }
+          if (++stage == C::kStages) stage = 0;
+          if (++slot == C::kSfSlots) {
+            slot = 0;
             phase ^= 1u;
           }
         }
-        if (!ok) break;
       }
-      if (kPair)
+      if (elect_one()) {
         tc_commit_pair_mc(&sf_done[sw], 1);
-      else
-        tc_commit(&sf_done[sw]);
-      mbar_drain(&sf_done[sw], 0, p.timeout_ns, p.err);
+        mbar_drain(&sf_done[sw], 0, p.timeout_ns, p.err);
+      }
+    }
+  } else if (warp < C::kEpiWarp0) {
+    // ------------------------------ NVFP4 scale warps (single-CTA tiles) ---
+    // Block scales go from global memory through registers into TMEM
+    // (tcgen05.st): lane l of the warp of each lane quarter takes the 16 bytes
+    // of row l of every atom, which are its lane's four columns of the atom.
+    // (In a pair each CTA would have to fill its own TMEM and arrive on the
+    // leader's barrier: measured far slower than the copies above.)  The four
+    // warps read the same bytes, so three of four reads hit L1; the lines are prefetched there
+    // kAhead stages before (the ring of slots is too short to hide L2).
+    if constexpr (kFp4 && !kPair) {
+      constexpr int kAhead = 4;
+      constexpr int kAtoms = 1 + C::kSfbAtoms;      // 128-row atom rows: A's, then W's
+      const int q = warp & 3;
+      const int64_t k64 = p.K >> 6;                 // atoms of a 128-row block
+      const int arows = (int)((p.M + 127) >> 7), wrows = (int)((p.N + 127) >> 7);
+      // the operand bytes of atom row r (0: A; 1..: W) of a tile, or null
+      auto atom_row = [&](int ct, int r) -> const uint8_t* {
+        int mg, nb;
+        tile_coords(ct, groups_m, tiles_n, &mg, &nb);
+        const int i = r == 0 ? mg * kCM + rank : ((nb * kBN) >> 7) + r - 1;
+        if (i >= (r == 0 ? arows : wrows)) return nullptr;
+        return (r == 0 ? p.sfa : p.sfb) + (int64_t)i * k64 * 512;
+      };
+      // prefetch position: kAhead stages ahead of the loads
+      int pct = cid, pkb = 0;
+      const uint8_t* prow = nullptr;                // this lane's atom row
+      // lane -> 128-byte line of a stage: atom row lane / 4, 16 lines each,
+      // four of them by each warp
+      const int pr = lane >> 2;
+      auto prefetch_next = [&] {
+        if (pct >= num_ctiles) return;
+        if (pkb == 0) prow = pr < kAtoms ? atom_row(pct, pr) : nullptr;
+        const int64_t off = (int64_t)pkb * 2048 + q * 512 + (lane & 3) * 128;
+        if (prow != nullptr && off < k64 * 512)
+          asm volatile("prefetch.global.L1 [%0];" ::"l"(prow + off));
+        if (++pkb == num_kb) {
+          pkb = 0;
+          pct += ncl;
+        }
+      };
+      for (int i = 0; i < kAhead; ++i) prefetch_next();
+      int stage = 0, slot = 0;
+      int estage = 0;                               // the slot's last use: its stage and phase
+      uint32_t ephase = 0;
+      int filled = 0;
+      bool ok = true;
+      for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
+        const uint8_t* rows[kAtoms];
+#pragma unroll
+        for (int r = 0; r < kAtoms; ++r) rows[r] = atom_row(ct, r);
+        for (int kb = 0; kb < num_kb; ++kb) {
+          prefetch_next();
+          const int ngroups = min(kStepsPerStage, k_steps - kb * kStepsPerStage);
+          uint4 v[kAtoms][kStepsPerStage];
+#pragma unroll
+          for (int r = 0; r < kAtoms; ++r)
+#pragma unroll
+            for (int j = 0; j < kStepsPerStage; ++j)
+              v[r][j] = rows[r] != nullptr && j < ngroups
+                            ? ld_global_v4(rows[r] + (int64_t)(kb * kStepsPerStage + j) * 512 +
+                                           lane * 16)
+                            : make_uint4(0u, 0u, 0u, 0u);
+          // the slot is free once the MMAs of the stage that last used it
+          // have completed (kSfSlots <= kStages, so that stage's barrier
+          // cannot be a phase further on)
+          if (filled == C::kSfSlots) {
+            if (!mbar_wait_warp(&empty[estage], ephase, ctl)) {
+              ok = false;
+              break;
+            }
+            if (++estage == C::kStages) {
+              estage = 0;
+              ephase ^= 1u;
+            }
+          } else {
+            ++filled;
+          }
+          tc_fence_after();
+          const uint32_t t = tmem_base + ((uint32_t)(q * 32) << 16) +
+                             (uint32_t)(C::kSfColBase + slot * C::kSfColsPerSlot);
+#pragma unroll
+          for (int j = 0; j < kStepsPerStage; ++j) {
+            tmem_st4(t + 4 * j, v[0][j]);
+#pragma unroll
+            for (int r = 1; r < kAtoms; ++r)
+              tmem_st4(t + (uint32_t)(kStepsPerStage * C::kSfaCols + j * C::kSfbCols + 4 * (r - 1)),
+                       v[r][j]);
+          }
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&full[stage]);
+          if (++stage == C::kStages) stage = 0;
+          if (++slot == C::kSfSlots) slot = 0;
+        }
+      }
     }
   } else {
     // --------------------------------------------------------- epilogue ---
@@ -646,7 +772,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           __syncwarp();
           if (lane == 0) {
             if (kPair && rank == 1)
-              mbar_arrive_cluster(mapa_shared(&tmem_empty[acc], 0));   // CTA 0 owns the MMA
+              mbar_arrive_cluster(mapa_shared(&tmem_empty[acc], 0));   // the leader owns the MMA
             else
               mbar_arrive(&tmem_empty[acc]);
           }
@@ -975,9 +1101,9 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned*
   if (encode_codes(&ta, a.a_codes, k_bytes, (uint64_t)a.M, kBM / kSplit,
                    (uint64_t)a.a_row_bytes) != CUDA_SUCCESS ||
       encode_codes(&tb, a.w_codes, k_bytes, (uint64_t)a.N, kBN / kCM / kSplit) != CUDA_SUCCESS ||
-      (kFp4 && (encode_scales(&tsa, a.sfa, (uint64_t)a.M, (uint64_t)a.K, 1) != CUDA_SUCCESS ||
-                encode_scales(&tsb, a.sfb, (uint64_t)a.N, (uint64_t)a.K, C::kSfbAtoms) !=
-                    CUDA_SUCCESS)) ||
+      (C::kSfCopy && (encode_scales(&tsa, a.sfa, (uint64_t)a.M, (uint64_t)a.K, 1) != CUDA_SUCCESS ||
+                     encode_scales(&tsb, a.sfb, (uint64_t)a.N, (uint64_t)a.K, C::kSfbAtoms) !=
+                         CUDA_SUCCESS)) ||
       (a.y != nullptr &&
        encode_tensor_map_out_bf16(&ty, a.y, (uint64_t)a.N, (uint64_t)a.M, kBf16 && a.fp16) !=
            CUDA_SUCCESS))
