@@ -182,6 +182,13 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The same without ordering any memory operation: the arrival does not wait
+// for this thread's outstanding stores.
+__device__ __forceinline__ void cluster_sync_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
 // 4-D tiled load; the completion barrier is given by its shared-memory address
 // (shared::cta, or shared::cluster for a barrier of another CTA).
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint32_t bar,
@@ -202,6 +209,15 @@ __device__ __forceinline__ void tma_load_4d_pair(void* dst, const CUtensorMap* m
       ".cta_group::2 [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
+}
+
+// Prefetch of a tiled box into L2 (a hint: no data comes back and nothing
+// waits for it).
+__device__ __forceinline__ void l2_prefetch_4d(const CUtensorMap* map, int32_t c0, int32_t c1) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %3}];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(c0), "r"(c1), "r"(0)
+               : "memory");
 }
 
 // Untiled bulk copy global -> shared (both 16-byte aligned, bytes % 16 == 0).
@@ -647,15 +663,6 @@ __device__ __forceinline__ void mul2_rn(float& a, float& b, float s) {
       "mov.b64 {%0, %1}, r;\n\t}"
       : "=f"(a), "=f"(b)
       : "f"(a), "f"(b), "f"(s));
-}
-
-// Block scale code s_b = E4M3((amax_b * S_enc) / 6) and the element
-// multiplier r_b = s_b == 0 ? 0 : S_enc / s_b (fp32, each op rounded once).
-__device__ __forceinline__ uint32_t nvfp4_block_scale(float amax_b, float s_enc, float* r_b) {
-  const float t = __fmul_rn(amax_b, s_enc);
-  const uint32_t sb = e4m3_code_div6(t);
-  *r_b = (sb == 0u) ? 0.0f : __fdiv_rn(s_enc, e4m3_value(sb));
-  return sb;
 }
 
 // Byte offset of block scale (row r, scale column c) in the 128x4-atom layout

@@ -12,27 +12,26 @@
 //          drives both SMs' tensor cores; each CTA holds its own 128 rows of A
 //          and its own half of the W tile in shared memory.
 //   single 128 x 128 tiles on one CTA, for small M (the translator's linears).
-// Roles (one persistent CTA per SM; 12 warps, 15 for NVFP4 pair tiles):
-//   warp 0      TMA producer: per pipeline stage one 4-D tensor copy per lane,
-//               the A tile and the W tile as two row boxes each from four
-//               lanes, as one instruction (and, except for NVFP4 pair tiles,
-//               the A and W scale atoms from two more lanes).  In a pair,
-//               CTA 1's copies complete on CTA 0's barriers (cta_group::2
-//               form).
+// Roles (one persistent CTA per SM; 10 warps, NVFP4 14, NVFP4 pairs 15).  Each
+// role runs its warp in step and one elected lane issues:
+//   warp 0      TMA producer: per pipeline stage the A tile and the W tile, as
+//               a few row boxes each.  In a pair, CTA 1's copies complete on
+//               CTA 0's barriers (cta_group::2 form).
 //   warp 1      TMEM allocation; MMA issue (per 32 bytes of K one tcgen05.mma:
-//               NVFP4 kind::mxf4nvf4 scale_vec::4X with K = 64, FP8
-//               kind::f8f6f4 with K = 32, bf16 / fp16 kind::f16 with K = 16)
-//               into an fp32 TMEM accumulator.
-//   warps 2..   NVFP4: block scales shared -> TMEM (tcgen05.cp), beside the
-//               MMA stream (two warps, four for pair tiles), each warp the
-//               atoms of an equal share of the stage's MMA steps.
-//   next warp   NVFP4 pair tiles: TMA producer of the scale atoms.
+//               FP8 kind::f8f6f4 with K = 32, bf16 / fp16 kind::f16 with
+//               K = 16; NVFP4 kind::mxf4nvf4 with K = 96, 96 and 64 per 256
+//               elements) into an fp32 TMEM accumulator.
+//   warps 2-5   NVFP4: block scales into TMEM.  Pair tiles: from shared memory
+//               (tcgen05.cp), beside the MMA stream, each warp the atoms of a
+//               quarter of the stage; single-CTA tiles: from global memory
+//               through registers (tcgen05.st), each warp its lane quarter.
+//   warp 6      NVFP4 pair tiles: TMA producer of the scale atoms.
 //   last 8      epilogue: tcgen05.ld of the accumulator, alpha, 16-bit
-//               rounding; pair tiles store y straight from registers (FP8 /
-//               16-bit tiles use the freed staging memory for a seventh
-//               stage), single-CTA tiles by TMA through swizzled staging;
-//               optional re-quantization of the 16-bit values, one row per
-//               thread, and optional output amax.
+//               rounding; pair tiles store y straight from registers (the
+//               staging's shared memory holds pipeline stages instead),
+//               single-CTA tiles by TMA through swizzled staging; optional
+//               re-quantization of the 16-bit values, one row per thread, and
+//               optional output amax.
 // Every wait is bounded (see WaitCtl).
 #include <cstring>
 #include <mutex>
@@ -46,29 +45,16 @@ namespace {
 constexpr int kBM = 128;
 constexpr int kRowBytes = 128;      // bytes of K per stage and row: one swizzle row
 constexpr int kStepsPerStage = 4;   // one MMA per 32 bytes of K
-constexpr int kEpiWarps = 8;
 // Build-time layout choices (the defaults measured fastest): scale-copy warps
 // of NVFP4 pair tiles, a warp of its own for their scale boxes, and row boxes
 // per operand tile and stage.
-#ifndef QLIN_TMA_SPLIT
-#define QLIN_TMA_SPLIT 2
-#endif
-// NVFP4 pair tiles store y straight from registers (no staging boxes and no
-// TMA stores sharing the copy engine with the operand loads)
-#ifndef QLIN_FP4_DIRECT_STORE
-#define QLIN_FP4_DIRECT_STORE 1
-#endif
 // Tile order: cluster tiles are visited in groups of this many M tile groups
 // (0: all of M, i.e. M fastest within each N tile; on the 4608 x 12288 x 3072
 // NVFP4 GEMM groups of 1 to 9 measured 3-6% slower)
 #ifndef QLIN_GROUP_M
 #define QLIN_GROUP_M 0
 #endif
-#ifndef QLIN_SF_SLOTS
-#define QLIN_SF_SLOTS 5
-#endif
 constexpr int kSmemBudget = 232448 - 1536;  // opt-in shared memory minus barriers/alignment
-constexpr int kSplit = QLIN_TMA_SPLIT;      // row boxes per operand tile and stage
 
 constexpr int pow2_at_least(int x) {
   int p = 32;
@@ -89,20 +75,27 @@ struct Cfg {
   static_assert(!kSfCopy || kStepsPerStage % kSfWarps == 0, "whole MMA steps per copy warp");
   static constexpr int kSfProducer = kSfCopy ? 2 + kSfWarps : -1;
   static constexpr int kEpiWarp0 = 2 + kSfWarps + (kSfCopy ? 1 : 0);
+  static constexpr int kEpiWarps = 8;
   static constexpr int kThreads = (kEpiWarp0 + kEpiWarps) * 32;
+  // Row boxes per operand tile and stage: copies of separate boxes overlap
+  // (pairs, 4608 x 12288 x 3072 NVFP4: one box 58.1, two 56.0, four 54.8 us).
+  static constexpr int kSplit = kPair ? 4 : 2;
   static constexpr int kSfbAtoms = kFp4 ? (kBN + 127) / 128 : 0;
   static constexpr int kABytes = kBM * kRowBytes;
   static constexpr int kBBytes = (kPair ? kBN / 2 : kBN) * kRowBytes;
   static constexpr int kStageBytes = kABytes + kBBytes;
   // Pair tiles store y straight from registers (each thread its row's 64
-  // bytes per 32 columns): for FP8 / 16-bit tiles the staging's shared memory
-  // holds a seventh pipeline stage, and for NVFP4 tiles the operand loads
-  // keep the copy engine to themselves (measured 70.1 -> 66.7 us on the
-  // 4608 x 12288 x 3072 GEMM).  Otherwise per epilogue warp two 32 x 32 bf16
-  // boxes (2 KB each) stage TMA stores.
-  static constexpr bool kDirectStore = kPair && kBN == 256 && (!kFp4 || QLIN_FP4_DIRECT_STORE);
+  // bytes per 32 columns): the staging's shared memory holds a pipeline stage
+  // more, and the operand loads keep the copy engine to themselves.  (The
+  // stores cost 6 of 53.5 us on the 4608 x 12288 x 3072 NVFP4 GEMM; whole
+  // 256-byte row segments per instruction measured slower, 58.0 us.)
+  // Otherwise per epilogue warp two 32 x 32 bf16 boxes (2 KB each) stage TMA
+  // stores.
+  static constexpr bool kDirectStore = kPair && kBN == 256;
   static constexpr int kOutBytes = kDirectStore ? 0 : kEpiWarps * 2 * 2048;
-  static constexpr int kSfSmemSlots = kSfCopy ? QLIN_SF_SLOTS : 0;
+  // Pairs: five scale slots beside six operand stages (four slots: 58.3 us
+  // instead of 54.8; TMEM has no room for a sixth beside the accumulator).
+  static constexpr int kSfSmemSlots = kSfCopy ? 5 : 0;
   static constexpr int kSfSlotBytes = (1 + kSfbAtoms) * kStepsPerStage * 512;
   static constexpr int kSfBytes = kSfSmemSlots * kSfSlotBytes;
   static constexpr int kStagesRaw = (kSmemBudget - kOutBytes - kSfBytes) / kStageBytes;
@@ -202,9 +195,10 @@ __device__ __forceinline__ void st_global_v4(void* p, uint32_t a, uint32_t b, ui
                : "memory");
 }
 
-// 32-byte store (p 32-byte aligned): a whole L2 sector from one lane.
+// 32-byte store (p 32-byte aligned): a whole L2 sector from one lane, kept out
+// of L1 (4608 x 12288 x 3072 NVFP4: plain 54.0 -> 53.5 us, fused 60.7 -> 59.6).
 __device__ __forceinline__ void st_global_v8(void* p, const uint32_t* v) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
+  asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
                "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                : "memory");
 }
@@ -273,7 +267,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     for (int w = 0; w < C::kSfWarps; ++w) mbar_init(&sf_done[w], 1);
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tmem_full[a], 1);
-      mbar_init(&tmem_empty[a], kCM * kEpiWarps);   // every epilogue warp of the cluster
+      mbar_init(&tmem_empty[a], kCM * C::kEpiWarps);   // every epilogue warp of the cluster
     }
     mbar_init(mma_done, 1);
     *abort_flag = 0;
@@ -294,10 +288,6 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot, 0);
   const WaitCtl ctl{abort_flag, p.err, p.timeout_ns};
-  // the prologue above overlaps the previous kernel; global data only below
-  grid_dep_wait();
-  grid_dep_launch();
-
   const int tiles_m = (int)((p.M + kBM - 1) / kBM);
   const int tiles_n = (int)((p.N + kBN - 1) / kBN);
   const int groups_m = (tiles_m + kCM - 1) / kCM;
@@ -308,13 +298,30 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   const int num_kb = (int)((k_bytes + kRowBytes - 1) / kRowBytes);
   const int k_steps = (int)(k_bytes / 32);
 
+  // The first W boxes into L2 while the previous kernel still runs: a prefetch
+  // is a hint that returns no data, so it is correct even if that kernel
+  // writes W.  (4608 x 3072 x 3072 NVFP4 in a chain of launches: 19.2 -> 18.7 us.)
+  if (warp == 0 && elect_one()) {
+    int mg, nb;
+    tile_coords(cid, groups_m, tiles_n, &mg, &nb);
+    constexpr int kWRows = kBN / kCM / C::kSplit;
+    const int w_row = nb * kBN + rank * (kBN / kCM);
+    for (int kb = 0; kb < min(num_kb, C::kStages); ++kb)
+#pragma unroll
+      for (int b = 0; b < C::kSplit; ++b)
+        l2_prefetch_4d(&tmap_b, kb * kRowBytes, w_row + b * kWRows);
+  }
+  // the prologue above overlaps the previous kernel; global data only below
+  grid_dep_wait();
+  grid_dep_launch();
+
   if (warp == 0) {
     // ------------------------------------------------------ TMA producer ---
     // One elected lane issues a stage's A and W boxes (kSplit row boxes each).
     // Out-of-range boxes (rows past M or N, K bytes past the end) are
     // zero-filled and still count their full bytes, so every stage expects the
     // same byte counts.
-    constexpr int kARows = kBM / kSplit, kWRows = kBN / kCM / kSplit;
+    constexpr int kSplit = C::kSplit, kARows = kBM / kSplit, kWRows = kBN / kCM / kSplit;
     // barrier the copies complete on: this CTA's, or in a pair the leader's
     const uint32_t bar0 = kPair ? __shfl_sync(0xFFFFFFFFu, mapa_shared(full, 0), 0) : smem_u32(full);
     int stage = 0;
@@ -454,19 +461,32 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           };
           // Full stages issue their MMAs with no branch between them; only a
           // partial last stage (K % 256 != 0) takes the loop.
-          if (nsteps == kStepsPerStage) {
+          bool next_ready = false;
+          if (C::kK96 && nsteps == kStepsPerStage) {
+            // 256 elements as 96 + 96 + 64: an MMA of K = 96 takes the time of
+            // one of K = 64.  The next stage's barrier is tested (without
+            // waiting) while the first two run, so that a stage that is ready
+            // costs no test after the release (4608 x 12288 x 3072: 53.8 ->
+            // 53.5 us; with the four MMAs of an FP8 stage it gains nothing).
             if (elect_one()) {
-              if (C::kK96) {
-                // 256 elements as 96 + 96 + 64: an MMA of K = 96 takes the
-                // time of one of K = 64
-                issue96(0, acc0);
-                issue96(1, 1u);
-                issue(3, 1u);
-              } else {
-                issue(0, acc0);
+              issue96(0, acc0);
+              issue96(1, 1u);
+            }
+            if (kb + 1 < num_kb) {
+              const bool wrap = stage + 1 == C::kStages;
+              next_ready = __all_sync(0xFFFFFFFFu,
+                                      mbar_test_wait(smem_u32(&full[wrap ? 0 : stage + 1]),
+                                                     wrap ? phase ^ 1u : phase));
+            }
+            if (elect_one()) {
+              issue(3, 1u);
+              release();
+            }
+          } else if (nsteps == kStepsPerStage) {
+            if (elect_one()) {
+              issue(0, acc0);
 #pragma unroll
-                for (int jj = 1; jj < kStepsPerStage; ++jj) issue(jj, 1u);
-              }
+              for (int jj = 1; jj < kStepsPerStage; ++jj) issue(jj, 1u);
               release();
             }
           } else if (elect_one()) {
@@ -481,7 +501,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           // the tile's next stage: one barrier test per stage (the scale
           // warps arrive on the same barrier as the operands)
           if (kb + 1 < num_kb) {
-            if (!wait_ready(stage, phase)) {
+            if (!next_ready && !wait_ready(stage, phase)) {
               ok = false;
               break;
             }
@@ -502,7 +522,14 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           acc_phase ^= 1u;
         }
       }
-      // Every MMA / scale copy issued must finish before TMEM is released.
+      // The epilogues' last arrivals have landed here (the cluster barrier at
+      // the end orders nothing).
+      if (ok) {
+        (void)mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1u, ctl);
+        if (C::kNumAcc == 2)
+          (void)mbar_wait_warp(&tmem_empty[acc ^ 1], acc == 0 ? acc_phase ^ 1u : acc_phase, ctl);
+      }
+      // Every MMA issued must finish before TMEM is released.
       if (elect_one()) {
         if (kPair)
           tc_commit_pair_mc(mma_done, 1);
@@ -715,7 +742,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     }
   } else {
     // --------------------------------------------------------- epilogue ---
-    constexpr int kCols = kBN / 2;  // columns per thread
+    constexpr int kCols = kBN / (C::kEpiWarps / 4);  // columns per thread
     constexpr int kChunks = kCols / 32;
     const int e = warp - C::kEpiWarp0;
     const int quarter = warp & 3;   // the TMEM lane quarter this warp may access
@@ -723,11 +750,21 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     const float sdec_a = kBf16 ? 1.0f : *p.sdec_a;
     const float alpha = kFp4 ? __fmul_rn(sdec_a, *p.sdec_w) : kBf16 ? 1.0f : 0.0f;
     float s_enc_next = 0.0f;
+    __shared__ float r_table[kFp4 && kRequant ? 256 : 1];
     if (kRequant) {
       const float s_next = *p.next_scale;
       s_enc_next = encode_scale(s_next);
       if (blockIdx.x == 0 && threadIdx.x == C::kEpiWarp0 * 32 && p.rq_tensor_scale != p.next_scale)
         *p.rq_tensor_scale = s_next;
+      if constexpr (kFp4) {
+        // r_b = S_enc / s_b of every E4M3 code, by the division that
+        // defines it (one table look-up instead of a division per block:
+        // 59.8 -> 59.3 us at 4608 x 12288 x 3072)
+        const uint32_t c = threadIdx.x - C::kEpiWarp0 * 32;
+        static_assert(C::kEpiWarps * 32 == 256, "one entry per epilogue thread");
+        r_table[c] = c == 0u ? 0.0f : __fdiv_rn(s_enc_next, e4m3_value(c));
+        asm volatile("bar.sync 1, %0;" ::"n"(C::kEpiWarps * 32) : "memory");
+      }
     }
     int acc = 0;
     uint32_t acc_phase = 0;
@@ -755,11 +792,9 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kBN + half * kCols);
       // Accumulator columns in batches of tcgen05.ld per wait; TMEM goes back
       // to the MMA issuer right after the last batch has landed in registers.
-      // With a single accumulator the next tile's MMAs wait for that, so all
-      // columns form one batch where the register budget (168 a thread at
-      // 12 warps, 128 above) allows.
-      constexpr int kBatch =
-          (C::kNumAcc == 1 && C::kThreads <= 384) ? kChunks : (kChunks < 2 ? kChunks : 2);
+      // (Sixteen epilogue warps of 64 columns each, so one batch, measured
+      // 1-2% slower: 56.1 against 54.8 us on 4608 x 12288 x 3072 NVFP4.)
+      constexpr int kBatch = kChunks < 2 ? kChunks : 2;
       static_assert(kChunks % kBatch == 0, "TMEM is released after the last batch");
 #pragma unroll
       for (int cb = 0; cb < kChunks; cb += kBatch) {
@@ -939,8 +974,8 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
 #pragma unroll
               for (int i = 0; i < 8; ++i) m = __vmaxu2(m, pk[i] & 0x7FFF7FFFu);
               m = max(m & 0xFFFFu, m >> 16);
-              float r_b;
-              const uint32_t sb = nvfp4_block_scale(__uint_as_float(m << 16), s_enc_next, &r_b);
+              const uint32_t sb = e4m3_code_div6(__fmul_rn(__uint_as_float(m << 16), s_enc_next));
+              const float r_b = r_table[sb];
               sw |= sb << (8 * b);
 #pragma unroll
               for (int h8 = 0; h8 < 2; ++h8) {
@@ -979,7 +1014,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
       // output), writes it where the quantizer of y reads its scale, and
       // resets both scratch words for the next call (so no clearing node
       // precedes the kernel).
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+      asm volatile("bar.sync 1, %0;" ::"n"(C::kEpiWarps * 32) : "memory");
       if (threadIdx.x == C::kEpiWarp0 * 32) {
         __threadfence();
         if (atomicAdd(p.y_departures, 1u) == gridDim.x - 1) {
@@ -999,7 +1034,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   __syncwarp();
   tc_fence_before();
   if (kPair)
-    cluster_sync();
+    cluster_sync_relaxed();
   else
     __syncthreads();
   if (warp == 1) {
@@ -1098,9 +1133,9 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned*
   std::memset(&tsa, 0, sizeof tsa);
   std::memset(&tsb, 0, sizeof tsb);
   std::memset(&ty, 0, sizeof ty);
-  if (encode_codes(&ta, a.a_codes, k_bytes, (uint64_t)a.M, kBM / kSplit,
+  if (encode_codes(&ta, a.a_codes, k_bytes, (uint64_t)a.M, kBM / C::kSplit,
                    (uint64_t)a.a_row_bytes) != CUDA_SUCCESS ||
-      encode_codes(&tb, a.w_codes, k_bytes, (uint64_t)a.N, kBN / kCM / kSplit) != CUDA_SUCCESS ||
+      encode_codes(&tb, a.w_codes, k_bytes, (uint64_t)a.N, kBN / kCM / C::kSplit) != CUDA_SUCCESS ||
       (C::kSfCopy && (encode_scales(&tsa, a.sfa, (uint64_t)a.M, (uint64_t)a.K, 1) != CUDA_SUCCESS ||
                      encode_scales(&tsb, a.sfb, (uint64_t)a.N, (uint64_t)a.K, C::kSfbAtoms) !=
                          CUDA_SUCCESS)) ||
