@@ -53,6 +53,15 @@ __device__ __forceinline__ uint4 lds128(const uint4* p) {
   return v;
 }
 
+// A load that stays after the grid dependency wait (volatile, as that is).
+__device__ __forceinline__ uint4 ldg128(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
 // The per-tile work of each kernel (called by every thread for each tile).
 struct AmaxOp {
   static constexpr int kUnit = 1;   // chunks per thread and call
@@ -92,12 +101,16 @@ struct Nvfp4Op {
   }
   // The codes of one 16-element block (block amax bits mb) and its scale
   // code (in `word`).
+  // kDivide: r_b by its division instead of the table (one block per thread).
+  template <bool kDivide = false>
   __device__ __forceinline__ void quantize_block(const uint4 (&v)[2], uint32_t mb,
                                                  uint32_t& code0, uint32_t& code1,
                                                  uint32_t& word) const {
     const float t = __fmul_rn(__uint_as_float(mb << 16), s_enc);
     const uint32_t sb = e4m3_code_div6(t);
-    const float r_b = r_table[sb];
+    const float r_b = !kDivide ? r_table[sb]
+                      : sb == 0u ? 0.0f
+                                 : __fdiv_rn(s_enc, e4m3_value(sb));
     float f[8];
     unpack8(v[0], f);
 #pragma unroll
@@ -109,9 +122,10 @@ struct Nvfp4Op {
     code1 = e2m1x8(f);
     word = sb;
   }
+  template <bool kDivide = false>
   __device__ __forceinline__ void unit(const uint4 (&v)[2], uint64_t c, bool valid) {
     uint32_t code0, code1, word;
-    quantize_block(v, max(chunk_abs_max_bits(v[0]), chunk_abs_max_bits(v[1])), code0, code1,
+    quantize_block<kDivide>(v, max(chunk_abs_max_bits(v[0]), chunk_abs_max_bits(v[1])), code0, code1,
                    word);
     if (valid) {
       reinterpret_cast<uint2*>(codes)[c >> 1] = make_uint2(code0, code1);
@@ -131,6 +145,10 @@ struct Nvfp4Op {
         }
       }
     }
+  }
+  // The two chunks of one thread, with no table.
+  __device__ __forceinline__ void block(const uint4 (&v)[2], uint32_t c, bool valid) {
+    unit<true>(v, c, valid);
   }
   // A slice of n chunks held in shared memory, global chunks [c0, c0 + n)
   // (c0 and n multiples of 8): each thread takes units of two chunks at a
@@ -203,6 +221,11 @@ struct Fp8Op {
 #pragma unroll
     for (int i = 0; i < 8; ++i) f[i] = __fmul_rn(f[i], s_enc);
     codes[c] = make_uint2(e4m3x4(f[0], f[1], f[2], f[3]), e4m3x4(f[4], f[5], f[6], f[7]));
+  }
+  __device__ __forceinline__ void block(const uint4 (&v)[2], uint32_t c, bool valid) {
+    const uint4 a[1] = {v[0]}, b[1] = {v[1]};
+    unit(a, c, valid);
+    unit(b, c + 1, valid);
   }
   template <int kThreadsPerBlock>
   __device__ __forceinline__ void run_slice(const uint4* buf, uint32_t n, uint64_t c0) const {
@@ -600,6 +623,76 @@ __global__ void __launch_bounds__(kOnePassThreads, 1)
     op.template run_slice<kOnePassThreads>(buf, n, c_begin);
 }
 
+// Small x: every cluster of eight CTAs reads all of x (an eighth per CTA, from
+// L2 after the first), combines the maxima through distributed shared memory
+// and quantizes its share, so the grid needs neither a grid-wide barrier nor a
+// cooperative launch.  One 16-element block (two chunks) per thread, loaded
+// first and kept in registers.  Bound by latency: launch, one load, one
+// cluster barrier.
+#ifndef QLIN_CLUSTER_MAX_KB
+#define QLIN_CLUSTER_MAX_KB 1024
+#endif
+constexpr int kClusterCtas = 8;
+constexpr int kClusterThreads = 512;
+constexpr uint32_t kClusterSub = 2 * kClusterThreads;   // chunks a CTA quantizes at most
+
+__device__ __forceinline__ void st_shared_cluster_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// range: chunks of a CTA's eighth of x; sub: chunks of it that each of the
+// grid's clusters quantizes (both multiples of 8, sub <= kClusterSub).
+template <typename Op>
+__global__ void __launch_bounds__(kClusterThreads)
+    cluster_quant_kernel(const uint4* __restrict__ x, uint32_t n_chunks, uint32_t range,
+                         uint32_t sub, Op op, float qmax, float* sdec_out) {
+  __shared__ uint32_t warp_max[kClusterThreads / 32];
+  __shared__ uint32_t cta_max[kClusterCtas];
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  grid_dep_wait();
+  const uint32_t tid = threadIdx.x;
+  const uint32_t rank = cluster_ctarank();
+  const uint32_t r0 = min(rank * range, n_chunks), r1 = min(r0 + range, n_chunks);
+  const uint32_t s0 = r0 + (blockIdx.x / kClusterCtas) * sub;
+  const uint32_t s1 = min(s0 + sub, r1);
+  const uint32_t c = s0 + 2u * tid;
+  const bool own = c < s1;
+  uint4 v[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) v[k] = own ? ldg128(x + c + k) : make_uint4(0u, 0u, 0u, 0u);
+  uint32_t m = 0;
+  uint32_t i = r0 + tid;
+  for (; i + 7u * kClusterThreads < r1; i += 8u * kClusterThreads) {   // eight loads in flight
+    uint4 t[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = ldg128(x + i + k * kClusterThreads);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m = max(m, chunk_abs_max_bits(t[k]));
+  }
+  for (; i < r1; i += kClusterThreads) m = max(m, chunk_abs_max_bits(ldg128(x + i)));
+  grid_dep_launch();
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  if ((tid & 31u) == 0u) warp_max[tid >> 5] = m;
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");   // the peers have started
+  __syncthreads();
+  if (tid < (uint32_t)kClusterCtas) {
+    uint32_t b = 0;
+#pragma unroll
+    for (int w = 0; w < kClusterThreads / 32; ++w) b = max(b, warp_max[w]);
+    st_shared_cluster_u32(mapa_shared(&cta_max[rank], tid), b);
+  }
+  __syncwarp();
+  cluster_sync();
+  uint32_t b = 0;
+#pragma unroll
+  for (int r = 0; r < kClusterCtas; ++r) b = max(b, cta_max[r]);
+  const float amax = __uint_as_float(b << 16);
+  const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
+  if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
+  op.s_enc = encode_scale(s_dec);
+  op.block(v, c, own);
+}
+
 // Opt each kernel into kSmem bytes of dynamic shared memory, once.
 template <auto kKern>
 cudaError_t set_smem() {
@@ -698,6 +791,42 @@ static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op
   return e;
 }
 
+// Multiplier and shifts that divide a 32-bit index by d (1 <= d < 2^31)
+// without a division instruction: the round-up form of Granlund and
+// Montgomery (PLDI 1994), exact for every 32-bit dividend.
+static uint3 invariant_divisor(uint32_t d) {
+  int l = 0;
+  while ((1ull << l) < d) ++l;   // ceil(log2 d)
+  const uint64_t m = ((1ull << 32) * ((1ull << l) - d)) / d + 1;
+  return make_uint3((uint32_t)m, (uint32_t)(l < 1 ? l : 1), (uint32_t)(l > 1 ? l - 1 : 0));
+}
+
+// The cluster route takes x of up to kClusterMaxChunks chunks.
+constexpr uint64_t kClusterMaxChunks = QLIN_CLUSTER_MAX_KB * 64ull;
+
+template <typename Op>
+static cudaError_t launch_cluster_quant(const void* x, uint32_t n_chunks, const Op& op,
+                                        float qmax, float* sdec_out, cudaStream_t s) {
+  const uint32_t range = ((n_chunks + kClusterCtas - 1) / kClusterCtas + 7) / 8 * 8;
+  const uint32_t clusters = (range + kClusterSub - 1) / kClusterSub;
+  const uint32_t sub = ((range + clusters - 1) / clusters + 7) / 8 * 8;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kClusterCtas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(clusters * kClusterCtas, 1, 1);
+  cfg.blockDim = dim3(kClusterThreads, 1, 1);
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, cluster_quant_kernel<Op>, static_cast<const uint4*>(x), n_chunks,
+                            range, sub, op, qmax, sdec_out);
+}
+
 cudaError_t launch_quant_nvfp4_onepass(const void* x, int64_t M, int64_t K,
                                        const qlin_nvfp4_t& out, unsigned* sync, bool clear,
                                        cudaStream_t s, int num_sms, unsigned* err,
@@ -707,11 +836,16 @@ cudaError_t launch_quant_nvfp4_onepass(const void* x, int64_t M, int64_t K,
   Nvfp4Op<uint32_t> op;
   op.s_enc = 0.0f;   // set in the kernel once amax is known
   op.chunks_per_row = (uint32_t)(K >> 3);
-  op.div_m = op.div_s1 = op.div_s2 = 0;   // run_slice tracks rows without dividing
+  const uint3 row_div = invariant_divisor((uint32_t)(K >> 3));   // run_slice does without
+  op.div_m = row_div.x;
+  op.div_s1 = row_div.y;
+  op.div_s2 = row_div.z;
   op.K = K;
   op.codes = reinterpret_cast<uint32_t*>(out.codes);
   op.scales = out.scales;
   op.r_table = nullptr;   // set in the kernel (shared memory)
+  if (n_chunks <= kClusterMaxChunks)
+    return launch_cluster_quant(x, (uint32_t)n_chunks, op, 2688.0f, out.tensor_scale, s);
   return launch_onepass(x, n_chunks, op, 2688.0f, out.tensor_scale, sync, clear, s, num_sms, err,
                         timeout_ns);
 }
@@ -723,18 +857,10 @@ cudaError_t launch_quant_fp8_onepass(const void* x, int64_t M, int64_t K, const 
   Fp8Op op;
   op.s_enc = 0.0f;
   op.codes = reinterpret_cast<uint2*>(out.codes);
+  if (n_chunks <= kClusterMaxChunks)
+    return launch_cluster_quant(x, (uint32_t)n_chunks, op, 448.0f, out.scale, s);
   return launch_onepass(x, n_chunks, op, 448.0f, out.scale, sync, clear, s, num_sms, err,
                         timeout_ns);
-}
-
-// Multiplier and shifts that divide a 32-bit index by d (1 <= d < 2^31)
-// without a division instruction: the round-up form of Granlund and
-// Montgomery (PLDI 1994), exact for every 32-bit dividend.
-static uint3 invariant_divisor(uint32_t d) {
-  int l = 0;
-  while ((1ull << l) < d) ++l;   // ceil(log2 d)
-  const uint64_t m = ((1ull << 32) * ((1ull << l) - d)) / d + 1;
-  return make_uint3((uint32_t)m, (uint32_t)(l < 1 ? l : 1), (uint32_t)(l > 1 ? l - 1 : 0));
 }
 
 template <bool kDynamic>
