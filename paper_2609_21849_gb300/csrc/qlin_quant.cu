@@ -19,6 +19,8 @@
 // 16-element block per lane, so four neighbouring lanes hold one 64-element
 // group, whose four block scales form one 32-bit word of the scale layout;
 // because K % 64 == 0 a group never straddles a row).
+#include <atomic>
+
 #include "qlin_internal.h"
 
 namespace qlin {
@@ -63,16 +65,6 @@ __device__ __forceinline__ uint4 ldg128(const uint4* p) {
 }
 
 // The per-tile work of each kernel (called by every thread for each tile).
-struct AmaxOp {
-  static constexpr int kUnit = 1;   // chunks per thread and call
-  uint32_t m = 0;
-  __device__ __forceinline__ void bind(float*) {}
-  __device__ __forceinline__ void init() {}
-  __device__ __forceinline__ void unit(const uint4 (&v)[1], uint64_t, bool valid) {
-    if (valid) m = max(m, chunk_abs_max_bits(v[0]));
-  }
-};
-
 // One lane per 16-element block (two chunks); each lane stores its block's
 // scale code as one byte of the atom layout (one store instruction per warp,
 // instead of gathering a 64-element group's four codes by shuffles: measured
@@ -143,6 +135,36 @@ struct Nvfp4Op {
           const Idx col = (ci - row * chunks_per_row) << 3;
           scales[scale_offset((int64_t)row, (int64_t)(col >> 4), K)] = (uint8_t)word;
         }
+      }
+    }
+  }
+  // The thread's units of two chunks, kStride chunks apart, held in registers
+  // (bm: their block amax bits); row and column are tracked without dividing.
+  template <int kUnits, uint32_t kStride>
+  __device__ __forceinline__ void run_units(const uint4 (&v)[kUnits][2],
+                                            const uint32_t (&bm)[kUnits / 2], uint32_t n,
+                                            uint64_t c0) const {
+    const uint32_t cpr = (uint32_t)chunks_per_row;
+    const uint32_t dq = kStride / cpr, dr = kStride % cpr;
+    const uint64_t cg = c0 + 2u * threadIdx.x;
+    uint32_t row = (uint32_t)(cg / cpr), col = (uint32_t)(cg % cpr);   // col in chunks
+    const uint32_t kgroups = (uint32_t)(K >> 6);
+#pragma unroll
+    for (int u = 0; u < kUnits; ++u) {
+      if ((uint32_t)u * kStride >= n) break;   // block-uniform
+      const uint32_t cl = (uint32_t)u * kStride + 2u * threadIdx.x;
+      uint32_t a0, a1, aw;
+      quantize_block(v[u], (u & 1) ? bm[u / 2] >> 16 : bm[u / 2] & 0xFFFFu, a0, a1, aw);
+      if (cl < n) {
+        reinterpret_cast<uint2*>(codes)[(c0 + cl) >> 1] = make_uint2(a0, a1);
+        scales[((row >> 7) * kgroups + (col >> 3)) * 512u + (row & 31u) * 16u +
+               ((row >> 5) & 3u) * 4u + ((col >> 1) & 3u)] = (uint8_t)aw;
+      }
+      row += dq;
+      col += dr;
+      if (col >= cpr) {
+        col -= cpr;
+        ++row;
       }
     }
   }
@@ -244,11 +266,8 @@ struct Fp8Op {
 // flight; every thread applies `op` to its chunks of each landed tile.
 // `setup(op)` runs once the first copies are on their way (reads that only
 // the arithmetic needs, such as the tensor scale, overlap the loads).
-// kReverse visits the tiles last-first: a second pass over data that a
-// first pass has just streamed forward starts on the lines still in L2
-// (NVFP4 dynamic route at 18432 x 3072, amax pass then quantizer: 49.5 ->
-// 48.2 us).  Returns false if a bounded wait expired (recorded in *err).
-template <bool kReverse = false, typename Op, typename Setup>
+// Returns false if a bounded wait expired (recorded in *err).
+template <typename Op, typename Setup>
 __device__ __forceinline__ bool stream_tiles(const uint4* __restrict__ x, uint64_t n_chunks,
                                              Op& op, Setup setup, unsigned* err,
                                              uint64_t timeout_ns) {
@@ -260,7 +279,7 @@ __device__ __forceinline__ bool stream_tiles(const uint4* __restrict__ x, uint64
   const int tid = threadIdx.x;
 
   auto issue = [&](uint64_t t, int s) {
-    const uint64_t c0 = (kReverse ? n_tiles - 1 - t : t) * kTileChunks;
+    const uint64_t c0 = t * kTileChunks;
     const uint64_t left = n_chunks - c0;
     const uint32_t nc = left < (uint64_t)kTileChunks ? (uint32_t)left : (uint32_t)kTileChunks;
     mbar_arrive_expect_tx(&full[s], nc * 16u);
@@ -294,7 +313,7 @@ __device__ __forceinline__ bool stream_tiles(const uint4* __restrict__ x, uint64
       t_stop = t;
       break;
     }
-    const uint64_t c0 = (kReverse ? n_tiles - 1 - t : t) * kTileChunks;
+    const uint64_t c0 = t * kTileChunks;
     constexpr int kU = Op::kUnit;
 #pragma unroll
     for (int u = 0; u < kTileChunks / (kU * kThreads); ++u) {
@@ -352,54 +371,20 @@ __device__ __forceinline__ void l2_prefetch_first_tile(const uint4* x, uint64_t 
   }
 }
 
-// amax over n_chunks 16-byte chunks, folded into *amax_bits (fp32 bits;
-// cleared before the launch).
-__global__ void __launch_bounds__(kThreads, kBlocksPerSm)
-    amax_kernel(const uint4* __restrict__ x, uint64_t n_chunks, unsigned* __restrict__ amax_bits,
-                unsigned* err, uint64_t timeout_ns) {
-  l2_prefetch_first_tile(x, n_chunks);
-  grid_dep_wait();
-  grid_dep_launch();
-  __shared__ uint32_t warp_max[kThreads / 32];
-  AmaxOp op;
-  stream_tiles(x, n_chunks, op, [](AmaxOp&) {}, err, timeout_ns);
-  const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, op.m);
-  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t b = 0;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) b = max(b, warp_max[w]);
-    if (b) atomicMax(amax_bits, b << 16);
-  }
-}
-
-// Tensor scale: kDynamic -> scale_src holds amax, S_dec = amax / qmax (1 if
-// amax == 0); otherwise scale_src holds S_dec.  Block 0 records S_dec.
-template <bool kDynamic>
-__device__ __forceinline__ float tensor_scale(const float* scale_src, float* sdec_out,
-                                              float qmax) {
-  float s_dec;
-  if (kDynamic) {
-    const float amax = *scale_src;
-    s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
-  } else {
-    s_dec = *scale_src;
-  }
+// Block 0 records the static tensor scale S_dec.
+__device__ __forceinline__ float static_scale(const float* scale_src, float* sdec_out) {
+  const float s_dec = *scale_src;
   if (blockIdx.x == 0 && threadIdx.x == 0 && sdec_out != scale_src) *sdec_out = s_dec;
   return s_dec;
 }
 
-template <bool kDynamic, typename Idx>
+template <typename Idx>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
     quant_nvfp4_kernel(const uint4* __restrict__ x, uint64_t n_chunks, int64_t K,
                        const float* scale_src, float* sdec_out, uint32_t* __restrict__ codes,
                        uint8_t* __restrict__ scales, uint3 row_div, unsigned* err,
                        uint64_t timeout_ns) {
-  // The dynamic-scale instance is the second pass over x (after amax_kernel,
-  // or over y after the GEMM that reduced its amax): it reads last-first, and
-  // its first tiles are then the ones most recently in L2.
-  if (!kDynamic) l2_prefetch_first_tile(x, n_chunks);
+  l2_prefetch_first_tile(x, n_chunks);
   grid_dep_wait();
   grid_dep_launch();
   __shared__ float r_table[128];
@@ -412,28 +397,22 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
   op.K = K;
   op.codes = codes;
   op.scales = scales;
-  stream_tiles<kDynamic>(
+  stream_tiles(
       x, n_chunks, op,
-      [&](Nvfp4Op<Idx>& o) {
-        o.s_enc = encode_scale(tensor_scale<kDynamic>(scale_src, sdec_out, 2688.0f));
-      },
-      err, timeout_ns);
+      [&](Nvfp4Op<Idx>& o) { o.s_enc = encode_scale(static_scale(scale_src, sdec_out)); }, err,
+      timeout_ns);
 }
 
-template <bool kDynamic>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
     quant_fp8_kernel(const uint4* __restrict__ x, uint64_t n_chunks, const float* scale_src,
-                     float* sdec_out, uint2* __restrict__ codes, unsigned* err,
-                     uint64_t timeout_ns) {
+                     float* sdec_out, Fp8Op op, unsigned* err, uint64_t timeout_ns) {
   l2_prefetch_first_tile(x, n_chunks);
   grid_dep_wait();
   grid_dep_launch();
-  Fp8Op op;
-  op.codes = codes;
   stream_tiles(
       x, n_chunks, op,
-      [&](Fp8Op& o) { o.s_enc = encode_scale(tensor_scale<kDynamic>(scale_src, sdec_out, 448.0f)); },
-      err, timeout_ns);
+      [&](Fp8Op& o) { o.s_enc = encode_scale(static_scale(scale_src, sdec_out)); }, err,
+      timeout_ns);
 }
 
 // FP8 weights, one scale per row: one warp per row, two passes over the row
@@ -505,6 +484,51 @@ __device__ __forceinline__ void cp_async_wait_pending(int pending) {
   }
 }
 
+// The maximum of the grid's warp maxima into *s_amax (shared memory, for every
+// thread): combine the CTA's, publish, arrive, wait (bounded) for every CTA,
+// depart.  False if the wait expired (recorded in *err).
+template <int kThreadsPerBlock>
+__device__ __forceinline__ bool grid_amax(const uint32_t* warp_max, unsigned* sync, float* s_amax,
+                                          int* abort_flag, unsigned* err, uint64_t timeout_ns) {
+  const int tid = threadIdx.x;
+  if (tid == 0) *abort_flag = 0;
+  __syncthreads();
+  if (tid == 0) {
+    uint32_t b = 0;
+#pragma unroll
+    for (int w = 0; w < kThreadsPerBlock / 32; ++w) b = max(b, warp_max[w]);
+    // publish, arrive, and wait (bounded) for every CTA of the grid
+    if (b) atomicMax(&sync[0], b << 16);
+    // the arrival releases the maximum above to every CTA that sees it
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&sync[1]) : "memory");
+    // The count and the amax are read together: a load that sees every
+    // CTA's arrival also sees every maximum released before it, which saves
+    // the second round trip to L2 that reading the amax afterwards took.
+    const uint64_t t0 = global_timer_ns();
+    uint64_t pair = ld_acquire_gpu_pair(&sync[0]);
+    while ((uint32_t)(pair >> 32) < gridDim.x) {
+      if (global_timer_ns() - t0 > timeout_ns) {
+        atomicExch(err, kErrTimeout);
+        *abort_flag = 1;
+        break;
+      }
+      pair = ld_acquire_gpu_pair(&sync[0]);
+    }
+    *s_amax = __uint_as_float((uint32_t)pair);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    // depart (after a timeout too); the last CTA out resets the words.  The
+    // other warps do not wait for this atomic's round trip.
+    if (atomicAdd(&sync[2], 1u) == gridDim.x - 1u) {
+      sync[0] = 0u;
+      sync[1] = 0u;
+      sync[2] = 0u;
+    }
+  }
+  return *abort_flag == 0;
+}
+
 // sync[0]: amax bits (fp32), sync[1]: arrival count, sync[2]: departure
 // count; all zero at launch, and the last CTA to depart zeroes them again, so
 // back-to-back launches (graph replays included) need no clearing between.
@@ -574,42 +598,8 @@ __global__ void __launch_bounds__(kOnePassThreads, 1)
   }
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31) == 0) warp_max[tid >> 5] = m;
-  if (tid == 0) abort_flag = 0;
-  __syncthreads();
-  if (tid == 0) {
-    uint32_t b = 0;
-#pragma unroll
-    for (int w = 0; w < kOnePassThreads / 32; ++w) b = max(b, warp_max[w]);
-    // publish, arrive, and wait (bounded) for every CTA of the grid
-    if (b) atomicMax(&sync[0], b << 16);
-    // the arrival releases the maximum above to every CTA that sees it
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&sync[1]) : "memory");
-    // The count and the amax are read together: a load that sees every
-    // CTA's arrival also sees every maximum released before it, which saves
-    // the second round trip to L2 that reading the amax afterwards took.
-    const uint64_t t0 = global_timer_ns();
-    uint64_t pair = ld_acquire_gpu_pair(&sync[0]);
-    while ((uint32_t)(pair >> 32) < gridDim.x) {
-      if (global_timer_ns() - t0 > timeout_ns) {
-        atomicExch(err, kErrTimeout);
-        abort_flag = 1;
-        break;
-      }
-      pair = ld_acquire_gpu_pair(&sync[0]);
-    }
-    s_amax = __uint_as_float((uint32_t)pair);
-  }
-  __syncthreads();
-  if (tid == 0) {
-    // depart (after a timeout too); the last CTA out resets the words.  The
-    // other warps do not wait for this atomic's round trip.
-    if (atomicAdd(&sync[2], 1u) == gridDim.x - 1u) {
-      sync[0] = 0u;
-      sync[1] = 0u;
-      sync[2] = 0u;
-    }
-  }
-  if (abort_flag) return;
+  const bool ok = grid_amax<kOnePassThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns);
+  if (!ok) return;
   const float amax = s_amax;
   const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
@@ -621,6 +611,196 @@ __global__ void __launch_bounds__(kOnePassThreads, 1)
     op.template run_slice<kOnePassThreads, kOnePassSteps>(buf, n, c_begin, bm);
   else
     op.template run_slice<kOnePassThreads>(buf, n, c_begin);
+}
+
+// NVFP4, x held in registers instead of shared memory (up to kRegUnits 32-byte
+// units, one block each, per thread): no trip through shared memory, whose
+// 32-byte-strided reads (each block twice, with two-way bank conflicts) made up
+// 6500 of the 21 000 cycles of the shared-memory kernel.  4608 x 3072: 12.2 ->
+// 11.45 us, 1000 x 3072: 5.45 -> 5.3 us.  (FP8 in this form: 11.1 -> 10.9 us,
+// but 3.9 -> 4.6 us at 2.5 MB, so it keeps the shared-memory kernel.)  Reading
+// x from HBM takes ~6 us of it, the grid barrier ~1.3 us.
+constexpr int kRegThreads = 512;
+constexpr int kRegUnits = 12;
+constexpr uint32_t kRegStride = 2u * kRegThreads;               // chunks between a thread's units
+constexpr uint32_t kRegSliceMax = kRegUnits * kRegStride;       // 192 KB of x per CTA
+
+template <typename Op>
+__global__ void __launch_bounds__(kRegThreads, 1)
+    regpass_kernel(const uint4* __restrict__ x, uint64_t n_chunks, uint32_t slice, Op op,
+                   float qmax, float* sdec_out, unsigned* sync, unsigned* err,
+                   uint64_t timeout_ns) {
+  __shared__ uint32_t warp_max[kRegThreads / 32];
+  __shared__ float op_table[128];
+  __shared__ float s_amax;
+  __shared__ int abort_flag;
+  grid_dep_wait();
+  const uint32_t tid = threadIdx.x;
+  const uint64_t c_begin = (uint64_t)blockIdx.x * slice;
+  const uint32_t n = c_begin >= n_chunks ? 0u
+                     : (uint32_t)(n_chunks - c_begin < slice ? n_chunks - c_begin : slice);
+  const uint4* xs = x + c_begin + 2u * tid;
+  uint4 v[kRegUnits][2];
+#pragma unroll
+  for (int u = 0; u < kRegUnits; ++u) {
+    const bool in = (uint32_t)u * kRegStride + 2u * tid < n;   // units never straddle n
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      v[u][k] = in ? ldg128(xs + u * kRegStride + k) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  uint32_t m = 0;
+  uint32_t bm[kRegUnits / 2];   // block maxima, two to a word
+#pragma unroll
+  for (int u = 0; u < kRegUnits; ++u) {
+    const uint32_t b = max(chunk_abs_max_bits(v[u][0]), chunk_abs_max_bits(v[u][1]));
+    if (u & 1)
+      bm[u / 2] |= b << 16;
+    else
+      bm[u / 2] = b;
+    m = max(m, b);
+  }
+  grid_dep_launch();   // x is on chip: the next kernel may begin launching
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  if ((tid & 31u) == 0u) warp_max[tid >> 5] = m;
+  if (!grid_amax<kRegThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns)) return;
+  const float amax = s_amax;
+  const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
+  if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
+  op.s_enc = encode_scale(s_dec);
+  op.bind(op_table);
+  op.init();
+  __syncthreads();
+  op.template run_units<kRegUnits, kRegStride>(v, bm, n, c_begin);
+}
+
+// Dynamic scale of an x that does not fit on chip: one cooperative launch (the
+// streaming kernels' grid, three CTAs per SM) reads x for its amax, meets at
+// the grid barrier and quantizes its tiles in reverse order.  The last
+// kStages tiles of every CTA (29 MB in all) are still in its ring, and the
+// ones before them are the lines most recently in L2.  Bound by HBM: x once and
+// what of it L2 has lost a second time.
+template <typename Op>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm)
+    two_phase_kernel(const uint4* __restrict__ x, uint64_t n_chunks, Op op, float qmax,
+                     float* sdec_out, unsigned* sync, unsigned* err, uint64_t timeout_ns) {
+  extern __shared__ __align__(128) uint8_t qsm[];
+  uint4* buf = reinterpret_cast<uint4*>(qsm);
+  uint64_t* full = reinterpret_cast<uint64_t*>(qsm + kStages * kTileChunks * 16);
+  __shared__ uint32_t warp_max[kThreads / 32];
+  __shared__ float op_table[128];
+  __shared__ float s_amax;
+  __shared__ int abort_flag;
+  l2_prefetch_first_tile(x, n_chunks);
+  grid_dep_wait();
+  grid_dep_launch();
+  const int tid = threadIdx.x;
+  const uint64_t n_tiles = (n_chunks + kTileChunks - 1) / kTileChunks;
+  // this CTA's tiles are blockIdx.x + i * gridDim.x, i in [0, n_own); tile i
+  // sits in stage i % kStages
+  const int64_t n_own = (int64_t)((n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x);
+  uint32_t landing = 0;   // thread 0: stages with a copy in flight
+  uint32_t phase = 0;     // thread 0: parity of each stage's next completion
+  auto tile_chunk0 = [&](int64_t i) {
+    return (blockIdx.x + (uint64_t)i * gridDim.x) * kTileChunks;
+  };
+  auto issue = [&](int64_t i) {   // thread 0
+    const int s = (int)(i % kStages);
+    const uint64_t c0 = tile_chunk0(i), left = n_chunks - c0;
+    const uint32_t nc = left < (uint64_t)kTileChunks ? (uint32_t)left : (uint32_t)kTileChunks;
+    mbar_arrive_expect_tx(&full[s], nc * 16u);
+    bulk_load(buf + s * kTileChunks, x + c0, nc * 16u, &full[s]);
+    landing |= 1u << s;
+  };
+  // Thread 0 waits for stage s's copy, if one is in flight; all leave together.
+  auto landed = [&](int s) {
+    if (tid == 0 && (landing >> s & 1u)) {
+      const WaitCtl ctl{&abort_flag, err, timeout_ns};
+      if (!mbar_wait(&full[s], phase >> s & 1u, ctl)) {
+        abort_flag = 1;
+      } else {
+        landing &= ~(1u << s);
+        phase ^= 1u << s;
+      }
+    }
+    __syncthreads();
+    return abort_flag == 0;
+  };
+  // After an expired wait: copies in flight land before the CTA exits.
+  auto drain = [&] {
+    if (tid != 0) return;
+    for (int s = 0; s < kStages; ++s) {
+      if (!(landing >> s & 1u)) continue;
+      const uint64_t t0 = global_timer_ns();
+      while (!mbar_try_wait(smem_u32(&full[s]), phase >> s & 1u) &&
+             global_timer_ns() - t0 < timeout_ns) {
+      }
+    }
+  };
+  if (tid == 0) {
+    for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1);
+    abort_flag = 0;
+    mbar_fence_init();
+    for (int64_t i = 0; i < kStages && i < n_own; ++i) issue(i);
+  }
+  uint32_t m = 0;
+  bool ok = true;
+  __syncthreads();
+  for (int64_t i = 0; i < n_own; ++i) {
+    const int s = (int)(i % kStages);
+    if (!landed(s)) {
+      ok = false;
+      break;
+    }
+    const uint64_t c0 = tile_chunk0(i);
+#pragma unroll
+    for (int u = 0; u < kTileChunks / kThreads; ++u)
+      if (c0 + u * kThreads + tid < n_chunks)
+        m = max(m, chunk_abs_max_bits(lds128(buf + s * kTileChunks + u * kThreads + tid)));
+    if (i + kStages < n_own) {   // the last kStages tiles stay
+      __syncthreads();
+      if (tid == 0) issue(i + kStages);
+    }
+  }
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  if ((tid & 31) == 0) warp_max[tid >> 5] = m;
+  __syncthreads();   // every thread has read abort_flag
+  // (a CTA whose wait expired still arrives, so that no other waits for it)
+  const bool met = grid_amax<kThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns);
+  if (!ok || !met) {
+    drain();
+    return;
+  }
+  const float amax = s_amax;
+  const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
+  if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
+  op.s_enc = encode_scale(s_dec);
+  op.bind(op_table);
+  op.init();
+  __syncthreads();
+  for (int64_t i = n_own - 1; i >= 0; --i) {
+    const int s = (int)(i % kStages);
+    if (!landed(s)) {
+      drain();
+      return;
+    }
+    const uint64_t c0 = tile_chunk0(i);
+    constexpr int kU = Op::kUnit;
+#pragma unroll
+    for (int u = 0; u < kTileChunks / (kU * kThreads); ++u) {
+      const int cl = (u * kThreads + tid) * kU;
+      const uint64_t c = c0 + cl;
+      const bool valid = c < n_chunks;
+      uint4 v[kU];
+#pragma unroll
+      for (int k = 0; k < kU; ++k)
+        v[k] = valid ? lds128(buf + s * kTileChunks + cl + k) : make_uint4(0u, 0u, 0u, 0u);
+      op.unit(v, c, valid);
+    }
+    if (i >= kStages) {
+      __syncthreads();   // every thread is done with this stage
+      if (tid == 0) issue(i - kStages);
+    }
+  }
 }
 
 // Small x: every cluster of eight CTAs reads all of x (an eighth per CTA, from
@@ -643,7 +823,7 @@ __device__ __forceinline__ void st_shared_cluster_u32(uint32_t addr, uint32_t v)
 // range: chunks of a CTA's eighth of x; sub: chunks of it that each of the
 // grid's clusters quantizes (both multiples of 8, sub <= kClusterSub).
 template <typename Op>
-__global__ void __launch_bounds__(kClusterThreads)
+__global__ void __launch_bounds__(kClusterThreads, 1)
     cluster_quant_kernel(const uint4* __restrict__ x, uint32_t n_chunks, uint32_t range,
                          uint32_t sub, Op op, float qmax, float* sdec_out) {
   __shared__ uint32_t warp_max[kClusterThreads / 32];
@@ -725,14 +905,33 @@ int stream_grid(uint64_t n_chunks, int num_sms) {
 
 }  // namespace
 
-cudaError_t launch_amax(const void* x, int64_t n_elems, unsigned* amax_bits, cudaStream_t s,
-                        int num_sms, unsigned* err, uint64_t timeout_ns) {
-  cudaError_t e = cudaMemsetAsync(amax_bits, 0, sizeof(unsigned), s);
-  if (e != cudaSuccess) return e;
-  if ((e = set_smem<amax_kernel>()) != cudaSuccess) return e;
-  const uint64_t n_chunks = (uint64_t)n_elems / 8;
-  return launch_pdl(amax_kernel, stream_grid(n_chunks, num_sms), kThreads, kSmem, s,
-                    static_cast<const uint4*>(x), n_chunks, amax_bits, err, timeout_ns);
+// Cooperative launch (all CTAs resident: the grid waits on itself), with
+// programmatic serialization where the driver accepts it alongside, else
+// without.
+template <typename... Params, typename... Args>
+static cudaError_t launch_cooperative(void (*kern)(Params...), int grid, int block, int smem,
+                                      cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3((unsigned)block, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  static std::atomic<bool> pdl_ok{true};
+  cfg.numAttrs = pdl_ok.load(std::memory_order_relaxed) ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+  if (e != cudaSuccess && cfg.numAttrs == 2) {
+    (void)cudaGetLastError();
+    pdl_ok.store(false, std::memory_order_relaxed);
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, args...);
+  }
+  return e;
 }
 
 // One-pass dynamic quantization when x fits on chip: returns
@@ -747,58 +946,53 @@ static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op
   slice = (slice + 7) / 8 * 8;
   if (slice > (uint64_t)kOnePassSliceMax || slice == 0) return cudaErrorNotSupported;
   const int grid = (int)((n_chunks + slice - 1) / slice);
+  // NVFP4: held in registers where the slice fits, else in shared memory
+  bool reg = false;
   auto kern = onepass_kernel<Op>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePassSmem);
-  if (attr != cudaSuccess) return attr;
-  static int resident = -1;   // CTAs of this kernel one SM can hold
-  if (resident < 0) {
-    int r = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kern, kOnePassThreads, kOnePassSmem) !=
-        cudaSuccess)
-      r = 0;
-    resident = r;
+  if constexpr (Op::kBlockMax) {
+    reg = slice <= (uint64_t)kRegSliceMax;
+    if (reg) kern = regpass_kernel<Op>;
   }
-  if (resident < 1 || grid > num_sms * resident) return cudaErrorNotSupported;
+  const int threads = reg ? kRegThreads : kOnePassThreads, smem = reg ? 0 : kOnePassSmem;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      onepass_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePassSmem);
+  if (attr != cudaSuccess) return attr;
+  static int resident[2] = {-1, -1};   // CTAs of each kernel one SM can hold
+  if (resident[reg] < 0) {
+    int r = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kern, threads, smem) != cudaSuccess) r = 0;
+    resident[reg] = r;
+  }
+  if (resident[reg] < 1 || grid > num_sms * resident[reg]) return cudaErrorNotSupported;
   if (clear) {
     const cudaError_t e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeCooperative;   // all CTAs resident: the grid waits on itself
-  at[0].val.cooperative = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(kOnePassThreads, 1, 1);
-  cfg.dynamicSmemBytes = kOnePassSmem;
-  cfg.stream = s;
-  cfg.attrs = at;
-  // with programmatic serialization where the driver accepts it alongside a
-  // cooperative launch, else without
-  static bool pdl_ok = true;
-  cfg.numAttrs = pdl_ok ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<const uint4*>(x), n_chunks,
-                                     (uint32_t)slice, op, qmax, sdec_out, sync, err, timeout_ns);
-  if (e != cudaSuccess && pdl_ok) {
-    (void)cudaGetLastError();
-    pdl_ok = false;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, static_cast<const uint4*>(x), n_chunks, (uint32_t)slice,
-                           op, qmax, sdec_out, sync, err, timeout_ns);
-  }
-  return e;
+  return launch_cooperative(kern, grid, threads, smem, s, static_cast<const uint4*>(x), n_chunks,
+                            (uint32_t)slice, op, qmax, sdec_out, sync, err, timeout_ns);
 }
 
-// Multiplier and shifts that divide a 32-bit index by d (1 <= d < 2^31)
-// without a division instruction: the round-up form of Granlund and
-// Montgomery (PLDI 1994), exact for every 32-bit dividend.
-static uint3 invariant_divisor(uint32_t d) {
-  int l = 0;
-  while ((1ull << l) < d) ++l;   // ceil(log2 d)
-  const uint64_t m = ((1ull << 32) * ((1ull << l) - d)) / d + 1;
-  return make_uint3((uint32_t)m, (uint32_t)(l < 1 ? l : 1), (uint32_t)(l > 1 ? l - 1 : 0));
+// x of any size: two phases over it in one cooperative launch.
+template <typename Op>
+static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& op, float qmax,
+                                    float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
+                                    int num_sms, unsigned* err, uint64_t timeout_ns) {
+  cudaError_t e = set_smem<two_phase_kernel<Op>>();
+  if (e != cudaSuccess) return e;
+  static int resident = -1;   // CTAs one SM can hold
+  if (resident < 0) {
+    int r = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, two_phase_kernel<Op>, kThreads,
+                                                           kSmem)) != cudaSuccess)
+      return e;
+    resident = r;
+  }
+  if (resident < 1) return cudaErrorLaunchOutOfResources;
+  if (clear && (e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s)) != cudaSuccess) return e;
+  const int grid = std::min(stream_grid(n_chunks, num_sms), num_sms * resident);
+  return launch_cooperative(two_phase_kernel<Op>, grid, kThreads, kSmem, s,
+                            static_cast<const uint4*>(x), n_chunks, op, qmax, sdec_out, sync, err,
+                            timeout_ns);
 }
 
 // The cluster route takes x of up to kClusterMaxChunks chunks.
@@ -827,89 +1021,103 @@ static cudaError_t launch_cluster_quant(const void* x, uint32_t n_chunks, const 
                             range, sub, op, qmax, sdec_out);
 }
 
-cudaError_t launch_quant_nvfp4_onepass(const void* x, int64_t M, int64_t K,
-                                       const qlin_nvfp4_t& out, unsigned* sync, bool clear,
-                                       cudaStream_t s, int num_sms, unsigned* err,
-                                       uint64_t timeout_ns) {
-  const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
-  if (n_chunks >= (1ull << 32)) return cudaErrorNotSupported;
-  Nvfp4Op<uint32_t> op;
-  op.s_enc = 0.0f;   // set in the kernel once amax is known
-  op.chunks_per_row = (uint32_t)(K >> 3);
-  const uint3 row_div = invariant_divisor((uint32_t)(K >> 3));   // run_slice does without
+// Multiplier and shifts that divide a 32-bit index by d (1 <= d < 2^31)
+// without a division instruction: the round-up form of Granlund and
+// Montgomery (PLDI 1994), exact for every 32-bit dividend.
+static uint3 invariant_divisor(uint32_t d) {
+  int l = 0;
+  while ((1ull << l) < d) ++l;   // ceil(log2 d)
+  const uint64_t m = ((1ull << 32) * ((1ull << l) - d)) / d + 1;
+  return make_uint3((uint32_t)m, (uint32_t)(l < 1 ? l : 1), (uint32_t)(l > 1 ? l - 1 : 0));
+}
+
+// The arithmetic and addressing of an NVFP4 quantizer of x [M, K] into `out`;
+// s_enc and the table are set in the kernel.
+template <typename Idx>
+static Nvfp4Op<Idx> nvfp4_op(int64_t K, const qlin_nvfp4_t& out) {
+  Nvfp4Op<Idx> op;
+  op.s_enc = 0.0f;
+  op.chunks_per_row = (Idx)(K >> 3);
+  const uint3 row_div = invariant_divisor((uint32_t)(K >> 3));
   op.div_m = row_div.x;
   op.div_s1 = row_div.y;
   op.div_s2 = row_div.z;
   op.K = K;
   op.codes = reinterpret_cast<uint32_t*>(out.codes);
   op.scales = out.scales;
-  op.r_table = nullptr;   // set in the kernel (shared memory)
-  if (n_chunks <= kClusterMaxChunks)
-    return launch_cluster_quant(x, (uint32_t)n_chunks, op, 2688.0f, out.tensor_scale, s);
-  return launch_onepass(x, n_chunks, op, 2688.0f, out.tensor_scale, sync, clear, s, num_sms, err,
-                        timeout_ns);
+  op.r_table = nullptr;
+  return op;
 }
 
-cudaError_t launch_quant_fp8_onepass(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
-                                     unsigned* sync, bool clear, cudaStream_t s, int num_sms,
-                                     unsigned* err, uint64_t timeout_ns) {
-  const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
+static Fp8Op fp8_op(const qlin_fp8_t& out) {
   Fp8Op op;
   op.s_enc = 0.0f;
   op.codes = reinterpret_cast<uint2*>(out.codes);
-  if (n_chunks <= kClusterMaxChunks)
-    return launch_cluster_quant(x, (uint32_t)n_chunks, op, 448.0f, out.scale, s);
-  return launch_onepass(x, n_chunks, op, 448.0f, out.scale, sync, clear, s, num_sms, err,
-                        timeout_ns);
+  return op;
 }
 
-template <bool kDynamic>
-static cudaError_t launch_nvfp4_t(const void* x, int64_t M, int64_t K, const float* scale_src,
-                                  const qlin_nvfp4_t& out, cudaStream_t s, int num_sms,
-                                  unsigned* err, uint64_t timeout_ns) {
+// By size: every cluster reads x (latency), x held on chip (one read), two
+// phases over x.
+template <typename Op>
+static cudaError_t launch_dynamic(const void* x, uint64_t n_chunks, const Op& op, float qmax,
+                                  float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
+                                  int num_sms, unsigned* err, uint64_t timeout_ns) {
+  if (n_chunks <= kClusterMaxChunks)
+    return launch_cluster_quant(x, (uint32_t)n_chunks, op, qmax, sdec_out, s);
+  const cudaError_t e = launch_onepass(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms,
+                                       err, timeout_ns);
+  if (e != cudaErrorNotSupported) return e;
+  return launch_two_phase(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms, err,
+                          timeout_ns);
+}
+
+cudaError_t launch_quant_nvfp4_dynamic(const void* x, int64_t M, int64_t K,
+                                       const qlin_nvfp4_t& out, unsigned* sync, bool clear,
+                                       cudaStream_t s, int num_sms, unsigned* err,
+                                       uint64_t timeout_ns) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
-  const uint3 row_div = invariant_divisor((uint32_t)(K >> 3));
-  const int grid = stream_grid(n_chunks, num_sms);
-  auto* xin = static_cast<const uint4*>(x);
-  auto* codes = reinterpret_cast<uint32_t*>(out.codes);
-  cudaError_t e;
-  if (n_chunks < (1ull << 32)) {   // 32-bit index math is enough
-    if ((e = set_smem<quant_nvfp4_kernel<kDynamic, uint32_t>>()) != cudaSuccess) return e;
-    e = launch_pdl(quant_nvfp4_kernel<kDynamic, uint32_t>, grid, kThreads, kSmem, s, xin,
-                   n_chunks, K, scale_src, out.tensor_scale, codes, out.scales, row_div, err,
-                   timeout_ns);
-  } else {
-    if ((e = set_smem<quant_nvfp4_kernel<kDynamic, uint64_t>>()) != cudaSuccess) return e;
-    e = launch_pdl(quant_nvfp4_kernel<kDynamic, uint64_t>, grid, kThreads, kSmem, s, xin,
-                   n_chunks, K, scale_src, out.tensor_scale, codes, out.scales, row_div, err,
-                   timeout_ns);
-  }
-  return e;
+  if (n_chunks < (1ull << 32))   // 32-bit index math is enough
+    return launch_dynamic(x, n_chunks, nvfp4_op<uint32_t>(K, out), 2688.0f, out.tensor_scale, sync,
+                          clear, s, num_sms, err, timeout_ns);
+  return launch_two_phase(x, n_chunks, nvfp4_op<uint64_t>(K, out), 2688.0f, out.tensor_scale, sync,
+                          clear, s, num_sms, err, timeout_ns);
+}
+
+cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
+                                     unsigned* sync, bool clear, cudaStream_t s, int num_sms,
+                                     unsigned* err, uint64_t timeout_ns) {
+  return launch_dynamic(x, (uint64_t)M * (uint64_t)K / 8, fp8_op(out), 448.0f, out.scale, sync,
+                        clear, s, num_sms, err, timeout_ns);
 }
 
 cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float* scale_src,
-                               bool dynamic, const qlin_nvfp4_t& out, cudaStream_t s,
-                               int num_sms, unsigned* err, uint64_t timeout_ns) {
-  return dynamic ? launch_nvfp4_t<true>(x, M, K, scale_src, out, s, num_sms, err, timeout_ns)
-                 : launch_nvfp4_t<false>(x, M, K, scale_src, out, s, num_sms, err, timeout_ns);
-}
-
-cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* scale_src,
-                             bool dynamic, const qlin_fp8_t& out, cudaStream_t s, int num_sms,
-                             unsigned* err, uint64_t timeout_ns) {
+                               const qlin_nvfp4_t& out, cudaStream_t s, int num_sms,
+                               unsigned* err, uint64_t timeout_ns) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
   const int grid = stream_grid(n_chunks, num_sms);
   auto* xin = static_cast<const uint4*>(x);
-  auto* codes = reinterpret_cast<uint2*>(out.codes);
+  auto* codes = reinterpret_cast<uint32_t*>(out.codes);
+  const uint3 row_div = invariant_divisor((uint32_t)(K >> 3));
   cudaError_t e;
-  if (dynamic) {
-    if ((e = set_smem<quant_fp8_kernel<true>>()) != cudaSuccess) return e;
-    return launch_pdl(quant_fp8_kernel<true>, grid, kThreads, kSmem, s, xin, n_chunks, scale_src,
-                      out.scale, codes, err, timeout_ns);
+  if (n_chunks < (1ull << 32)) {   // 32-bit index math is enough
+    if ((e = set_smem<quant_nvfp4_kernel<uint32_t>>()) != cudaSuccess) return e;
+    return launch_pdl(quant_nvfp4_kernel<uint32_t>, grid, kThreads, kSmem, s, xin, n_chunks, K,
+                      scale_src, out.tensor_scale, codes, out.scales, row_div, err, timeout_ns);
   }
-  if ((e = set_smem<quant_fp8_kernel<false>>()) != cudaSuccess) return e;
-  return launch_pdl(quant_fp8_kernel<false>, grid, kThreads, kSmem, s, xin, n_chunks, scale_src,
-                    out.scale, codes, err, timeout_ns);
+  if ((e = set_smem<quant_nvfp4_kernel<uint64_t>>()) != cudaSuccess) return e;
+  return launch_pdl(quant_nvfp4_kernel<uint64_t>, grid, kThreads, kSmem, s, xin, n_chunks, K,
+                    scale_src, out.tensor_scale, codes, out.scales, row_div, err, timeout_ns);
+}
+
+cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* scale_src,
+                             const qlin_fp8_t& out, cudaStream_t s, int num_sms, unsigned* err,
+                             uint64_t timeout_ns) {
+  const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
+  const cudaError_t e = set_smem<quant_fp8_kernel>();
+  if (e != cudaSuccess) return e;
+  return launch_pdl(quant_fp8_kernel, stream_grid(n_chunks, num_sms), kThreads, kSmem, s,
+                    static_cast<const uint4*>(x), n_chunks, scale_src, out.scale, fp8_op(out), err,
+                    timeout_ns);
 }
 
 cudaError_t launch_quant_fp8_rows(const void* w, int64_t N, int64_t K, const qlin_fp8_t& out,
