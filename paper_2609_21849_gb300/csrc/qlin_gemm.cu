@@ -462,15 +462,21 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
           // Full stages issue their MMAs with no branch between them; only a
           // partial last stage (K % 256 != 0) takes the loop.
           bool next_ready = false;
-          if (C::kK96 && nsteps == kStepsPerStage) {
-            // 256 elements as 96 + 96 + 64: an MMA of K = 96 takes the time of
-            // one of K = 64.  The next stage's barrier is tested (without
-            // waiting) while the first two run, so that a stage that is ready
-            // costs no test after the release (4608 x 12288 x 3072: 53.8 ->
-            // 53.5 us; with the four MMAs of an FP8 stage it gains nothing).
+          if (nsteps == kStepsPerStage) {
+            // The next stage's barrier is tested (without waiting) before the
+            // last MMA is issued, so that a stage that is ready costs no test
+            // after the release (4608 x 12288 x 3072 NVFP4: 53.8 -> 53.5 us).
+            // NVFP4: 256 elements as 96 + 96 + 64, an MMA of K = 96 taking the
+            // time of one of K = 64.
             if (elect_one()) {
-              issue96(0, acc0);
-              issue96(1, 1u);
+              if (C::kK96) {
+                issue96(0, acc0);
+                issue96(1, 1u);
+              } else {
+                issue(0, acc0);
+                issue(1, 1u);
+                issue(2, 1u);
+              }
             }
             if (kb + 1 < num_kb) {
               const bool wrap = stage + 1 == C::kStages;
@@ -480,13 +486,6 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
             }
             if (elect_one()) {
               issue(3, 1u);
-              release();
-            }
-          } else if (nsteps == kStepsPerStage) {
-            if (elect_one()) {
-              issue(0, acc0);
-#pragma unroll
-              for (int jj = 1; jj < kStepsPerStage; ++jj) issue(jj, 1u);
               release();
             }
           } else if (elect_one()) {
@@ -649,95 +648,85 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     // (tcgen05.st): lane l of the warp of each lane quarter takes the 16 bytes
     // of row l of every atom, which are its lane's four columns of the atom.
     // (In a pair each CTA would have to fill its own TMEM and arrive on the
-    // leader's barrier: measured far slower than the copies above.)  The four
-    // warps read the same bytes, so three of four reads hit L1; the lines are prefetched there
-    // kAhead stages before (the ring of slots is too short to hide L2).
+    // leader's barrier: measured far slower than the copies above.)  Two
+    // stages at a time, the next two loading meanwhile: one at a time, these
+    // warps' waits (~670 cycles a stage) held up the MMAs.
     if constexpr (kFp4 && !kPair) {
-      constexpr int kAhead = 4;
-      constexpr int kAtoms = 1 + C::kSfbAtoms;      // 128-row atom rows: A's, then W's
+      static_assert(C::kSfColsPerSlot == 32, "A's sixteen scale columns a stage, then W's");
       const int q = warp & 3;
       const int64_t k64 = p.K >> 6;                 // atoms of a 128-row block
-      const int arows = (int)((p.M + 127) >> 7), wrows = (int)((p.N + 127) >> 7);
-      // the operand bytes of atom row r (0: A; 1..: W) of a tile, or null
-      auto atom_row = [&](int ct, int r) -> const uint8_t* {
-        int mg, nb;
-        tile_coords(ct, groups_m, tiles_n, &mg, &nb);
-        const int i = r == 0 ? mg * kCM + rank : ((nb * kBN) >> 7) + r - 1;
-        if (i >= (r == 0 ? arows : wrows)) return nullptr;
-        return (r == 0 ? p.sfa : p.sfb) + (int64_t)i * k64 * 512;
-      };
-      // prefetch position: kAhead stages ahead of the loads
-      int pct = cid, pkb = 0;
-      const uint8_t* prow = nullptr;                // this lane's atom row
-      // lane -> 128-byte line of a stage: atom row lane / 4, 16 lines each,
-      // four of them by each warp
-      const int pr = lane >> 2;
-      auto prefetch_next = [&] {
-        if (pct >= num_ctiles) return;
-        if (pkb == 0) prow = pr < kAtoms ? atom_row(pct, pr) : nullptr;
-        const int64_t off = (int64_t)pkb * 2048 + q * 512 + (lane & 3) * 128;
-        if (prow != nullptr && off < k64 * 512)
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(prow + off));
-        if (++pkb == num_kb) {
-          pkb = 0;
-          pct += ncl;
+      // position of the next load: tile, stage and this lane's bytes of the
+      // tile's two atom rows (they exist: tiles start inside M and N)
+      int lct = cid, lkb = 0;
+      const uint8_t *arow = nullptr, *wrow = nullptr;
+      auto load_next = [&](uint32_t (&v)[32]) {
+        if (lct >= num_ctiles) return;
+        if (lkb == 0) {
+          int mg, nb;
+          tile_coords(lct, groups_m, tiles_n, &mg, &nb);
+          arow = p.sfa + mg * k64 * 512 + lane * 16;
+          wrow = p.sfb + ((nb * kBN) >> 7) * k64 * 512 + lane * 16;
+        }
+        const int ngroups = min(kStepsPerStage, k_steps - lkb * kStepsPerStage);
+#pragma unroll
+        for (int j = 0; j < kStepsPerStage; ++j) {
+          const int64_t off = (int64_t)(lkb * kStepsPerStage + j) * 512;
+          const uint4 a = j < ngroups ? ld_global_v4(arow + off) : make_uint4(0u, 0u, 0u, 0u);
+          const uint4 w = j < ngroups ? ld_global_v4(wrow + off) : make_uint4(0u, 0u, 0u, 0u);
+          v[4 * j] = a.x; v[4 * j + 1] = a.y; v[4 * j + 2] = a.z; v[4 * j + 3] = a.w;
+          v[16 + 4 * j] = w.x; v[17 + 4 * j] = w.y; v[18 + 4 * j] = w.z; v[19 + 4 * j] = w.w;
+        }
+        if (++lkb == num_kb) {
+          lkb = 0;
+          lct += ncl;
         }
       };
-      for (int i = 0; i < kAhead; ++i) prefetch_next();
       int stage = 0, slot = 0;
       int estage = 0;                               // the slot's last use: its stage and phase
       uint32_t ephase = 0;
       int filled = 0;
-      bool ok = true;
-      for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
-        const uint8_t* rows[kAtoms];
-#pragma unroll
-        for (int r = 0; r < kAtoms; ++r) rows[r] = atom_row(ct, r);
-        for (int kb = 0; kb < num_kb; ++kb) {
-          prefetch_next();
-          const int ngroups = min(kStepsPerStage, k_steps - kb * kStepsPerStage);
-          uint4 v[kAtoms][kStepsPerStage];
-#pragma unroll
-          for (int r = 0; r < kAtoms; ++r)
-#pragma unroll
-            for (int j = 0; j < kStepsPerStage; ++j)
-              v[r][j] = rows[r] != nullptr && j < ngroups
-                            ? ld_global_v4(rows[r] + (int64_t)(kb * kStepsPerStage + j) * 512 +
-                                           lane * 16)
-                            : make_uint4(0u, 0u, 0u, 0u);
-          // the slot is free once the MMAs of the stage that last used it
-          // have completed (kSfSlots <= kStages, so that stage's barrier
-          // cannot be a phase further on)
-          if (filled == C::kSfSlots) {
-            if (!mbar_wait_warp(&empty[estage], ephase, ctl)) {
-              ok = false;
-              break;
-            }
-            if (++estage == C::kStages) {
-              estage = 0;
-              ephase ^= 1u;
-            }
-          } else {
-            ++filled;
-          }
-          tc_fence_after();
-          const uint32_t t = tmem_base + ((uint32_t)(q * 32) << 16) +
-                             (uint32_t)(C::kSfColBase + slot * C::kSfColsPerSlot);
-#pragma unroll
-          for (int j = 0; j < kStepsPerStage; ++j) {
-            tmem_st4(t + 4 * j, v[0][j]);
-#pragma unroll
-            for (int r = 1; r < kAtoms; ++r)
-              tmem_st4(t + (uint32_t)(kStepsPerStage * C::kSfaCols + j * C::kSfbCols + 4 * (r - 1)),
-                       v[r][j]);
-          }
-          tmem_st_wait();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&full[stage]);
-          if (++stage == C::kStages) stage = 0;
-          if (++slot == C::kSfSlots) slot = 0;
+      // The next slot is free once the MMAs of the stage that last used it have
+      // completed (kSfSlots <= kStages, so that stage's barrier cannot be a
+      // phase further on).
+      auto acquire = [&]() -> bool {
+        if (filled < C::kSfSlots) {
+          ++filled;
+          return true;
         }
+        if (!mbar_wait_warp(&empty[estage], ephase, ctl)) return false;
+        if (++estage == C::kStages) {
+          estage = 0;
+          ephase ^= 1u;
+        }
+        return true;
+      };
+      auto store = [&](const uint32_t (&v)[32]) {
+        tmem_st32(tmem_base + ((uint32_t)(q * 32) << 16) +
+                      (uint32_t)(C::kSfColBase + slot * C::kSfColsPerSlot),
+                  v);
+        if (++slot == C::kSfSlots) slot = 0;
+      };
+      auto arrive = [&] {
+        if (lane == 0) mbar_arrive(&full[stage]);
+        if (++stage == C::kStages) stage = 0;
+      };
+      const int64_t total = (int64_t)((num_ctiles - cid + ncl - 1) / ncl) * num_kb;
+      uint32_t v0[32], v1[32];
+      load_next(v0);
+      load_next(v1);
+      for (int64_t it = 0; it < total; it += 2) {
+        const bool two = it + 1 < total;
+        if (!acquire() || (two && !acquire())) break;
+        tc_fence_after();
+        store(v0);
+        if (two) store(v1);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        arrive();
+        if (two) arrive();
+        load_next(v0);
+        load_next(v1);
       }
     }
   } else {
