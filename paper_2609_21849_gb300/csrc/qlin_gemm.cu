@@ -72,7 +72,6 @@ struct Cfg {
   // every lane).
   static constexpr int kSfWarps = kFp4 ? 4 : 0;
   static constexpr bool kSfCopy = kFp4 && kPair;   // scales by TMA and tcgen05.cp
-  static_assert(!kSfCopy || kStepsPerStage % kSfWarps == 0, "whole MMA steps per copy warp");
   static constexpr int kSfProducer = kSfCopy ? 2 + kSfWarps : -1;
   static constexpr int kEpiWarp0 = 2 + kSfWarps + (kSfCopy ? 1 : 0);
   static constexpr int kEpiWarps = 8;
@@ -93,9 +92,12 @@ struct Cfg {
   // stores.
   static constexpr bool kDirectStore = kPair && kBN == 256;
   static constexpr int kOutBytes = kDirectStore ? 0 : kEpiWarps * 2 * 2048;
-  // Pairs: five scale slots beside six operand stages (four slots: 58.3 us
-  // instead of 54.8; TMEM has no room for a sixth beside the accumulator).
-  static constexpr int kSfSmemSlots = kSfCopy ? 5 : 0;
+  // Pairs: one shared-memory scale slot per scale warp.  The warps take the
+  // stages in turn, so each waits on a barrier of its own slot only and sees
+  // every phase of it; with another number of slots a warp would wait for a
+  // phase whose predecessor it has not seen complete, and a parity wait
+  // returns at once in that case.
+  static constexpr int kSfSmemSlots = kSfCopy ? kSfWarps : 0;
   static constexpr int kSfSlotBytes = (1 + kSfbAtoms) * kStepsPerStage * 512;
   static constexpr int kSfBytes = kSfSmemSlots * kSfSlotBytes;
   static constexpr int kStagesRaw = (kSmemBudget - kOutBytes - kSfBytes) / kStageBytes;
@@ -112,9 +114,10 @@ struct Cfg {
   // ring (the scale warps' wait for a slot relies on that).
   static constexpr int kSfColsPerSlot = kStepsPerStage * kSfColsPerStep;
   static constexpr int kSfSlotsRaw = kFp4 ? (512 - kSfColBase) / kSfColsPerSlot : 1;
-  static constexpr int kSfSlots =
-      kSfCopy ? kSfSmemSlots : kSfSlotsRaw < kStages ? kSfSlotsRaw : kStages;
-  static_assert(!kFp4 || (kSfSlots <= kSfSlotsRaw && kSfSlots <= kStages), "scale slots");
+  static constexpr int kSfSlots = kSfSlotsRaw < kStages ? kSfSlotsRaw : kStages;
+  // (a scale warp of a pair waits for the MMAs of every kSfWarps-th stage only;
+  // its wait before covers the phase between as long as this holds)
+  static_assert(!kSfCopy || kSfWarps < kStages, "phases between two waits of a scale warp");
   static constexpr int kTmemCols =
       pow2_at_least(kSfColBase + kSfSlots * kSfColsPerSlot);
   static constexpr int kBarrierBytes = 512;
@@ -238,7 +241,8 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   uint64_t* full = reinterpret_cast<uint64_t*>(sf_ring + C::kSfBytes);
   uint64_t* empty = full + C::kStages;
   uint64_t* sf_full = empty + C::kStages;       // kSfCopy: a slot's scale bytes landed
-  uint64_t* tmem_full = sf_full + C::kSfSmemSlots;
+  uint64_t* sf_empty = sf_full + C::kSfSmemSlots;   // and its copies to TMEM are done
+  uint64_t* tmem_full = sf_empty + C::kSfSmemSlots;
   uint64_t* tmem_empty = tmem_full + 2;
   uint64_t* mma_done = tmem_empty + 2;
   uint64_t* sf_done = mma_done + 1;             // kSfCopy: one per scale warp
@@ -256,13 +260,14 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
-      // NVFP4: the scale warps also arrive on full, so the MMA issuer waits
-      // on one barrier per stage
-      mbar_init(&full[s], 1 + C::kSfWarps);
+      // NVFP4: the scale warps also arrive on full (pairs: the one that copies
+      // the stage), so the MMA issuer waits on one barrier per stage
+      mbar_init(&full[s], C::kSfCopy ? 2 : 1 + C::kSfWarps);
       mbar_init(&empty[s], 1);
     }
     for (int s = 0; s < C::kSfSmemSlots; ++s) {
       mbar_init(&sf_full[s], 1);
+      mbar_init(&sf_empty[s], 1);
     }
     for (int w = 0; w < C::kSfWarps; ++w) mbar_init(&sf_done[w], 1);
     for (int a = 0; a < 2; ++a) {
@@ -540,28 +545,21 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   } else if (C::kSfCopy && warp == C::kSfProducer) {
     // ------------------------------------------- scale producer (pairs) ---
     // The A scale atoms of this CTA's M tile (2 KB a stage) and the W scale
-    // atoms of the whole N tile (4 KB); both complete on the leader.  The scale slots (shared memory and TMEM) are a ring of their
-    // own: a slot is free once the MMAs of the stage that last used it have
-    // completed.  (kSfSlots <= kStages: that stage's next MMAs wait for these
-    // scales, so its barrier cannot be a phase further on.)
+    // atoms of the whole N tile (4 KB); both complete on the leader.  A slot
+    // is free once its copies to TMEM have read it, so that the scales of the
+    // next stages wait in shared memory for their TMEM slot.
     const uint32_t bar0 = __shfl_sync(0xFFFFFFFFu, mapa_shared(sf_full, 0), 0);
-    int slot = 0, issued = 0, estage = 0;
-    uint32_t phase = 0, ephase = 0;
+    int slot = 0, issued = 0;
+    uint32_t phase = 0;
     bool ok = true;
     for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
       int mg, nb;
       tile_coords(ct, groups_m, tiles_n, &mg, &nb);
       const int a_row = mg * kCM + rank, w_row = (nb * kBN) >> 7;
       for (int kb = 0; kb < num_kb; ++kb) {
-        if (issued >= C::kSfSlots) {
-          if (!mbar_wait_warp(&empty[estage], ephase, ctl)) {
-            ok = false;
-            break;
-          }
-          if (++estage == C::kStages) {
-            estage = 0;
-            ephase ^= 1u;
-          }
+        if (!mbar_wait_warp(&sf_empty[slot], phase ^ 1u, ctl)) {
+          ok = false;
+          break;
         }
         uint8_t* const dst = sf_ring + slot * C::kSfSlotBytes;
         const uint32_t bar = bar0 + (uint32_t)(slot * 8);
@@ -572,17 +570,17 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
                            w_row, 0, 0);
         }
         ++issued;
-        if (++slot == C::kSfSlots) {
+        if (++slot == C::kSfSmemSlots) {
           slot = 0;
           phase ^= 1u;
         }
       }
     }
     if (leader && lane == 0) {   // the last copies land before the pair exits
-      const int n_drain = min(issued, C::kSfSlots);
+      const int n_drain = min(issued, C::kSfSmemSlots);
       for (int i = 0; i < n_drain; ++i) {
         if (--slot < 0) {
-          slot = C::kSfSlots - 1;
+          slot = C::kSfSmemSlots - 1;
           phase ^= 1u;
         }
         mbar_drain(&sf_full[slot], phase, p.timeout_ns, p.err);
@@ -590,50 +588,63 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     }
   } else if (C::kSfCopy && warp < C::kEpiWarp0) {
     // ------------------------------------- NVFP4 scale copies (pairs) ---
-    // Block scales move shared -> TMEM from threads of their own (one lane of
-    // each scale warp), beside the MMA stream: a tcgen05.cp occupies its
-    // issuing thread ~80-120 cycles while the MMAs run, and a stage needs 12,
-    // so each warp copies the atoms of an equal share of the stage's 64-element
-    // groups.  Copies issued from separate warps overlap (12 take ~850 cycles
-    // from two warps, ~510 from four, with the MMAs running: the MMAs' rate is
-    // unaffected).  (A converged instruction from several lanes of one warp
-    // does not issue one copy per lane.)  The leader's copies fill both SMs'
-    // TMEM from their own shared memory.
+    // Block scales move shared -> TMEM beside the MMA stream, the stages in
+    // turn to the four scale warps: a tcgen05.cp occupies its issuing thread
+    // ~60-120 cycles while the MMAs run, and a stage needs 12, so one warp
+    // takes a stage in about two stages' time.  The leader's copies fill both
+    // SMs' TMEM from their own shared memory.
     if (leader) {
       const int sw = warp - 2;
-      int stage = 0, slot = 0;
+      int turn = 0;                       // stage count modulo the warps
+      int stage = 0, slot = 0, tslot = 0;
       uint32_t phase = 0;
+      int filled = 0, estage = 0;         // the TMEM slot's last use: its stage and phase
+      uint32_t ephase = 0;
       bool ok = true;
       for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait_warp(&sf_full[slot], phase, ctl)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sSFA = smem_u32(sf_ring + slot * C::kSfSlotBytes);
-          const uint32_t sSFB = sSFA + kStepsPerStage * 512;
-          const uint32_t sf0 = tmem_base + (uint32_t)(C::kSfColBase + slot * C::kSfColsPerSlot);
-          const int nsteps = min(kStepsPerStage, k_steps - kb * kStepsPerStage);
-          constexpr int kShare = C::kSfCopy ? kStepsPerStage / C::kSfWarps : 1;
-          const int j_end = min(nsteps, (sw + 1) * kShare);
-          if (elect_one()) {
-            for (int j = sw * kShare; j < j_end; ++j) {
-              tc_cp_scales_pair(sf0 + (uint32_t)(j * C::kSfaCols), sdesc_scales(sSFA + j * 512));
-#pragma unroll
-              for (int r = 0; r < C::kSfbAtoms; ++r)
-                tc_cp_scales_pair(
-                    sf0 + (uint32_t)(kStepsPerStage * C::kSfaCols + j * C::kSfbCols + 4 * r),
-                    sdesc_scales(sSFB + r * kStepsPerStage * 512 + j * 512));
+          if (turn == sw) {
+            // the slot's scales have landed, and the MMAs of the stage that
+            // last used the TMEM slot have completed (kSfSlots <= kStages:
+            // that stage's next MMAs wait for these scales, so its barrier
+            // cannot be a phase further on)
+            if (!mbar_wait_warp(&sf_full[slot], phase, ctl) ||
+                (filled == C::kSfSlots && !mbar_wait_warp(&empty[estage], ephase, ctl))) {
+              ok = false;
+              break;
             }
-            // the stage is ready for its MMAs once these copies and its
-            // operands have landed: both arrive on its full barrier
-            tc_commit_pair_mc(&full[stage], 1);
+            tc_fence_after();
+            const uint32_t sSFA = smem_u32(sf_ring + slot * C::kSfSlotBytes);
+            const uint32_t sSFB = sSFA + kStepsPerStage * 512;
+            const uint32_t sf0 = tmem_base + (uint32_t)(C::kSfColBase + tslot * C::kSfColsPerSlot);
+            const int nsteps = min(kStepsPerStage, k_steps - kb * kStepsPerStage);
+            if (elect_one()) {
+              for (int j = 0; j < nsteps; ++j) {
+                tc_cp_scales_pair(sf0 + (uint32_t)(j * C::kSfaCols), sdesc_scales(sSFA + j * 512));
+#pragma unroll
+                for (int r = 0; r < C::kSfbAtoms; ++r)
+                  tc_cp_scales_pair(
+                      sf0 + (uint32_t)(kStepsPerStage * C::kSfaCols + j * C::kSfbCols + 4 * r),
+                      sdesc_scales(sSFB + r * kStepsPerStage * 512 + j * 512));
+              }
+              // the stage is ready for its MMAs once these copies and its
+              // operands have landed: both arrive on its full barrier
+              tc_commit_pair_mc(&full[stage], 1);
+              tc_commit_pair_mc(&sf_empty[slot], kMask);   // both CTAs' slots are read
+            }
           }
+          if (++turn == C::kSfWarps) turn = 0;
           if (++stage == C::kStages) stage = 0;
-          if (++slot == C::kSfSlots) {
+          if (++slot == C::kSfSmemSlots) {
             slot = 0;
             phase ^= 1u;
+          }
+          if (++tslot == C::kSfSlots) tslot = 0;
+          if (filled < C::kSfSlots) {
+            ++filled;
+          } else if (++estage == C::kStages) {
+            estage = 0;
+            ephase ^= 1u;
           }
         }
       }
