@@ -1,0 +1,123 @@
+"""GPU parity at the edges of the size rules that choose a kernel: the dynamic
+quantizers' routes (clusters that each read x, x in registers or shared memory,
+two phases over x) and the GEMM's tile configurations and K stages (256 NVFP4
+elements as 96 + 96 + 64, partial stages, the scale rings' wrap-around).
+
+Codes and scales are compared bit for bit with the oracle's; GEMM outputs are
+within the tolerance of the exact product (2e-3 of the operands' row norms) on
+a few rows per 128-row tile."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_2609_21849_gb300 import qlin, synthetic
+
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    from gpu_util import (GEMM_TOL, assert_nvfp4_equal, bf16_bits, f32, gemm_errors, to_dev, u8)
+
+# x of n chunks (8 values): 1 MB is 65536 chunks, the cluster route's last
+# size; x in registers reaches 12288 chunks per SM, in shared memory 14336.
+SMS = 152
+ROUTES = [(1, 64), (3, 64), (17, 448), (256, 2048), (257, 2048), (1023, 512),
+          (12288 * SMS // 512, 4096), (12288 * SMS // 512 + 1, 4096),
+          (14336 * SMS // 512, 4096), (14336 * SMS // 512 + 1, 4096)]
+
+
+@pytest.mark.parametrize("M,K", ROUTES)
+def test_dynamic_routes_match_oracle(M, K):
+    # twice with one workspace, the smaller amax second: the scratch is left
+    # zero, and a stale maximum would show
+    ws = qlin.alloc_workspace()
+    q4, q8 = qlin.alloc_nvfp4(M, K), qlin.alloc_fp8(M, K, False)
+    for seed, scale in ((5, 1), (6, 64)):
+        bits = synthetic.act_entry_outliers(seed, M, K)
+        x = (to_dev(bits).float() / scale).bfloat16()
+        bits = bf16_bits(x)
+        qlin.qlin_quantize_act_nvfp4(x, None, q4, ws)
+        qlin.qlin_quantize_act_fp8(x, None, q8, ws)
+        assert qlin.qlin_sync_status() == 0
+        assert_nvfp4_equal(q4, oracle.quant_nvfp4(bits), f"{M}x{K}")
+        c8, s8 = oracle.quant_fp8(bits)[:2]
+        assert f32(q8.scale)[0] == np.float32(s8)
+        assert np.array_equal(u8(q8.codes), c8)
+    assert int(ws.count_nonzero()) == 0
+
+
+@pytest.mark.parametrize("shift", [0, 8])
+def test_static_nvfp4_alignment_and_partial_tile(shift):
+    # x 32-byte aligned (one 32-byte load per block) and only 16-byte aligned
+    # (two 16-byte loads); 2055 * 64 / 8 chunks end in a partial tile
+    M, K = 2055, 64
+    bits = synthetic.act_entry_outliers(9, M, K)
+    buf = torch.zeros(M * K + 16, dtype=torch.bfloat16, device="cuda")
+    x = buf[shift:shift + M * K].view(M, K)
+    x.copy_(to_dev(bits))
+    s = np.float32(0.03)
+    q = qlin.qlin_quantize_act_nvfp4(x, torch.tensor([s], device="cuda"))
+    assert qlin.qlin_sync_status() == 0
+    assert_nvfp4_equal(q, oracle.quant_nvfp4(bits, s), f"shift {shift}")
+
+
+@pytest.mark.parametrize("N,K", [(200, 64), (200, 3072), (33, 3136), (9, 12288)])
+def test_fp8_weight_rows(N, K):
+    # rows held in registers up to K = 3072, read twice beyond
+    (w,) = synthetic.weights(11, [(N, K)], 0.02)
+    q = qlin.qlin_quantize_weight(to_dev(w), qlin.QLIN_FMT_FP8)
+    codes, scales = oracle.quant_fp8_rows(w)[:2]
+    assert np.array_equal(u8(q.codes), codes) and np.array_equal(f32(q.scale), scales)
+
+
+def _rows(M):
+    r = {0, M - 1} | {t * 128 + (37 * t) % 128 for t in range((M + 127) // 128)}
+    return np.array(sorted(i for i in r if i < M))
+
+
+# (M, N): 64-wide, 128-wide and pair tiles (with a partial pair); K: one
+# partial stage, full ones, every remainder of a stage, and K long enough that
+# every ring wraps
+@pytest.mark.parametrize("M,N", [(40, 192), (300, 2560), (3000, 1024), (4700, 2112)])
+@pytest.mark.parametrize("K", [64, 192, 256, 832, 2688])
+@pytest.mark.parametrize("fmt", ["nvfp4", "fp8"])
+def test_gemm_tiles_and_stages(fmt, M, N, K):
+    x = synthetic.act_entry_outliers(21, M, K)
+    (w,) = synthetic.weights(22, [(N, K)], 0.02)
+    rows = _rows(M)
+    if fmt == "nvfp4":
+        A = qlin.qlin_quantize_act_nvfp4(to_dev(x))
+        W = qlin.qlin_quantize_weight(to_dev(w), qlin.QLIN_FMT_NVFP4)
+        y = qlin.qlin_gemm_nvfp4(A, W)
+        c, s, ts = oracle.quant_nvfp4(x)
+        ref = oracle.gemm_nvfp4((c[rows], s[rows], ts), oracle.quant_nvfp4(w))
+    else:
+        A = qlin.qlin_quantize_act_fp8(to_dev(x))
+        W = qlin.qlin_quantize_weight(to_dev(w), qlin.QLIN_FMT_FP8)
+        y = qlin.qlin_gemm_fp8(A, W)
+        c, s = oracle.quant_fp8(x)[:2]
+        ref = oracle.gemm_fp8((c[rows], s), oracle.quant_fp8_rows(w))
+    assert qlin.qlin_sync_status() == 0
+    err, exact = gemm_errors(bf16_bits(y)[rows], *ref)
+    assert err.max() <= GEMM_TOL and exact >= 0.99, (err.max(), exact)
+
+
+def test_back_to_back_launches_see_new_operands():
+    # the scales of single-CTA tiles are read through L1: two activations
+    # quantized in turn into one operand, no wait between the launches
+    M, N, K = 256, 384, 1024
+    xs = [to_dev(synthetic.act_entry_outliers(s, M, K)) for s in (31, 32)]
+    (w,) = synthetic.weights(33, [(N, K)], 0.02)
+    W = qlin.qlin_quantize_weight(to_dev(w), qlin.QLIN_FMT_NVFP4)
+    A, ws = qlin.alloc_nvfp4(M, K), qlin.alloc_workspace()
+    want = []
+    for x in xs:
+        want.append(qlin.qlin_gemm_nvfp4(qlin.qlin_quantize_act_nvfp4(x, None, None, ws), W))
+        torch.cuda.synchronize()
+    got = [torch.empty_like(want[0]) for _ in range(40)]
+    for i, y in enumerate(got):
+        qlin.qlin_quantize_act_nvfp4(xs[i & 1], None, A, ws)
+        qlin.qlin_gemm_nvfp4(A, W, y)
+    assert qlin.qlin_sync_status() == 0
+    assert all(torch.equal(y, want[i & 1]) for i, y in enumerate(got))
