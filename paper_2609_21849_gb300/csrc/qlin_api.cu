@@ -160,7 +160,7 @@ qlin_status qlin_quantize_act_nvfp4(const void* x_bf16, int64_t M, int64_t K,
                                          static_cast<unsigned*>(workspace) + kWsQuant, false, s,
                                          sms, status, timeout()));
   } else {
-    QLIN_CUDA(launch_quant_nvfp4(x_bf16, M, K, static_scale, *out, s, sms, status, timeout()));
+    QLIN_CUDA(launch_quant_nvfp4(x_bf16, M, K, static_scale, *out, s, sms));
   }
   return QLIN_OK;
 }
@@ -380,8 +380,7 @@ qlin_status qlin_linear_dynamic(const qlin_nvfp4_t* A, const qlin_nvfp4_t* W, vo
   unsigned* status;
   int sms;
   QLIN_TRY(device_state(&status, &sms));
-  QLIN_CUDA(launch_quant_nvfp4(y_bf16, A->rows, W->rows, y_q->tensor_scale, *y_q, s, sms, status,
-                               timeout()));
+  QLIN_CUDA(launch_quant_nvfp4(y_bf16, A->rows, W->rows, y_q->tensor_scale, *y_q, s, sms));
   return QLIN_OK;
 }
 

@@ -2,23 +2,27 @@
 // post-training quantization; activations are quantized at run time, weights
 // once).  All kernels here are HBM-bandwidth bound streaming kernels:
 //
-//   onepass_kernel<Op>    dynamic scale in one read of x: the grid holds x in
-//                         shared memory, reduces amax across the grid, then
-//                         quantizes from shared memory (when x fits on chip)
-//   amax_kernel           max |x| over a tensor (the dynamic tensor scale)
-//   quant_kernel<NVFP4>   bf16 -> packed e2m1 codes + E4M3 block scales in the
+// Dynamic tensor scale, by the size of x (launch_dynamic):
+//   cluster_quant_kernel  up to 1 MB: every cluster of eight CTAs reads all of
+//                         x, so no grid-wide barrier
+//   regpass_kernel        (NVFP4) x held in registers: one read of x, the amax
+//                         reduced across a cooperative grid
+//   onepass_kernel        the same with x in shared memory
+//   two_phase_kernel      larger x: amax, then the tiles again in reverse order,
+//                         in one cooperative launch
+// Static tensor scale:
+//   quant_nvfp4_kernel    bf16 -> packed e2m1 codes + E4M3 block scales in the
 //                         tensor-core scale layout + FP32 tensor scale
-//   quant_kernel<FP8>     bf16 -> E4M3 codes with one tensor scale
-//   quant_fp8_rows_kernel bf16 weights -> E4M3 codes with one scale per row
+//   quant_fp8_kernel      bf16 -> E4M3 codes with one tensor scale
+// Weights:
+//   quant_fp8_rows_kernel bf16 -> E4M3 codes with one scale per row
 //
-// Streaming structure: the [M, K] input is a flat array of 16-byte chunks (8
-// bf16), cut into 16 KB tiles.  A persistent grid (three CTAs per SM)
-// streams tiles through a four-deep shared-memory ring filled by bulk copies,
-// so ~192 KB per SM of input is in flight regardless of register pressure.
-// Inside a tile, each thread takes consecutive units of chunks (NVFP4: one
-// 16-element block per lane, so four neighbouring lanes hold one 64-element
-// group, whose four block scales form one 32-bit word of the scale layout;
-// because K % 64 == 0 a group never straddles a row).
+// The [M, K] input is a flat array of 16-byte chunks (8 bf16); a unit is the
+// two chunks of one NVFP4 block, and four neighbouring lanes hold one
+// 64-element group (because K % 64 == 0 a group never straddles a row).  The
+// kernels that stream (stream_tiles, two_phase_kernel) cut it into 16 KB tiles
+// that a persistent grid (three CTAs per SM) takes through a four-deep
+// shared-memory ring filled by bulk copies, ~192 KB per SM of input in flight.
 #include <atomic>
 
 #include "qlin_internal.h"
@@ -118,7 +122,7 @@ struct Nvfp4Op {
   __device__ __forceinline__ void unit(const uint4 (&v)[2], uint64_t c, bool valid) {
     uint32_t code0, code1, word;
     quantize_block<kDivide>(v, max(chunk_abs_max_bits(v[0]), chunk_abs_max_bits(v[1])), code0, code1,
-                   word);
+                            word);
     if (valid) {
       reinterpret_cast<uint2*>(codes)[c >> 1] = make_uint2(code0, code1);
       {
@@ -378,12 +382,30 @@ __device__ __forceinline__ float static_scale(const float* scale_src, float* sde
   return s_dec;
 }
 
+// NVFP4 with a static scale: x goes straight to registers (32 bytes, one block,
+// per load where x is 32-byte aligned), each thread loading its next tile's
+// units while it quantizes this one's.  Two CTAs of 512 threads per SM keep
+// 64 KB per SM of loads in flight.  Bound by HBM: 18432 x 3072 in 22.4 us
+// (6.5 TB/s), through the shared-memory ring of the other streaming kernels
+// 24.1 us (its block reads have two-way bank conflicts); 4608 x 3072 7.5 us,
+// was 7.7.  256-thread CTAs with one to three units measured 22.3-23.6 us and
+// 7.7-8.6 us.
+constexpr int kDirectPerSm = 2;
+constexpr int kDirectUnits = 2;                                       // per thread and tile
+constexpr uint32_t kDirectTile = 2u * kThreads * kDirectUnits;        // chunks: 32 KB
+
+__device__ __forceinline__ void ldg256(const uint4* p, uint4 (&v)[2]) {
+  asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0].x), "=r"(v[0].y), "=r"(v[0].z), "=r"(v[0].w), "=r"(v[1].x),
+                 "=r"(v[1].y), "=r"(v[1].z), "=r"(v[1].w)
+               : "l"(p));
+}
+
 template <typename Idx>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSm)
+__global__ void __launch_bounds__(kThreads, kDirectPerSm)
     quant_nvfp4_kernel(const uint4* __restrict__ x, uint64_t n_chunks, int64_t K,
                        const float* scale_src, float* sdec_out, uint32_t* __restrict__ codes,
-                       uint8_t* __restrict__ scales, uint3 row_div, unsigned* err,
-                       uint64_t timeout_ns) {
+                       uint8_t* __restrict__ scales, uint3 row_div) {
   l2_prefetch_first_tile(x, n_chunks);
   grid_dep_wait();
   grid_dep_launch();
@@ -397,10 +419,49 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
   op.K = K;
   op.codes = codes;
   op.scales = scales;
-  stream_tiles(
-      x, n_chunks, op,
-      [&](Nvfp4Op<Idx>& o) { o.s_enc = encode_scale(static_scale(scale_src, sdec_out)); }, err,
-      timeout_ns);
+  const uint64_t n_tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
+  const bool v8 = (reinterpret_cast<uintptr_t>(x) & 31u) == 0;
+  auto first = [&](uint64_t t, int k) {   // first chunk of unit k of tile t
+    return t * kDirectTile + 2u * (uint32_t)(k * kThreads + threadIdx.x);
+  };
+  auto load = [&](uint64_t t, uint4 (&v)[kDirectUnits][2]) {
+#pragma unroll
+    for (int k = 0; k < kDirectUnits; ++k) {
+      const uint64_t c = first(t, k);   // units never straddle n_chunks
+      if (c >= n_chunks) {
+        v[k][0] = v[k][1] = make_uint4(0u, 0u, 0u, 0u);
+      } else if (v8) {
+        ldg256(x + c, v[k]);
+      } else {
+        v[k][0] = ldg128(x + c);
+        v[k][1] = ldg128(x + c + 1);
+      }
+    }
+  };
+  auto quantize = [&](uint64_t t, const uint4 (&v)[kDirectUnits][2]) {
+#pragma unroll
+    for (int k = 0; k < kDirectUnits; ++k) {
+      const uint64_t c = first(t, k);
+      op.unit(v[k], c, c < n_chunks);
+    }
+  };
+  uint4 v[kDirectUnits][2], w[kDirectUnits][2];
+  uint64_t t = blockIdx.x;
+  if (t < n_tiles) load(t, v);
+  op.s_enc = encode_scale(static_scale(scale_src, sdec_out));
+  op.init();
+  __syncthreads();
+  while (t < n_tiles) {
+    uint64_t nt = t + gridDim.x;
+    if (nt < n_tiles) load(nt, w);
+    quantize(t, v);
+    t = nt;
+    if (t >= n_tiles) break;
+    nt = t + gridDim.x;
+    if (nt < n_tiles) load(nt, v);
+    quantize(t, w);
+    t = nt;
+  }
 }
 
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
@@ -415,12 +476,14 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
       timeout_ns);
 }
 
-// FP8 weights, one scale per row: one warp per row, two passes over the row
-// (the second hits L1/L2).  Offline, once per layer.
-__global__ void __launch_bounds__(kThreads) quant_fp8_rows_kernel(const uint4* __restrict__ w,
-                                                                  int64_t rows, int64_t K,
-                                                                  float* __restrict__ s_rows,
-                                                                  uint2* __restrict__ codes) {
+// FP8 weights, one scale per row: one warp per row, held in registers up to
+// K = 3072 (12288 x 3072: 21.3 -> 19.1 us), else two passes over it (the second
+// hits L1/L2).  Offline, once per layer.
+constexpr int kRowRegs = 12;   // chunks per lane
+
+__global__ void __launch_bounds__(kThreads, 2)
+    quant_fp8_rows_kernel(const uint4* __restrict__ w, int64_t rows, int64_t K,
+                          float* __restrict__ s_rows, uint2* __restrict__ codes) {
   grid_dep_wait();
   grid_dep_launch();
   const int lane = threadIdx.x & 31;
@@ -430,6 +493,30 @@ __global__ void __launch_bounds__(kThreads) quant_fp8_rows_kernel(const uint4* _
   for (int64_t r = warp; r < rows; r += nwarps) {
     const uint4* wr = w + r * cpr;
     uint32_t m = 0;
+    if (cpr <= 32 * kRowRegs) {
+      uint4 v[kRowRegs];
+#pragma unroll
+      for (int i = 0; i < kRowRegs; ++i)
+        v[i] = lane + 32 * i < cpr ? ldg128(wr + lane + 32 * i) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int i = 0; i < kRowRegs; ++i) m = max(m, chunk_abs_max_bits(v[i]));
+      m = __reduce_max_sync(0xFFFFFFFFu, m);
+      const float amax = __uint_as_float(m << 16);
+      const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f);
+      const float s_enc = encode_scale(s_dec);
+      if (lane == 0) s_rows[r] = s_dec;
+#pragma unroll
+      for (int i = 0; i < kRowRegs; ++i) {
+        if (lane + 32 * i >= cpr) continue;
+        float f[8];
+        unpack8(v[i], f);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) f[e] = __fmul_rn(f[e], s_enc);
+        codes[r * cpr + lane + 32 * i] =
+            make_uint2(e4m3x4(f[0], f[1], f[2], f[3]), e4m3x4(f[4], f[5], f[6], f[7]));
+      }
+      continue;
+    }
     for (int64_t c = lane; c < cpr; c += 32) m = max(m, chunk_abs_max_bits(__ldg(wr + c)));
     m = __reduce_max_sync(0xFFFFFFFFu, m);
     const float amax = __uint_as_float(m << 16);
@@ -1091,22 +1178,17 @@ cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const 
 }
 
 cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float* scale_src,
-                               const qlin_nvfp4_t& out, cudaStream_t s, int num_sms,
-                               unsigned* err, uint64_t timeout_ns) {
+                               const qlin_nvfp4_t& out, cudaStream_t s, int num_sms) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
-  const int grid = stream_grid(n_chunks, num_sms);
+  const uint64_t tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
+  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms * kDirectPerSm);
   auto* xin = static_cast<const uint4*>(x);
   auto* codes = reinterpret_cast<uint32_t*>(out.codes);
   const uint3 row_div = invariant_divisor((uint32_t)(K >> 3));
-  cudaError_t e;
-  if (n_chunks < (1ull << 32)) {   // 32-bit index math is enough
-    if ((e = set_smem<quant_nvfp4_kernel<uint32_t>>()) != cudaSuccess) return e;
-    return launch_pdl(quant_nvfp4_kernel<uint32_t>, grid, kThreads, kSmem, s, xin, n_chunks, K,
-                      scale_src, out.tensor_scale, codes, out.scales, row_div, err, timeout_ns);
-  }
-  if ((e = set_smem<quant_nvfp4_kernel<uint64_t>>()) != cudaSuccess) return e;
-  return launch_pdl(quant_nvfp4_kernel<uint64_t>, grid, kThreads, kSmem, s, xin, n_chunks, K,
-                    scale_src, out.tensor_scale, codes, out.scales, row_div, err, timeout_ns);
+  auto kern = n_chunks < (1ull << 32) ? quant_nvfp4_kernel<uint32_t>   // 32-bit index math is enough
+                                      : quant_nvfp4_kernel<uint64_t>;
+  return launch_pdl(kern, grid, kThreads, 0, s, xin, n_chunks, K, scale_src, out.tensor_scale,
+                    codes, out.scales, row_div);
 }
 
 cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* scale_src,
