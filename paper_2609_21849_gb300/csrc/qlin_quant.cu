@@ -172,6 +172,9 @@ struct Nvfp4Op {
       }
     }
   }
+  __device__ __forceinline__ void pair(const uint4 (&v)[2], uint64_t c, bool valid) {
+    unit(v, c, valid);
+  }
   // The two chunks of one thread, with no table.
   __device__ __forceinline__ void block(const uint4 (&v)[2], uint32_t c, bool valid) {
     unit<true>(v, c, valid);
@@ -247,6 +250,20 @@ struct Fp8Op {
 #pragma unroll
     for (int i = 0; i < 8; ++i) f[i] = __fmul_rn(f[i], s_enc);
     codes[c] = make_uint2(e4m3x4(f[0], f[1], f[2], f[3]), e4m3x4(f[4], f[5], f[6], f[7]));
+  }
+  __device__ __forceinline__ void pair(const uint4 (&v)[2], uint64_t c, bool valid) {
+    if (!valid) return;
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      float f[8];
+      unpack8(v[k], f);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) f[i] = __fmul_rn(f[i], s_enc);
+      w[2 * k] = e4m3x4(f[0], f[1], f[2], f[3]);
+      w[2 * k + 1] = e4m3x4(f[4], f[5], f[6], f[7]);
+    }
+    *reinterpret_cast<uint4*>(codes + c) = make_uint4(w[0], w[1], w[2], w[3]);
   }
   __device__ __forceinline__ void block(const uint4 (&v)[2], uint32_t c, bool valid) {
     const uint4 a[1] = {v[0]}, b[1] = {v[1]};
@@ -760,19 +777,18 @@ __global__ void __launch_bounds__(kRegThreads, 1)
   op.template run_units<kRegUnits, kRegStride>(v, bm, n, c_begin);
 }
 
-// Dynamic scale of an x that does not fit on chip: one cooperative launch (the
-// streaming kernels' grid, three CTAs per SM) reads x for its amax, meets at
-// the grid barrier and quantizes its tiles in reverse order.  The last
-// kStages tiles of every CTA (29 MB in all) are still in its ring, and the
-// ones before them are the lines most recently in L2.  Bound by HBM: x once and
-// what of it L2 has lost a second time.
+// Dynamic scale of an x that does not fit on chip: one cooperative launch reads
+// x for its amax, meets at the grid barrier and quantizes its tiles in reverse
+// order, so that it starts on the lines most recently in L2 (the first of them
+// loading while the grid meets).  Loads as in quant_nvfp4_kernel.  Bound by HBM:
+// x once, and what of it L2 has lost a second time.  18432 x 3072: NVFP4 39.8
+// us, FP8 39.3 us; an amax kernel and the quantizer after it took 48.1 and 50.1
+// us, one launch through the shared-memory ring (its last tiles kept) 44.7 and
+// 40.0 us.
 template <typename Op>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSm)
+__global__ void __launch_bounds__(kThreads, kDirectPerSm)
     two_phase_kernel(const uint4* __restrict__ x, uint64_t n_chunks, Op op, float qmax,
                      float* sdec_out, unsigned* sync, unsigned* err, uint64_t timeout_ns) {
-  extern __shared__ __align__(128) uint8_t qsm[];
-  uint4* buf = reinterpret_cast<uint4*>(qsm);
-  uint64_t* full = reinterpret_cast<uint64_t*>(qsm + kStages * kTileChunks * 16);
   __shared__ uint32_t warp_max[kThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
@@ -780,113 +796,66 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
   l2_prefetch_first_tile(x, n_chunks);
   grid_dep_wait();
   grid_dep_launch();
-  const int tid = threadIdx.x;
-  const uint64_t n_tiles = (n_chunks + kTileChunks - 1) / kTileChunks;
-  // this CTA's tiles are blockIdx.x + i * gridDim.x, i in [0, n_own); tile i
-  // sits in stage i % kStages
-  const int64_t n_own = (int64_t)((n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x);
-  uint32_t landing = 0;   // thread 0: stages with a copy in flight
-  uint32_t phase = 0;     // thread 0: parity of each stage's next completion
-  auto tile_chunk0 = [&](int64_t i) {
-    return (blockIdx.x + (uint64_t)i * gridDim.x) * kTileChunks;
+  const uint32_t tid = threadIdx.x;
+  const int64_t n_tiles = (int64_t)((n_chunks + kDirectTile - 1) / kDirectTile);
+  const bool v8 = (reinterpret_cast<uintptr_t>(x) & 31u) == 0;
+  auto first = [&](int64_t t, int k) {
+    return (uint64_t)t * kDirectTile + 2u * (uint32_t)(k * kThreads + tid);
   };
-  auto issue = [&](int64_t i) {   // thread 0
-    const int s = (int)(i % kStages);
-    const uint64_t c0 = tile_chunk0(i), left = n_chunks - c0;
-    const uint32_t nc = left < (uint64_t)kTileChunks ? (uint32_t)left : (uint32_t)kTileChunks;
-    mbar_arrive_expect_tx(&full[s], nc * 16u);
-    bulk_load(buf + s * kTileChunks, x + c0, nc * 16u, &full[s]);
-    landing |= 1u << s;
-  };
-  // Thread 0 waits for stage s's copy, if one is in flight; all leave together.
-  auto landed = [&](int s) {
-    if (tid == 0 && (landing >> s & 1u)) {
-      const WaitCtl ctl{&abort_flag, err, timeout_ns};
-      if (!mbar_wait(&full[s], phase >> s & 1u, ctl)) {
-        abort_flag = 1;
-      } else {
-        landing &= ~(1u << s);
-        phase ^= 1u << s;
-      }
-    }
-    __syncthreads();
-    return abort_flag == 0;
-  };
-  // After an expired wait: copies in flight land before the CTA exits.
-  auto drain = [&] {
-    if (tid != 0) return;
-    for (int s = 0; s < kStages; ++s) {
-      if (!(landing >> s & 1u)) continue;
-      const uint64_t t0 = global_timer_ns();
-      while (!mbar_try_wait(smem_u32(&full[s]), phase >> s & 1u) &&
-             global_timer_ns() - t0 < timeout_ns) {
-      }
-    }
-  };
-  if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&full[s], 1);
-    abort_flag = 0;
-    mbar_fence_init();
-    for (int64_t i = 0; i < kStages && i < n_own; ++i) issue(i);
-  }
-  uint32_t m = 0;
-  bool ok = true;
-  __syncthreads();
-  for (int64_t i = 0; i < n_own; ++i) {
-    const int s = (int)(i % kStages);
-    if (!landed(s)) {
-      ok = false;
-      break;
-    }
-    const uint64_t c0 = tile_chunk0(i);
+  auto load = [&](int64_t t, uint4 (&v)[kDirectUnits][2]) {
 #pragma unroll
-    for (int u = 0; u < kTileChunks / kThreads; ++u)
-      if (c0 + u * kThreads + tid < n_chunks)
-        m = max(m, chunk_abs_max_bits(lds128(buf + s * kTileChunks + u * kThreads + tid)));
-    if (i + kStages < n_own) {   // the last kStages tiles stay
-      __syncthreads();
-      if (tid == 0) issue(i + kStages);
+    for (int k = 0; k < kDirectUnits; ++k) {
+      const uint64_t c = first(t, k);
+      if (t >= n_tiles || t < 0 || c >= n_chunks) {
+        v[k][0] = v[k][1] = make_uint4(0u, 0u, 0u, 0u);
+      } else if (v8) {
+        ldg256(x + c, v[k]);
+      } else {
+        v[k][0] = ldg128(x + c);
+        v[k][1] = ldg128(x + c + 1);
+      }
     }
+  };
+  uint32_t m = 0;
+  auto amax = [&](const uint4 (&v)[kDirectUnits][2]) {
+#pragma unroll
+    for (int k = 0; k < kDirectUnits; ++k)
+      m = max(m, max(chunk_abs_max_bits(v[k][0]), chunk_abs_max_bits(v[k][1])));
+  };
+  const int64_t g = gridDim.x;
+  uint4 v[kDirectUnits][2], w[kDirectUnits][2];
+  load(blockIdx.x, v);
+  for (int64_t t = blockIdx.x; t < n_tiles; t += 2 * g) {
+    load(t + g, w);
+    amax(v);
+    load(t + 2 * g, v);
+    amax(w);
   }
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31) == 0) warp_max[tid >> 5] = m;
-  __syncthreads();   // every thread has read abort_flag
-  // (a CTA whose wait expired still arrives, so that no other waits for it)
-  const bool met = grid_amax<kThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns);
-  if (!ok || !met) {
-    drain();
-    return;
-  }
-  const float amax = s_amax;
-  const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
+  const int64_t last = (int64_t)blockIdx.x + (n_tiles - 1 - (int64_t)blockIdx.x) / g * g;
+  load(last, v);
+  if (!grid_amax<kThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns)) return;
+  const float am = s_amax;
+  const float s_dec = (am == 0.0f) ? 1.0f : __fdiv_rn(am, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
   op.s_enc = encode_scale(s_dec);
   op.bind(op_table);
   op.init();
   __syncthreads();
-  for (int64_t i = n_own - 1; i >= 0; --i) {
-    const int s = (int)(i % kStages);
-    if (!landed(s)) {
-      drain();
-      return;
-    }
-    const uint64_t c0 = tile_chunk0(i);
-    constexpr int kU = Op::kUnit;
+  auto quantize = [&](int64_t t, const uint4 (&v)[kDirectUnits][2]) {
 #pragma unroll
-    for (int u = 0; u < kTileChunks / (kU * kThreads); ++u) {
-      const int cl = (u * kThreads + tid) * kU;
-      const uint64_t c = c0 + cl;
-      const bool valid = c < n_chunks;
-      uint4 v[kU];
-#pragma unroll
-      for (int k = 0; k < kU; ++k)
-        v[k] = valid ? lds128(buf + s * kTileChunks + cl + k) : make_uint4(0u, 0u, 0u, 0u);
-      op.unit(v, c, valid);
+    for (int k = 0; k < kDirectUnits; ++k) {
+      const uint64_t c = first(t, k);
+      op.pair(v[k], c, c < n_chunks);
     }
-    if (i >= kStages) {
-      __syncthreads();   // every thread is done with this stage
-      if (tid == 0) issue(i - kStages);
-    }
+  };
+  for (int64_t t = last; t >= 0; t -= 2 * g) {
+    load(t - g, w);
+    quantize(t, v);
+    if (t - g < 0) break;
+    load(t - 2 * g, v);
+    quantize(t - g, w);
   }
 }
 
@@ -1064,20 +1033,20 @@ template <typename Op>
 static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                     float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
                                     int num_sms, unsigned* err, uint64_t timeout_ns) {
-  cudaError_t e = set_smem<two_phase_kernel<Op>>();
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   static int resident = -1;   // CTAs one SM can hold
   if (resident < 0) {
     int r = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, two_phase_kernel<Op>, kThreads,
-                                                           kSmem)) != cudaSuccess)
+                                                           0)) != cudaSuccess)
       return e;
     resident = r;
   }
   if (resident < 1) return cudaErrorLaunchOutOfResources;
   if (clear && (e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s)) != cudaSuccess) return e;
-  const int grid = std::min(stream_grid(n_chunks, num_sms), num_sms * resident);
-  return launch_cooperative(two_phase_kernel<Op>, grid, kThreads, kSmem, s,
+  const uint64_t tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
+  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms * std::min(resident, kDirectPerSm));
+  return launch_cooperative(two_phase_kernel<Op>, grid, kThreads, 0, s,
                             static_cast<const uint4*>(x), n_chunks, op, qmax, sdec_out, sync, err,
                             timeout_ns);
 }
