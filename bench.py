@@ -366,9 +366,9 @@ def run_ours(args, dist: Dist):
     # ---- measured tensor-core ceilings (MMA-only probe, every SM at once)
     from paper_2609_21849_gb300 import probe
     ceil = probe.ceilings(sm_max_mhz=float(clk.get("sm_max_mhz") or 2070.0))
-    sms = ceil["nvfp4_pair_256x256x64"]["sms"]
+    sms = ceil["nvfp4_pair_256x256x96"]["sms"]
     mhz = float(clk.get("sm_mhz") or clk.get("sm_max_mhz") or 2070.0)
-    fp4_ceil = ceil["nvfp4_pair_256x256x64"]["flop_per_cycle_per_sm"] * sms * mhz * 1e6 / 1e12
+    fp4_ceil = ceil["nvfp4_pair_256x256x96"]["flop_per_cycle_per_sm"] * sms * mhz * 1e6 / 1e12
     fp8_ceil = ceil["fp8_pair_256x256x32"]["flop_per_cycle_per_sm"] * sms * mhz * 1e6 / 1e12
 
     traffic = committed_traffic()
@@ -398,7 +398,7 @@ def run_ours(args, dist: Dist):
                      "mma_ceiling": round(fp4_ceil, 1),
                      "frac_of_mma_ceiling": round(gemm_tflops / fp4_ceil, 4),
                      "mma_ceiling_source": f"measured kind::mxf4nvf4 CTA-pair MMA rate "
-                                           f"({ceil['nvfp4_pair_256x256x64']['flop_per_cycle_per_sm']:.0f} "
+                                           f"({ceil['nvfp4_pair_256x256x96']['flop_per_cycle_per_sm']:.0f} "
                                            f"FLOP/cycle/SM) x {sms} SMs x {mhz:.0f} MHz (median sampled SM clock)",
                      "traffic": traffic,
                      "algorithmic": f"{STEP_FLOPS / 1e9:.2f} GFLOP per launch; {gemm_s * 1e6:.2f} us avg launch"},

@@ -18,6 +18,8 @@ extern "C" {
  * `iters` back-to-back tcgen05.mma instructions from one thread, with its
  * operands resident in shared memory.
  *   kind  4 = NVFP4 (kind::mxf4nvf4, scale_vec::4X, K = 64 per instruction),
+ *         5 = the same with K = 96 (block16; pair only, n = 256, A in shared
+ *         memory),
  *         8 = FP8 E4M3 (kind::f8f6f4, K = 32), 16 = bf16 (kind::f16, K = 16);
  *         kind + 100: the same with the A operand read from TMEM (written
  *         there first by tcgen05.st) instead of shared memory

@@ -79,7 +79,8 @@ __device__ __forceinline__ void mma_ts(int kind, bool pair, uint32_t d, uint32_t
 }
 
 // kKind: 4 = NVFP4 (mxf4nvf4, K = 64), 8 = FP8 (f8f6f4, K = 32), 16 = bf16
-// (f16, K = 16); every instruction reads 32 bytes of K per operand row.
+// (f16, K = 16): every instruction reads 32 bytes of K per operand row; 5 =
+// NVFP4 with K = 96 (48 bytes; pairs).
 // kATmem: A from TMEM columns [384, 416) (8 columns per instruction).
 template <int kKind, bool kPair, int kN, bool kATmem = false>
 __global__ void __launch_bounds__(kProbeThreads, 1)
@@ -141,13 +142,15 @@ __global__ void __launch_bounds__(kProbeThreads, 1)
   }
   if (threadIdx.x == 0 && rank == 0) {
     constexpr int kM = kPair ? 256 : 128;
-    const uint32_t idesc = kKind == 4 ? idesc_nvfp4(kN, kM)
+    const uint32_t idesc = kKind == 5 ? idesc_nvfp4_k96(kN, kM, 0)
+                           : kKind == 4 ? idesc_nvfp4(kN, kM)
                            : kKind == 8 ? idesc_fp8(kN, kM)
                                         : idesc_bf16(kN, kM);
     const uint32_t a = smem_u32(sA), b = smem_u32(sB), sf = smem_u32(sSF);
     const uint32_t sf_t = tb + 256;   // scale columns: A at +0, B atoms at +4, +8
-    if (kKind == 4) {
-      for (int r = 0; r < 3; ++r) {
+    // K = 96 reads two groups of scales per operand (A at +0, W at +8)
+    if (kKind == 4 || kKind == 5) {
+      for (int r = 0; r < (kKind == 5 ? 6 : 3); ++r) {
         if (kPair)
           tc_cp_scales_pair(sf_t + 4 * r, sdesc_scales(sf + 512 * r));
         else
@@ -168,6 +171,9 @@ __global__ void __launch_bounds__(kProbeThreads, 1)
       const uint32_t acc = i > 0 ? 1u : 0u;
       if (kATmem) {
         mma_ts(kKind, kPair, tb, tb + 384 + (uint32_t)(i & 3) * 8, bd, idesc, sf_t, sf_t + 4, acc);
+      } else if (kKind == 5) {
+        const uint32_t h = (uint32_t)(i & 1) * 48;
+        mma_nvfp4_k96_pair(tb, sdesc_k128(a + h), sdesc_k128(b + h), idesc, sf_t, sf_t + 8, acc);
       } else if (kKind == 4) {
         if (kPair)
           mma_nvfp4_pair(tb, ad, bd, idesc, sf_t, sf_t + 4, acc);
@@ -397,6 +403,7 @@ extern "C" int qlin_probe_mma(int kind, int pair, int n, int ctas, int iters,
   // kind + 100: the same kind with A in TMEM
   const bool a_tmem = kind > 100;
   if (a_tmem) kind -= 100;
+  if (kind == 5 && a_tmem) return 1;
   if (out == nullptr || err == nullptr || iters < 1 || ctas < 1) return 1;
   if (pair && ctas % 2 != 0) return 1;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -409,6 +416,7 @@ extern "C" int qlin_probe_mma(int kind, int pair, int n, int ctas, int iters,
                : launch_probe<K, P, N, false>(ctas, iters, out, err, s); \
   }
   QLIN_PROBE_CASE(4, true, 256);
+  QLIN_PROBE_CASE(5, true, 256);
   QLIN_PROBE_CASE(4, false, 256);
   QLIN_PROBE_CASE(4, false, 128);
   QLIN_PROBE_CASE(8, true, 256);

@@ -864,10 +864,8 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
 // and quantizes its share, so the grid needs neither a grid-wide barrier nor a
 // cooperative launch.  One 16-element block (two chunks) per thread, loaded
 // first and kept in registers.  Bound by latency: launch, one load, one
-// cluster barrier.
-#ifndef QLIN_CLUSTER_MAX_KB
-#define QLIN_CLUSTER_MAX_KB 1024
-#endif
+// cluster barrier (128 x 256: NVFP4 4.46 -> 2.2 us, FP8 3.4 -> 2.0 us against
+// the cooperative routes).
 constexpr int kClusterCtas = 8;
 constexpr int kClusterThreads = 512;
 constexpr uint32_t kClusterSub = 2 * kClusterThreads;   // chunks a CTA quantizes at most
@@ -1051,8 +1049,12 @@ static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& 
                             timeout_ns);
 }
 
-// The cluster route takes x of up to kClusterMaxChunks chunks.
-constexpr uint64_t kClusterMaxChunks = QLIN_CLUSTER_MAX_KB * 64ull;
+// The cluster route takes x of up to 1 MB: there every CTA's eighth of x takes
+// as long to read as the grid barrier it saves (NVFP4, in a graph: 1 MB 3.9 us
+// against 4.7 on the cooperative routes, 2 MB 6.2 against 4.8; FP8: 3.6 against
+// 3.55 and 5.6 against 3.7; a cooperative launch outside a graph costs about
+// 2 us more).
+constexpr uint64_t kClusterMaxChunks = 1024 * 64;
 
 template <typename Op>
 static cudaError_t launch_cluster_quant(const void* x, uint32_t n_chunks, const Op& op,

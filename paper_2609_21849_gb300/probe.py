@@ -26,7 +26,8 @@ from . import build
 _lib = None
 
 # (name, kind, pair, n, K per instruction); kind + 100: A read from TMEM
-CASES = (("nvfp4_pair_256x256x64", 4, 1, 256, 64),
+CASES = (("nvfp4_pair_256x256x96", 5, 1, 256, 96),
+         ("nvfp4_pair_256x256x64", 4, 1, 256, 64),
          ("nvfp4_cta_128x256x64", 4, 0, 256, 64),
          ("nvfp4_cta_128x128x64", 4, 0, 128, 64),
          ("fp8_pair_256x256x32", 8, 1, 256, 32),

@@ -18,6 +18,13 @@ def test_mma_probe_nvfp4_pair():
     assert r["cycles_per_mma"] >= 127.0
 
 
+def test_mma_probe_nvfp4_pair_k96():
+    # K = 96 in the same 128 cycles
+    r = probe.measure(5, 1, 256, 96, iters=2048)
+    assert 32768 < r["flop_per_cycle_per_sm"] <= 49152 * 1.01
+    assert r["cycles_per_mma"] >= 127.0
+
+
 def test_scale_copy_probe():
     alone = probe.scale_copy_cycles(4, 12, 0, iters=200)
     beside = probe.scale_copy_cycles(4, 12, 4, iters=200)
