@@ -158,7 +158,7 @@ qlin_status qlin_quantize_act_nvfp4(const void* x_bf16, int64_t M, int64_t K,
   if (static_scale == nullptr) {
     QLIN_CUDA(launch_quant_nvfp4_dynamic(x_bf16, M, K, *out,
                                          static_cast<unsigned*>(workspace) + kWsQuant, false, s,
-                                         sms, status, timeout()));
+                                         sms, timeout()));
   } else {
     QLIN_CUDA(launch_quant_nvfp4(x_bf16, M, K, static_scale, *out, s, sms));
   }
@@ -185,7 +185,7 @@ qlin_status qlin_quantize_act_nvfp4_noalloc(const void* x_bf16, int64_t M, int64
   // the scratch words are cleared by the launch that uses them
   QLIN_CUDA(launch_quant_nvfp4_dynamic(x_bf16, M, K, *out,
                                        reinterpret_cast<unsigned*>(scratch) + kWsQuant, true, s,
-                                       sms, status, timeout()));
+                                       sms, timeout()));
   return QLIN_OK;
 }
 
@@ -205,7 +205,7 @@ qlin_status qlin_quantize_act_fp8(const void* x_bf16, int64_t M, int64_t K,
   if (static_scale == nullptr) {
     QLIN_CUDA(launch_quant_fp8_dynamic(x_bf16, M, K, *out,
                                        static_cast<unsigned*>(workspace) + kWsQuant, false, s, sms,
-                                       status, timeout()));
+                                       timeout()));
   } else {
     QLIN_CUDA(launch_quant_fp8(x_bf16, M, K, static_scale, *out, s, sms, status, timeout()));
   }

@@ -23,11 +23,11 @@ cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* s
 // (clear = zero them first) and zero again when the kernel ends.
 cudaError_t launch_quant_nvfp4_dynamic(const void* x, int64_t M, int64_t K,
                                        const qlin_nvfp4_t& out, unsigned* sync, bool clear,
-                                       cudaStream_t s, int num_sms, unsigned* err,
+                                       cudaStream_t s, int num_sms,
                                        uint64_t timeout_ns);
 cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
                                      unsigned* sync, bool clear, cudaStream_t s, int num_sms,
-                                     unsigned* err, uint64_t timeout_ns);
+                                     uint64_t timeout_ns);
 cudaError_t launch_quant_fp8_rows(const void* w, int64_t N, int64_t K, const qlin_fp8_t& out,
                                   cudaStream_t s, int num_sms);
 

@@ -6,10 +6,10 @@
 //   cluster_quant_kernel  up to 1 MB: every cluster of eight CTAs reads all of
 //                         x, so no grid-wide barrier
 //   regpass_kernel        (NVFP4) x held in registers: one read of x, the amax
-//                         reduced across a cooperative grid
+//                         reduced across the grid
 //   onepass_kernel        the same with x in shared memory
 //   two_phase_kernel      larger x: amax, then the tiles again in reverse order,
-//                         in one cooperative launch
+//                         in one launch
 // Static tensor scale:
 //   quant_nvfp4_kernel    bf16 -> packed e2m1 codes + E4M3 block scales in the
 //                         tensor-core scale layout + FP32 tensor scale
@@ -554,10 +554,9 @@ __global__ void __launch_bounds__(kThreads, 2)
 // ------------------------------------------------ one-pass dynamic scale ---
 // The tensor scale depends on max |x| over the whole tensor (the amax pass),
 // and the codes depend on the tensor scale, so a streaming quantizer reads x
-// twice.  When x fits in the aggregate shared memory of the grid (one CTA per
-// SM, launched cooperatively so every CTA is resident), each CTA loads its
-// slice once, the grid combines the slice maxima through two words of
-// global memory, and each CTA quantizes its slice from shared memory.
+// twice.  When x fits in the aggregate shared memory (or registers) of the grid,
+// one CTA per SM, each CTA loads its slice once, the grid combines the slice maxima through two words of
+// global memory, and each CTA quantizes its slice from where it holds it.
 constexpr int kOnePassThreads = 1024;
 constexpr int kOnePassSmem = 225 * 1024;
 constexpr int kOnePassSliceMax = 14 * 1024;       // chunks: 224 KB of data at most
@@ -588,20 +587,31 @@ __device__ __forceinline__ void cp_async_wait_pending(int pending) {
   }
 }
 
-// The maximum of the grid's warp maxima into *s_amax (shared memory, for every
-// thread): combine the CTA's, publish, arrive, wait (bounded) for every CTA,
-// depart.  False if the wait expired (recorded in *err).
+// The maximum of the grid's warp maxima (max |x|, as bits) into *s_amax (shared
+// memory, for every thread): combine the CTA's, publish, arrive, wait for every
+// CTA, depart.  The grid is no larger than the machine, so its CTAs are resident
+// together unless other streams' kernels hold SMs for long -- or hold them
+// waiting, as another grid like this one would.  So the wait is bounded, and a
+// CTA whose wait expires reads all of x for the maximum itself: slow, but the
+// same value, and nothing waits without end.  (A cooperative launch, which
+// keeps the grid together, costs about 2 us outside a graph: 2.5 MB of FP8 6.2
+// us instead of 4.5.)
+constexpr uint64_t kGridWaitNs = 1000000;
+
 template <int kThreadsPerBlock>
-__device__ __forceinline__ bool grid_amax(const uint32_t* warp_max, unsigned* sync, float* s_amax,
-                                          int* abort_flag, unsigned* err, uint64_t timeout_ns) {
+__device__ __forceinline__ void grid_amax(const uint4* x, uint64_t n_chunks, uint32_t* warp_max,
+                                          unsigned* sync, float* s_amax, int* alone,
+                                          uint64_t wait_ns) {
   const int tid = threadIdx.x;
-  if (tid == 0) *abort_flag = 0;
-  __syncthreads();
-  if (tid == 0) {
+  __syncthreads();   // warp_max is written
+  auto combine = [&] {
     uint32_t b = 0;
 #pragma unroll
     for (int w = 0; w < kThreadsPerBlock / 32; ++w) b = max(b, warp_max[w]);
-    // publish, arrive, and wait (bounded) for every CTA of the grid
+    return b;
+  };
+  if (tid == 0) {
+    const uint32_t b = combine();
     if (b) atomicMax(&sync[0], b << 16);
     // the arrival releases the maximum above to every CTA that sees it
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&sync[1]) : "memory");
@@ -610,27 +620,34 @@ __device__ __forceinline__ bool grid_amax(const uint32_t* warp_max, unsigned* sy
     // the second round trip to L2 that reading the amax afterwards took.
     const uint64_t t0 = global_timer_ns();
     uint64_t pair = ld_acquire_gpu_pair(&sync[0]);
-    while ((uint32_t)(pair >> 32) < gridDim.x) {
-      if (global_timer_ns() - t0 > timeout_ns) {
-        atomicExch(err, kErrTimeout);
-        *abort_flag = 1;
-        break;
-      }
+    bool expired = false;
+    while ((uint32_t)(pair >> 32) < gridDim.x && !expired) {
+      expired = global_timer_ns() - t0 > wait_ns;
       pair = ld_acquire_gpu_pair(&sync[0]);
     }
+    *alone = (uint32_t)(pair >> 32) < gridDim.x ? 1 : 0;
     *s_amax = __uint_as_float((uint32_t)pair);
   }
   __syncthreads();
   if (tid == 0) {
-    // depart (after a timeout too); the last CTA out resets the words.  The
-    // other warps do not wait for this atomic's round trip.
+    // depart; the last CTA out resets the words.  The other warps do not wait
+    // for this atomic's round trip.
     if (atomicAdd(&sync[2], 1u) == gridDim.x - 1u) {
       sync[0] = 0u;
       sync[1] = 0u;
       sync[2] = 0u;
     }
   }
-  return *abort_flag == 0;
+  if (*alone) {
+    uint32_t m = 0;
+    for (uint64_t c = tid; c < n_chunks; c += kThreadsPerBlock)
+      m = max(m, chunk_abs_max_bits(ldg128(x + c)));
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    if ((tid & 31) == 0) warp_max[tid >> 5] = m;
+    __syncthreads();
+    if (tid == 0) *s_amax = __uint_as_float(combine() << 16);
+    __syncthreads();
+  }
 }
 
 // sync[0]: amax bits (fp32), sync[1]: arrival count, sync[2]: departure
@@ -639,14 +656,13 @@ __device__ __forceinline__ bool grid_amax(const uint32_t* warp_max, unsigned* sy
 template <typename Op>
 __global__ void __launch_bounds__(kOnePassThreads, 1)
     onepass_kernel(const uint4* __restrict__ x, uint64_t n_chunks, uint32_t slice, Op op,
-                   float qmax, float* sdec_out, unsigned* sync, unsigned* err,
-                   uint64_t timeout_ns) {
+                   float qmax, float* sdec_out, unsigned* sync, uint64_t wait_ns) {
   extern __shared__ __align__(128) uint8_t qsm[];
   uint4* buf = reinterpret_cast<uint4*>(qsm);
   __shared__ uint32_t warp_max[kOnePassThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
-  __shared__ int abort_flag;
+  __shared__ int alone;
   grid_dep_wait();
   const int tid = threadIdx.x;
   const uint64_t c_begin = (uint64_t)blockIdx.x * slice;
@@ -702,8 +718,7 @@ __global__ void __launch_bounds__(kOnePassThreads, 1)
   }
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31) == 0) warp_max[tid >> 5] = m;
-  const bool ok = grid_amax<kOnePassThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns);
-  if (!ok) return;
+  grid_amax<kOnePassThreads>(x, n_chunks, warp_max, sync, &s_amax, &alone, wait_ns);
   const float amax = s_amax;
   const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
@@ -732,12 +747,11 @@ constexpr uint32_t kRegSliceMax = kRegUnits * kRegStride;       // 192 KB of x p
 template <typename Op>
 __global__ void __launch_bounds__(kRegThreads, 1)
     regpass_kernel(const uint4* __restrict__ x, uint64_t n_chunks, uint32_t slice, Op op,
-                   float qmax, float* sdec_out, unsigned* sync, unsigned* err,
-                   uint64_t timeout_ns) {
+                   float qmax, float* sdec_out, unsigned* sync, uint64_t wait_ns) {
   __shared__ uint32_t warp_max[kRegThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
-  __shared__ int abort_flag;
+  __shared__ int alone;
   grid_dep_wait();
   const uint32_t tid = threadIdx.x;
   const uint64_t c_begin = (uint64_t)blockIdx.x * slice;
@@ -766,7 +780,7 @@ __global__ void __launch_bounds__(kRegThreads, 1)
   grid_dep_launch();   // x is on chip: the next kernel may begin launching
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31u) == 0u) warp_max[tid >> 5] = m;
-  if (!grid_amax<kRegThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns)) return;
+  grid_amax<kRegThreads>(x, n_chunks, warp_max, sync, &s_amax, &alone, wait_ns);
   const float amax = s_amax;
   const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
@@ -777,8 +791,8 @@ __global__ void __launch_bounds__(kRegThreads, 1)
   op.template run_units<kRegUnits, kRegStride>(v, bm, n, c_begin);
 }
 
-// Dynamic scale of an x that does not fit on chip: one cooperative launch reads
-// x for its amax, meets at the grid barrier and quantizes its tiles in reverse
+// Dynamic scale of an x that does not fit on chip: one launch reads x for its
+// amax, meets at the grid barrier and quantizes its tiles in reverse
 // order, so that it starts on the lines most recently in L2 (the first of them
 // loading while the grid meets).  Loads as in quant_nvfp4_kernel.  Bound by HBM:
 // x once, and what of it L2 has lost a second time.  18432 x 3072: NVFP4 39.8
@@ -788,11 +802,11 @@ __global__ void __launch_bounds__(kRegThreads, 1)
 template <typename Op>
 __global__ void __launch_bounds__(kThreads, kDirectPerSm)
     two_phase_kernel(const uint4* __restrict__ x, uint64_t n_chunks, Op op, float qmax,
-                     float* sdec_out, unsigned* sync, unsigned* err, uint64_t timeout_ns) {
+                     float* sdec_out, unsigned* sync, uint64_t wait_ns) {
   __shared__ uint32_t warp_max[kThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
-  __shared__ int abort_flag;
+  __shared__ int alone;
   l2_prefetch_first_tile(x, n_chunks);
   grid_dep_wait();
   grid_dep_launch();
@@ -835,7 +849,7 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
   if ((tid & 31) == 0) warp_max[tid >> 5] = m;
   const int64_t last = (int64_t)blockIdx.x + (n_tiles - 1 - (int64_t)blockIdx.x) / g * g;
   load(last, v);
-  if (!grid_amax<kThreads>(warp_max, sync, &s_amax, &abort_flag, err, timeout_ns)) return;
+  grid_amax<kThreads>(x, n_chunks, warp_max, sync, &s_amax, &alone, wait_ns);
   const float am = s_amax;
   const float s_dec = (am == 0.0f) ? 1.0f : __fdiv_rn(am, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
@@ -861,11 +875,10 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
 
 // Small x: every cluster of eight CTAs reads all of x (an eighth per CTA, from
 // L2 after the first), combines the maxima through distributed shared memory
-// and quantizes its share, so the grid needs neither a grid-wide barrier nor a
-// cooperative launch.  One 16-element block (two chunks) per thread, loaded
+// and quantizes its share, so the grid needs no grid-wide barrier.  One 16-element block (two chunks) per thread, loaded
 // first and kept in registers.  Bound by latency: launch, one load, one
 // cluster barrier (128 x 256: NVFP4 4.46 -> 2.2 us, FP8 3.4 -> 2.0 us against
-// the cooperative routes).
+// the grid-wide routes).
 constexpr int kClusterCtas = 8;
 constexpr int kClusterThreads = 512;
 constexpr uint32_t kClusterSub = 2 * kClusterThreads;   // chunks a CTA quantizes at most
@@ -959,34 +972,8 @@ int stream_grid(uint64_t n_chunks, int num_sms) {
 
 }  // namespace
 
-// Cooperative launch (all CTAs resident: the grid waits on itself), with
-// programmatic serialization where the driver accepts it alongside, else
-// without.
-template <typename... Params, typename... Args>
-static cudaError_t launch_cooperative(void (*kern)(Params...), int grid, int block, int smem,
-                                      cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeCooperative;
-  at[0].val.cooperative = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3((unsigned)block, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = s;
-  cfg.attrs = at;
-  static std::atomic<bool> pdl_ok{true};
-  cfg.numAttrs = pdl_ok.load(std::memory_order_relaxed) ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
-  if (e != cudaSuccess && cfg.numAttrs == 2) {
-    (void)cudaGetLastError();
-    pdl_ok.store(false, std::memory_order_relaxed);
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, args...);
-  }
-  return e;
-}
+// Limit of the grid-wide wait (the caller's wait limit, if that is shorter).
+static uint64_t grid_wait(uint64_t timeout_ns) { return std::min(timeout_ns, kGridWaitNs); }
 
 // One-pass dynamic quantization when x fits on chip: returns
 // cudaErrorNotSupported (nothing launched) when it does not, or when the
@@ -994,7 +981,7 @@ static cudaError_t launch_cooperative(void (*kern)(Params...), int grid, int blo
 template <typename Op>
 static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                   float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                  int num_sms, unsigned* err, uint64_t timeout_ns) {
+                                  int num_sms, uint64_t timeout_ns) {
   // slices of whole 64-element groups (8 chunks), one per SM
   uint64_t slice = (n_chunks + num_sms - 1) / num_sms;
   slice = (slice + 7) / 8 * 8;
@@ -1022,15 +1009,15 @@ static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op
     const cudaError_t e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
   }
-  return launch_cooperative(kern, grid, threads, smem, s, static_cast<const uint4*>(x), n_chunks,
-                            (uint32_t)slice, op, qmax, sdec_out, sync, err, timeout_ns);
+  return launch_pdl(kern, grid, threads, smem, s, static_cast<const uint4*>(x), n_chunks,
+                    (uint32_t)slice, op, qmax, sdec_out, sync, grid_wait(timeout_ns));
 }
 
-// x of any size: two phases over it in one cooperative launch.
+// x of any size: two phases over it in one launch.
 template <typename Op>
 static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                     float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                    int num_sms, unsigned* err, uint64_t timeout_ns) {
+                                    int num_sms, uint64_t timeout_ns) {
   cudaError_t e;
   static int resident = -1;   // CTAs one SM can hold
   if (resident < 0) {
@@ -1044,16 +1031,14 @@ static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& 
   if (clear && (e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s)) != cudaSuccess) return e;
   const uint64_t tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
   const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms * std::min(resident, kDirectPerSm));
-  return launch_cooperative(two_phase_kernel<Op>, grid, kThreads, 0, s,
-                            static_cast<const uint4*>(x), n_chunks, op, qmax, sdec_out, sync, err,
-                            timeout_ns);
+  return launch_pdl(two_phase_kernel<Op>, grid, kThreads, 0, s, static_cast<const uint4*>(x),
+                    n_chunks, op, qmax, sdec_out, sync, grid_wait(timeout_ns));
 }
 
 // The cluster route takes x of up to 1 MB: there every CTA's eighth of x takes
-// as long to read as the grid barrier it saves (NVFP4, in a graph: 1 MB 3.9 us
-// against 4.7 on the cooperative routes, 2 MB 6.2 against 4.8; FP8: 3.6 against
-// 3.55 and 5.6 against 3.7; a cooperative launch outside a graph costs about
-// 2 us more).
+// as long to read as the grid barrier it saves (NVFP4: 1 MB 3.9 us against 4.7
+// on the grid-wide routes, 2 MB 6.2 against 4.8; FP8: 3.6 against 3.55 and 5.6
+// against 3.7).
 constexpr uint64_t kClusterMaxChunks = 1024 * 64;
 
 template <typename Op>
@@ -1119,33 +1104,33 @@ static Fp8Op fp8_op(const qlin_fp8_t& out) {
 template <typename Op>
 static cudaError_t launch_dynamic(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                   float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                  int num_sms, unsigned* err, uint64_t timeout_ns) {
+                                  int num_sms, uint64_t timeout_ns) {
   if (n_chunks <= kClusterMaxChunks)
     return launch_cluster_quant(x, (uint32_t)n_chunks, op, qmax, sdec_out, s);
   const cudaError_t e = launch_onepass(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms,
-                                       err, timeout_ns);
+                                       timeout_ns);
   if (e != cudaErrorNotSupported) return e;
-  return launch_two_phase(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms, err,
+  return launch_two_phase(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms,
                           timeout_ns);
 }
 
 cudaError_t launch_quant_nvfp4_dynamic(const void* x, int64_t M, int64_t K,
                                        const qlin_nvfp4_t& out, unsigned* sync, bool clear,
-                                       cudaStream_t s, int num_sms, unsigned* err,
+                                       cudaStream_t s, int num_sms,
                                        uint64_t timeout_ns) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
   if (n_chunks < (1ull << 32))   // 32-bit index math is enough
     return launch_dynamic(x, n_chunks, nvfp4_op<uint32_t>(K, out), 2688.0f, out.tensor_scale, sync,
-                          clear, s, num_sms, err, timeout_ns);
+                          clear, s, num_sms, timeout_ns);
   return launch_two_phase(x, n_chunks, nvfp4_op<uint64_t>(K, out), 2688.0f, out.tensor_scale, sync,
-                          clear, s, num_sms, err, timeout_ns);
+                          clear, s, num_sms, timeout_ns);
 }
 
 cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
                                      unsigned* sync, bool clear, cudaStream_t s, int num_sms,
-                                     unsigned* err, uint64_t timeout_ns) {
+                                     uint64_t timeout_ns) {
   return launch_dynamic(x, (uint64_t)M * (uint64_t)K / 8, fp8_op(out), 448.0f, out.scale, sync,
-                        clear, s, num_sms, err, timeout_ns);
+                        clear, s, num_sms, timeout_ns);
 }
 
 cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float* scale_src,

@@ -47,6 +47,30 @@ def test_dynamic_routes_match_oracle(M, K):
     assert int(ws.count_nonzero()) == 0
 
 
+@pytest.mark.parametrize("M,K", [(1025, 512), (4608, 3072), (12288 * SMS // 512 + 64, 4096),
+                                 (9217, 4096)])
+def test_grid_wait_that_expires_gives_the_same_codes(M, K):
+    # with the shortest wait limit, CTAs that miss the others' arrival read all
+    # of x for the maximum themselves: same codes, no error, scratch left zero
+    bits = synthetic.act_entry_outliers(7, M, K)
+    x, ws = to_dev(bits), qlin.alloc_workspace()
+    want4 = qlin.qlin_quantize_act_nvfp4(x, None, None, ws)
+    want8 = qlin.qlin_quantize_act_fp8(x, None, None, ws)
+    assert qlin.qlin_sync_status() == 0
+    qlin.qlin_set_wait_timeout_ns(1000)
+    try:
+        q4 = qlin.qlin_quantize_act_nvfp4(x, None, None, ws)
+        q8 = qlin.qlin_quantize_act_fp8(x, None, None, ws)
+        assert qlin.qlin_sync_status() == 0
+    finally:
+        qlin.qlin_set_wait_timeout_ns(2000000000)
+    assert_nvfp4_equal(q4, oracle.quant_nvfp4(bits), f"{M}x{K}")
+    for a, b in ((q4.codes, want4.codes), (q4.tensor_scale, want4.tensor_scale),
+                 (q8.codes, want8.codes), (q8.scale, want8.scale)):
+        assert torch.equal(a, b)
+    assert int(ws.count_nonzero()) == 0
+
+
 @pytest.mark.parametrize("shift", [0, 8])
 def test_static_nvfp4_alignment_and_partial_tile(shift):
     # x 32-byte aligned (one 32-byte load per block) and only 16-byte aligned
