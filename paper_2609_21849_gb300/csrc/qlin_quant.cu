@@ -792,17 +792,22 @@ __global__ void __launch_bounds__(kRegThreads, 1)
 }
 
 // Dynamic scale of an x that does not fit on chip: one launch reads x for its
-// amax, meets at the grid barrier and quantizes its tiles in reverse
-// order, so that it starts on the lines most recently in L2 (the first of them
-// loading while the grid meets).  Loads as in quant_nvfp4_kernel.  Bound by HBM:
-// x once, and what of it L2 has lost a second time.  18432 x 3072: NVFP4 39.8
-// us, FP8 39.3 us; an amax kernel and the quantizer after it took 48.1 and 50.1
-// us, one launch through the shared-memory ring (its last tiles kept) 44.7 and
-// 40.0 us.
+// amax, meets at the grid barrier and quantizes its tiles in reverse order: the
+// last three of every CTA (29 MB in all) wait in shared memory, and the ones
+// before them are the lines most recently in L2.  Loads as in
+// quant_nvfp4_kernel.  Bound by HBM and latency: 18432 x 3072 reads its 113 MB in
+// 19 us (of 165 MB read in all: L2 keeps ~30 MB of them) and quantizes in 20.
+// NVFP4 39.3 us, FP8 38.2 us; without the tiles kept 39.5 and 39.3; an amax
+// kernel and the quantizer after it took 48.1 and 50.1.
+constexpr int kKeep = 3;                                             // tiles of 32 KB per CTA
+constexpr int kKeepSmem = kKeep * (int)kDirectTile * 16;
+
 template <typename Op>
 __global__ void __launch_bounds__(kThreads, kDirectPerSm)
     two_phase_kernel(const uint4* __restrict__ x, uint64_t n_chunks, Op op, float qmax,
                      float* sdec_out, unsigned* sync, uint64_t wait_ns) {
+  extern __shared__ __align__(128) uint8_t qsm[];
+  uint4* const keep = reinterpret_cast<uint4*>(qsm);
   __shared__ uint32_t warp_max[kThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
@@ -836,19 +841,42 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
     for (int k = 0; k < kDirectUnits; ++k)
       m = max(m, max(chunk_abs_max_bits(v[k][0]), chunk_abs_max_bits(v[k][1])));
   };
+  // The CTA's last kKeep tiles also stay in shared memory (each thread keeps and
+  // reads back its own units; 16-byte accesses side by side).
+  auto slot = [&](int r, int k, int h) {
+    return keep + ((r * kDirectUnits + k) * 2 + h) * kThreads + tid;
+  };
   const int64_t g = gridDim.x;
-  uint4 v[kDirectUnits][2], w[kDirectUnits][2];
-  load(blockIdx.x, v);
-  for (int64_t t = blockIdx.x; t < n_tiles; t += 2 * g) {
-    load(t + g, w);
+  const int64_t own = (n_tiles - (int64_t)blockIdx.x + g - 1) / g;   // tiles of this CTA
+  const int64_t kept = own - kKeep;                                  // the first one kept
+  auto tile = [&](int64_t i) { return (int64_t)blockIdx.x + i * g; };
+  auto take = [&](int64_t i, const uint4 (&v)[kDirectUnits][2]) {
     amax(v);
-    load(t + 2 * g, v);
-    amax(w);
+    if (i < kept) return;
+#pragma unroll
+    for (int k = 0; k < kDirectUnits; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) *slot((int)(i - kept), k, h) = v[k][h];
+  };
+  uint4 v[kDirectUnits][2], w[kDirectUnits][2];
+  {
+    uint4 u[kDirectUnits][2];   // two tiles in flight beside the one taken
+    load(tile(0), v);
+    load(tile(1), w);
+    for (int64_t i = 0; i < own; i += 3) {
+      load(tile(i + 2), u);
+      take(i, v);
+      if (i + 1 >= own) break;
+      load(tile(i + 3), v);
+      take(i + 1, w);
+      if (i + 2 >= own) break;
+      load(tile(i + 4), w);
+      take(i + 2, u);
+    }
   }
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31) == 0) warp_max[tid >> 5] = m;
-  const int64_t last = (int64_t)blockIdx.x + (n_tiles - 1 - (int64_t)blockIdx.x) / g * g;
-  load(last, v);
+  load(kept > 0 ? tile(kept - 1) : -1, v);   // the first tile not kept, while the grid meets
   grid_amax<kThreads>(x, n_chunks, warp_max, sync, &s_amax, &alone, wait_ns);
   const float am = s_amax;
   const float s_dec = (am == 0.0f) ? 1.0f : __fdiv_rn(am, qmax);
@@ -864,12 +892,19 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
       op.pair(v[k], c, c < n_chunks);
     }
   };
-  for (int64_t t = last; t >= 0; t -= 2 * g) {
-    load(t - g, w);
-    quantize(t, v);
-    if (t - g < 0) break;
-    load(t - 2 * g, v);
-    quantize(t - g, w);
+  for (int64_t i = own - 1; i >= 0 && i >= kept; --i) {
+#pragma unroll
+    for (int k = 0; k < kDirectUnits; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) w[k][h] = *slot((int)(i - kept), k, h);
+    quantize(tile(i), w);
+  }
+  for (int64_t i = kept - 1; i >= 0; i -= 2) {
+    load(i >= 1 ? tile(i - 1) : -1, w);
+    quantize(tile(i), v);
+    if (i < 1) break;
+    load(i >= 2 ? tile(i - 2) : -1, v);
+    quantize(tile(i - 1), w);
   }
 }
 
@@ -1018,12 +1053,15 @@ template <typename Op>
 static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                     float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
                                     int num_sms, uint64_t timeout_ns) {
-  cudaError_t e;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      two_phase_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKeepSmem);
+  cudaError_t e = attr;
+  if (e != cudaSuccess) return e;
   static int resident = -1;   // CTAs one SM can hold
   if (resident < 0) {
     int r = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, two_phase_kernel<Op>, kThreads,
-                                                           0)) != cudaSuccess)
+                                                           kKeepSmem)) != cudaSuccess)
       return e;
     resident = r;
   }
@@ -1031,7 +1069,7 @@ static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& 
   if (clear && (e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s)) != cudaSuccess) return e;
   const uint64_t tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
   const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms * std::min(resident, kDirectPerSm));
-  return launch_pdl(two_phase_kernel<Op>, grid, kThreads, 0, s, static_cast<const uint4*>(x),
+  return launch_pdl(two_phase_kernel<Op>, grid, kThreads, kKeepSmem, s, static_cast<const uint4*>(x),
                     n_chunks, op, qmax, sdec_out, sync, grid_wait(timeout_ns));
 }
 
