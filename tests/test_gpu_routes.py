@@ -47,6 +47,25 @@ def test_dynamic_routes_match_oracle(M, K):
     assert int(ws.count_nonzero()) == 0
 
 
+@pytest.mark.parametrize("bits", [0x0001, 0x8001, 0x007F, 0x8080, 0x7F7F, 0xFF7F, 0x7F80, 0xFF80,
+                                  0x7FC0, 0xFF81, 0x7FFF])
+@pytest.mark.parametrize("M,K", [(3, 64), (1000, 3072), (9217, 4096)])
+def test_maximum_of_extreme_values(M, K, bits):
+    # one subnormal, largest finite value, infinity or NaN among zeros, at an
+    # odd element: scale = max |x| / 448 in fp32, NaN if x holds one
+    x = torch.zeros((M, K), dtype=torch.int16, device="cuda")
+    x[M - 1, K - 13] = bits - 65536 if bits > 32767 else bits
+    ws = qlin.alloc_workspace()
+    q = qlin.qlin_quantize_act_fp8(x.view(torch.bfloat16), None, None, ws)
+    assert qlin.qlin_sync_status() == 0
+    amax = np.array([(bits & 0x7FFF) << 16], np.uint32).view(np.float32)
+    assert np.array_equal(f32(q.scale), amax / np.float32(448), equal_nan=True)
+    q4 = qlin.qlin_quantize_act_nvfp4(x.view(torch.bfloat16), None, None, ws)
+    assert qlin.qlin_sync_status() == 0
+    assert np.array_equal(f32(q4.tensor_scale), amax / np.float32(2688), equal_nan=True)
+    assert int(ws.count_nonzero()) == 0
+
+
 @pytest.mark.parametrize("M,K", [(1025, 512), (4608, 3072), (12288 * SMS // 512 + 64, 4096),
                                  (9217, 4096)])
 def test_grid_wait_that_expires_gives_the_same_codes(M, K):
