@@ -458,7 +458,7 @@ def measure_headline_rows(torch, qlin, synthetic, stream, pk, fp4_peak, fp8_peak
     # ---- NVFP4 / FP8 activation quantizers: x [4608, 3072] (config 3's
     # activations) and [18432, 3072] (the stack input at B = 4, 113 MB: the
     # steady-state bandwidth check)
-    quant = {"kernel": "quant_nvfp4_kernel<static> (and onepass / two-pass dynamic routes)",
+    quant = {"kernel": "quant_nvfp4_kernel (static scale); regpass_kernel / two_phase_kernel (dynamic scale)",
              "peak_GB/s": hbm, "peak_source": f"{pk['source']} HBM copy bandwidth"}
     for (Mq, tag) in ((M, "4608x3072"), (4 * M, "18432x3072")):
         x_bits = synthetic.act_entry_outliers(2, Mq, K)
@@ -476,7 +476,7 @@ def measure_headline_rows(torch, qlin, synthetic, stream, pk, fp4_peak, fp8_peak
         t = g_time(torch, stream, lambda: (lambda r: qlin.qlin_quantize_act_nvfp4(xs[r], None, qs[r], wsp[r]))(nxt(R)), R)
         row["nvfp4_dynamic"] = {
             "us": round(t * 1e6, 2),
-            "route": "one read of x (x held on chip)" if Mq * K * 2 <= 152 * 224 * 1024 else "amax pass + quantizer",
+            "route": "one read of x (x held on chip)" if Mq * K * 2 <= 152 * 224 * 1024 else "two phases over x in one launch",
             "GB/s_moved": round((2.5625 if Mq * K * 2 <= 152 * 224 * 1024 else 4.5625) * elems / t / 1e9, 1),
             "GB/s_at_4.5625": round(4.5625 * elems / t / 1e9, 1),
             "frac_hbm_moved": round((2.5625 if Mq * K * 2 <= 152 * 224 * 1024 else 4.5625) * elems / t / 1e9 / hbm, 3)}

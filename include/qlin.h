@@ -102,8 +102,8 @@ typedef struct {
  * ceil(rows / 128) * (K / 64) * 512.  Returns 0 for invalid shapes. */
 size_t qlin_nvfp4_scale_bytes(int64_t rows, int64_t K);
 
-/* Workspace bytes the dynamic-scale quantizers need (a device amax word);
- * the same for every shape.  Returns 256. */
+/* Workspace bytes the dynamic-scale quantizers need (the grid-wide
+ * maximum and arrival counts); the same for every shape.  Returns 256. */
 size_t qlin_workspace_size(int64_t M, int64_t K);
 
 /*
@@ -112,8 +112,8 @@ size_t qlin_workspace_size(int64_t M, int64_t K);
  *  x:            bf16 [M, K], 16-byte aligned.
  *  static_scale: device fp32 S_dec from calibration (post-training
  *                quantization, Sec. 4); NULL selects the dynamic tensor
- *                scale S_dec = amax(|x|) / (6 * 448) (1 if amax == 0), which
- *                first runs an amax pass over x.
+ *                scale S_dec = amax(|x|) / (6 * 448) (1 if amax == 0), found
+ *                in the same launch.
  *  out:          rows == M, K == K; codes, scales and tensor_scale are written
  *                (tensor_scale receives S_dec in both modes).
  *  workspace:    device memory of >= qlin_workspace_size() bytes, 8-byte
@@ -205,7 +205,7 @@ qlin_status qlin_linear_fused(const qlin_nvfp4_t *A, const qlin_nvfp4_t *W,
  * integration aid.  Some callers own no allocator of their own -- a plugin
  * running inside an inference runtime that hands out all device memory, or a
  * real-time loop that must never stall on cudaMalloc.  They can still pass x
- * and the output buffers, but not the workspace the dynamic amax pass needs.
+ * and the output buffers, but not the workspace the dynamic scale needs.
  *
  * This entry point takes no workspace: its scratch (the amax and arrival
  * words) lives in a static device array of QLIN_NOALLOC_SCRATCH_BYTES bytes
@@ -308,7 +308,10 @@ qlin_status qlin_sync_status(void *stream);
  */
 qlin_status qlin_selftest_bounded_wait(uint64_t timeout_ns, void *stream);
 
-/* Wait limit used by every device-side spin (default 2 s), in ns. */
+/* Wait limit used by every device-side spin (default 2 s), in ns.  The dynamic
+ * quantizers wait at most 1 ms of it for the rest of their grid; a CTA whose
+ * wait expires there reads all of x for the maximum itself: no error, the same
+ * result. */
 void qlin_set_wait_timeout_ns(uint64_t ns);
 
 /* Short text for a status code (static storage). */

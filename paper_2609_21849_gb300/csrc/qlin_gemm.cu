@@ -45,9 +45,6 @@ namespace {
 constexpr int kBM = 128;
 constexpr int kRowBytes = 128;      // bytes of K per stage and row: one swizzle row
 constexpr int kStepsPerStage = 4;   // one MMA per 32 bytes of K
-// Build-time layout choices (the defaults measured fastest): scale-copy warps
-// of NVFP4 pair tiles, a warp of its own for their scale boxes, and row boxes
-// per operand tile and stage.
 // Tile order: cluster tiles are visited in groups of this many M tile groups
 // (0: all of M, i.e. M fastest within each N tile; on the 4608 x 12288 x 3072
 // NVFP4 GEMM groups of 1 to 9 measured 3-6% slower)

@@ -19,10 +19,11 @@
 //
 // The [M, K] input is a flat array of 16-byte chunks (8 bf16); a unit is the
 // two chunks of one NVFP4 block, and four neighbouring lanes hold one
-// 64-element group (because K % 64 == 0 a group never straddles a row).  The
-// kernels that stream (stream_tiles, two_phase_kernel) cut it into 16 KB tiles
-// that a persistent grid (three CTAs per SM) takes through a four-deep
-// shared-memory ring filled by bulk copies, ~192 KB per SM of input in flight.
+// 64-element group (because K % 64 == 0 a group never straddles a row).
+// quant_nvfp4_kernel and two_phase_kernel load straight to registers; the static
+// FP8 quantizer (stream_tiles) cuts x into 16 KB tiles that a persistent grid
+// (three CTAs per SM) takes through a four-deep shared-memory ring filled by
+// bulk copies, ~192 KB per SM of input in flight.
 #include <atomic>
 
 #include "qlin_internal.h"
@@ -392,13 +393,14 @@ __device__ __forceinline__ bool stream_tiles(const uint4* __restrict__ x, uint64
   return ok;
 }
 
-// The CTA's first tile into L2 (one bulk prefetch from thread 0), issued
-// before grid_dep_wait: a prefetch is a hint that returns no data, so it is
-// correct even while the previous kernel still writes x, and the tile's DRAM
-// read overlaps that kernel's tail.  NVFP4 4608 x 3072 static, measured:
-// 9.1 -> 8.0 us in a chain of launches, 9.3 -> 8.3 us right after a fused
-// GEMM, unchanged (15.0 us) alone after an L2 flush.  Prefetching all four
-// ring tiles gained 0.1-0.8 us more in chains but cost 1.1 us alone.
+// The first 16 KB per CTA of x into L2 (one bulk prefetch from thread 0 of
+// each), issued before grid_dep_wait: a prefetch is a hint that returns no
+// data, so it is correct even while the previous kernel still writes x, and the
+// DRAM reads overlap that kernel's tail.  (Static NVFP4 through the ring,
+// 4608 x 3072: 9.1 -> 8.0 us in a chain of launches, 9.3 -> 8.3 us right after a
+// fused GEMM, unchanged alone after an L2 flush.  The kernels that load straight
+// to registers have 32 KB tiles; prefetching those whole measured 7.5 -> 7.8 us
+// there, 38.9 -> 38.6 in two_phase_kernel at 18432 x 3072.)
 __device__ __forceinline__ void l2_prefetch_first_tile(const uint4* x, uint64_t n_chunks) {
   if (threadIdx.x == 0 && (uint64_t)blockIdx.x * kTileChunks < n_chunks) {
     const uint64_t c0 = (uint64_t)blockIdx.x * kTileChunks;
@@ -421,8 +423,8 @@ __device__ __forceinline__ float static_scale(const float* scale_src, float* sde
 // 64 KB per SM of loads in flight.  Bound by HBM: 18432 x 3072 in 22.4 us
 // (6.5 TB/s), through the shared-memory ring of the other streaming kernels
 // 24.1 us (its block reads have two-way bank conflicts); 4608 x 3072 7.5 us,
-// was 7.7.  256-thread CTAs with one to three units measured 22.3-23.6 us and
-// 7.7-8.6 us.
+// through the ring 7.8.  256-thread CTAs with one to three units
+// measured 22.3-23.6 us and 7.7-8.6 us.
 constexpr int kDirectPerSm = 2;
 constexpr int kDirectUnits = 2;                                       // per thread and tile
 constexpr uint32_t kDirectTile = 2u * kThreads * kDirectUnits;        // chunks: 32 KB
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
 }
 
 // FP8 weights, one scale per row: one warp per row, held in registers up to
-// K = 3072 (12288 x 3072: 21.3 -> 19.1 us), else two passes over it (the second
+// K = 3072 (12288 x 3072: 21.3 -> 18.6 us), else two passes over it (the second
 // hits L1/L2).  Offline, once per layer.
 constexpr int kRowRegs = 12;   // chunks per lane
 
@@ -568,11 +570,12 @@ __global__ void __launch_bounds__(kThreads, 2)
 }
 
 // ------------------------------------------------ one-pass dynamic scale ---
-// The tensor scale depends on max |x| over the whole tensor (the amax pass),
-// and the codes depend on the tensor scale, so a streaming quantizer reads x
-// twice.  When x fits in the aggregate shared memory (or registers) of the grid,
-// one CTA per SM, each CTA loads its slice once, the grid combines the slice maxima through two words of
-// global memory, and each CTA quantizes its slice from where it holds it.
+// The tensor scale depends on max |x| over the whole tensor, and the codes
+// depend on the tensor scale, so a streaming quantizer reads x twice.  When x
+// fits in the aggregate shared memory (or registers) of the grid, one CTA per
+// SM, each CTA loads its slice once, the grid combines the slice maxima through
+// two words of global memory, and each CTA quantizes its slice from where it
+// holds it.
 constexpr int kOnePassThreads = 1024;
 constexpr int kOnePassSmem = 225 * 1024;
 constexpr int kOnePassSliceMax = 14 * 1024;       // chunks: 224 KB of data at most
@@ -752,9 +755,10 @@ __global__ void __launch_bounds__(kOnePassThreads, 1)
 // units, one block each, per thread): no trip through shared memory, whose
 // 32-byte-strided reads (each block twice, with two-way bank conflicts) made up
 // 6500 of the 21 000 cycles of the shared-memory kernel.  4608 x 3072: 12.2 ->
-// 11.45 us, 1000 x 3072: 5.45 -> 5.3 us.  (FP8 in this form: 11.1 -> 10.9 us,
+// 11.2 us, 1000 x 3072: 5.45 -> 5.1 us.  (FP8 in this form: 11.1 -> 10.9 us,
 // but 3.9 -> 4.6 us at 2.5 MB, so it keeps the shared-memory kernel.)  Reading
-// x from HBM takes ~6 us of it, the grid barrier ~1.3 us.
+// x from HBM takes ~6 us of it, the grid barrier ~1.3 us.  (32-byte loads:
+// 1000 x 3072 5.1 -> 4.95 us, but 4608 x 3072 11.2 -> 11.4.)
 constexpr int kRegThreads = 512;
 constexpr int kRegUnits = 12;
 constexpr uint32_t kRegStride = 2u * kRegThreads;               // chunks between a thread's units
@@ -813,8 +817,9 @@ __global__ void __launch_bounds__(kRegThreads, 1)
 // before them are the lines most recently in L2.  Loads as in
 // quant_nvfp4_kernel.  Bound by HBM and latency: 18432 x 3072 reads its 113 MB in
 // 19 us (of 165 MB read in all: L2 keeps ~30 MB of them) and quantizes in 20.
-// NVFP4 39.3 us, FP8 38.2 us; without the tiles kept 39.5 and 39.3; an amax
-// kernel and the quantizer after it took 48.1 and 50.1.
+// NVFP4 39.0 us, FP8 38.1 us (6000 x 3072: 14.7 and 13.2); without the tiles
+// kept 39.2 and 39.3 (15.1 and 14.2); an amax kernel and the quantizer after it
+// took 48.1 and 50.1.
 constexpr int kKeep = 3;                                             // tiles of 32 KB per CTA
 constexpr int kKeepSmem = kKeep * (int)kDirectTile * 16;
 
@@ -926,9 +931,9 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
 
 // Small x: every cluster of eight CTAs reads all of x (an eighth per CTA, from
 // L2 after the first), combines the maxima through distributed shared memory
-// and quantizes its share, so the grid needs no grid-wide barrier.  One 16-element block (two chunks) per thread, loaded
-// first and kept in registers.  Bound by latency: launch, one load, one
-// cluster barrier (128 x 256: NVFP4 4.46 -> 2.2 us, FP8 3.4 -> 2.0 us against
+// and quantizes its share, so the grid needs no grid-wide barrier.  One
+// 16-element block (two chunks) per thread, loaded first and kept in registers.
+// Bound by latency: launch, one load, one cluster barrier (128 x 256: NVFP4 4.46 -> 2.2 us, FP8 3.4 -> 2.0 us against
 // the grid-wide routes).
 constexpr int kClusterCtas = 8;
 constexpr int kClusterThreads = 512;
