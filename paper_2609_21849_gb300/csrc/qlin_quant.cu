@@ -43,7 +43,8 @@ constexpr int kBlocksPerSm = 3;
 // Packed bf16 absolute maxima, one reduction of the two halves per block; with
 // masks and integer maxima of halves dynamic NVFP4 took 5.31 us (now 5.13) at
 // 1000 x 3072, 11.4 (11.2) at 4608 x 3072 and 39.4 (39.0) at 18432 x 3072; the
-// static kernels measured the same.
+// static kernels measured the same.  (Not so in the GEMM's re-quantizing
+// epilogue, which keeps the integer form: there these take 59.5 us to 61.7.)
 __device__ __forceinline__ uint32_t abs_max2(uint32_t a, uint32_t b) {
   uint32_t r;
   asm("{\n\t.reg .b32 x, y;\n\tabs.bf16x2 x, %1;\n\tabs.bf16x2 y, %2;\n\t"
