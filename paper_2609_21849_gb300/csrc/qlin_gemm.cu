@@ -303,12 +303,16 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   // The first W boxes into L2 while the previous kernel still runs: a prefetch
   // is a hint that returns no data, so it is correct even if that kernel
   // writes W.  (4608 x 3072 x 3072 NVFP4 in a chain of launches: 19.2 -> 18.7 us.)
+  // One cluster per W tile does it: the clusters of an N tile share its W, and
+  // where all of them prefetched, a tall narrow GEMM asked L2 for the same lines
+  // a hundred times over (18432 x 64 x 3072 NVFP4: 12.4 us, now 9.0).
   if (warp == 0 && elect_one()) {
     int mg, nb;
     tile_coords(cid, groups_m, tiles_n, &mg, &nb);
     constexpr int kWRows = kBN / kCM / C::kSplit;
     const int w_row = nb * kBN + rank * (kBN / kCM);
-    for (int kb = 0; kb < min(num_kb, C::kStages); ++kb)
+    const int boxes = mg == 0 ? min(num_kb, C::kStages) : 0;
+    for (int kb = 0; kb < boxes; ++kb)
 #pragma unroll
       for (int b = 0; b < C::kSplit; ++b)
         l2_prefetch_4d(&tmap_b, kb * kRowBytes, w_row + b * kWRows);

@@ -119,10 +119,12 @@ def _rows(M):
     return np.array(sorted(i for i in r if i < M))
 
 
-# (M, N): 64-wide, 128-wide and pair tiles (with a partial pair); K: one
+# (M, N): 64-wide, 128-wide and pair tiles (with a partial pair), and a single
+# N tile whose W every CTA shares; K: one
 # partial stage, full ones, every remainder of a stage, and K long enough that
 # every ring wraps
-@pytest.mark.parametrize("M,N", [(40, 192), (300, 2560), (3000, 1024), (4700, 2112)])
+@pytest.mark.parametrize("M,N", [(40, 192), (300, 2560), (3000, 1024), (4700, 2112),
+                                 (18400, 64)])
 @pytest.mark.parametrize("K", [64, 192, 256, 832, 2688])
 @pytest.mark.parametrize("fmt", ["nvfp4", "fp8"])
 def test_gemm_tiles_and_stages(fmt, M, N, K):
