@@ -37,13 +37,14 @@
 #include <mutex>
 
 #include "qlin_internal.h"
+#include "qlin_tiles.h"
 
 namespace qlin {
 
 namespace {
 
-constexpr int kBM = 128;
-constexpr int kRowBytes = 128;      // bytes of K per stage and row: one swizzle row
+constexpr int kBM = kTileM;
+constexpr int kRowBytes = kStageRowBytes;   // bytes of K per stage and row: one swizzle row
 constexpr int kStepsPerStage = 4;   // one MMA per 32 bytes of K
 // Tile order: cluster tiles are visited in groups of this many M tile groups
 // (0: all of M, i.e. M fastest within each N tile; on the 4608 x 12288 x 3072
@@ -1206,55 +1207,19 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned*
   return cudaLaunchKernelEx(&cfg, kern, ta, tb, tsa, tsb, ty, p);
 }
 
-// Time of a launch in a tile configuration, in microseconds: a launch, then
-// waves of tiles that each cost a start and end and their K stages.  Fitted
-// to graph-replayed launches over M 16-4608, N 256-6144, K 256-3072 (operands
-// in L2; rms error 5-9%).
-struct TileCost {
-  double launch, wave, stage;
-  double us(int64_t tiles, int64_t slots, int64_t stages) const {
-    return launch + (double)((tiles + slots - 1) / slots) * (wave + (double)stages * stage);
-  }
-};
-
-enum class Tile { kPair, kSingle, kNarrow };
-
-// Pair tiles when there are enough of them to fill the machine, else 128 x 128
-// single-CTA tiles, or 128 x 64 when those would leave at least half the SMs
-// idle -- unless the fitted times say that another configuration is at least 10%
-// faster: mostly a last wave that is nearly empty (NVFP4 3000 x 1024 x 3072:
-// 192 single tiles on 152 SMs 10.2 us, 48 pair tiles 7.6 us) or a K too short
-// for the pair tiles' start and end (3000 x 3072 x 256: pairs 6.8 us, single
-// tiles 5.6 us).  The margin covers the fit's error.
-Tile choose_tile(const GemmArgs& a, int num_sms, bool narrow_ok) {
-  static const TileCost kCosts[3][3] = {
-      {{2.5, 1.65, 0.24}, {2.7, 0.5, 0.29}, {2.7, 0.3, 0.26}},     // NVFP4
-      {{3.3, 2.2, 0.265}, {2.7, 1.1, 0.205}, {2.8, 0.5, 0.175}},   // FP8
-      {{3.0, 1.1, 0.275}, {2.6, 0.6, 0.18}, {2.6, 0.6, 0.18}}};    // bf16 / fp16
-  const TileCost* cost = kCosts[a.fp4 ? 0 : a.bf16 ? 2 : 1];
-  const int64_t k_bytes = a.fp4 ? a.K / 2 : a.bf16 ? a.K * 2 : a.K;
-  const int64_t stages = (k_bytes + kRowBytes - 1) / kRowBytes;
-  const int64_t tiles_m = (a.M + kBM - 1) / kBM;
-  const int64_t n128 = (a.N + 127) / 128, n256 = (a.N + 255) / 256;
-  double us[3] = {cost[0].us((tiles_m + 1) / 2 * n256, num_sms / 2, stages),
-                  cost[1].us(tiles_m * n128, num_sms, stages),
-                  cost[2].us(tiles_m * ((a.N + 63) / 64), num_sms, stages)};
-  // a pair tile's re-quantizing epilogue ends about this much later
-  if (a.next_scale != nullptr) us[0] += a.fp4 ? 1.0 : 0.6;
-  int pick = tiles_m * n256 >= num_sms ? 0 : narrow_ok && 2 * tiles_m * n128 <= num_sms ? 2 : 1;
-  int best = pick;
-  for (int t = 0; t < (narrow_ok ? 3 : 2); ++t)
-    if (us[t] < us[best]) best = t;
-  if (us[best] < 0.9 * us[pick]) pick = best;
-  return static_cast<Tile>(pick);
+Tile tile_of(const GemmArgs& a, int num_sms) {
+  return choose_tile(a.fp4 ? GemmKind::kNvfp4 : a.bf16 ? GemmKind::k16 : GemmKind::kFp8,
+                     a.next_scale != nullptr ? Epilogue::kRequant
+                     : a.y_amax != nullptr   ? Epilogue::kAmax
+                                             : Epilogue::kPlain,
+                     a.M, a.N, a.K, num_sms);
 }
 
 template <bool kFp4>
 cudaError_t dispatch_bn(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned* err,
                         uint64_t timeout_ns) {
-  // (the fused re-quantization's 64-column groups need 128-column tiles)
   const bool requant = a.next_scale != nullptr;
-  switch (choose_tile(a, num_sms, !requant)) {
+  switch (tile_of(a, num_sms)) {
     case Tile::kPair:
       return requant ? launch_cfg<kFp4, 256, true, true>(a, s, num_sms, err, timeout_ns)
                      : launch_cfg<kFp4, 256, true, false>(a, s, num_sms, err, timeout_ns);
@@ -1300,7 +1265,7 @@ CUresult encode_tensor_map_out_bf16(CUtensorMap* map, void* base, uint64_t cols,
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned* err,
                         uint64_t timeout_ns) {
   if (a.bf16) {
-    return choose_tile(a, num_sms, false) == Tile::kPair
+    return tile_of(a, num_sms) == Tile::kPair
                ? launch_cfg<false, 256, true, false, true>(a, s, num_sms, err, timeout_ns)
                : launch_cfg<false, 128, false, false, true>(a, s, num_sms, err, timeout_ns);
   }
