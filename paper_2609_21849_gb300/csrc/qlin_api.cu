@@ -380,7 +380,8 @@ qlin_status qlin_linear_dynamic(const qlin_nvfp4_t* A, const qlin_nvfp4_t* W, vo
   unsigned* status;
   int sms;
   QLIN_TRY(device_state(&status, &sms));
-  QLIN_CUDA(launch_quant_nvfp4(y_bf16, A->rows, W->rows, y_q->tensor_scale, *y_q, s, sms));
+  QLIN_CUDA(launch_quant_nvfp4_after(y_bf16, A->rows, W->rows, y_q->tensor_scale, *y_q, s, sms,
+                                     status, timeout()));
   return QLIN_OK;
 }
 

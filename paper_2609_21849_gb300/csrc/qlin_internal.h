@@ -16,6 +16,10 @@ namespace qlin {
 // err / timeout_ns: device status word and limit of the bounded waits.
 cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float* scale_src,
                                const qlin_nvfp4_t& out, cudaStream_t s, int num_sms);
+// The same of an x that the kernel launched before on s writes.
+cudaError_t launch_quant_nvfp4_after(const void* x, int64_t M, int64_t K, const float* scale_src,
+                                     const qlin_nvfp4_t& out, cudaStream_t s, int num_sms,
+                                     unsigned* err, uint64_t timeout_ns);
 cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* scale_src,
                              const qlin_fp8_t& out, cudaStream_t s, int num_sms, unsigned* err,
                              uint64_t timeout_ns);

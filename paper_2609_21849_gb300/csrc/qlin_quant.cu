@@ -13,6 +13,7 @@
 // Static tensor scale:
 //   quant_nvfp4_kernel    bf16 -> packed e2m1 codes + E4M3 block scales in the
 //                         tensor-core scale layout + FP32 tensor scale
+//   quant_nvfp4_ring_kernel  the same of an x that was just written
 //   quant_fp8_kernel      bf16 -> E4M3 codes with one tensor scale
 // Weights:
 //   quant_fp8_rows_kernel bf16 -> E4M3 codes with one scale per row
@@ -21,9 +22,9 @@
 // two chunks of one NVFP4 block, and four neighbouring lanes hold one
 // 64-element group (because K % 64 == 0 a group never straddles a row).
 // quant_nvfp4_kernel and two_phase_kernel load straight to registers; the static
-// FP8 quantizer (stream_tiles) cuts x into 16 KB tiles that a persistent grid
-// (three CTAs per SM) takes through a four-deep shared-memory ring filled by
-// bulk copies, ~192 KB per SM of input in flight.
+// FP8 quantizer and the dynamic chain's NVFP4 one (stream_tiles) cut x into 16 KB
+// tiles that a persistent grid (three CTAs per SM) takes through a four-deep
+// shared-memory ring filled by bulk copies, ~192 KB per SM of input in flight.
 #include <atomic>
 
 #include "qlin_internal.h"
@@ -498,6 +499,27 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
     quantize(t, w);
     t = nt;
   }
+}
+
+// NVFP4 with a static scale, of an x that the kernel before has just written (the
+// dynamic chain's y): through the ring, whose 192 KB per SM of bulk copies in
+// flight start on x as soon as that kernel ends.  The direct loads above are
+// faster on an x that comes from HBM alone, but took 25.3 us instead of 20.6
+// right after a 4608 x 12288 GEMM (chains: 4608 x 12288 x 256 61.0 -> 56.7 us,
+// 4608 x 9216 x 3072 60.8 -> 59.7, 18432 x 6144 x 256 117 -> 111).
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm)
+    quant_nvfp4_ring_kernel(const uint4* __restrict__ x, uint64_t n_chunks,
+                            const float* scale_src, float* sdec_out, Nvfp4Op<uint32_t> op,
+                            unsigned* err, uint64_t timeout_ns) {
+  l2_prefetch_first_tile(x, n_chunks);
+  grid_dep_wait();
+  grid_dep_launch();
+  __shared__ float r_table[128];
+  op.bind(r_table);
+  stream_tiles(
+      x, n_chunks, op,
+      [&](Nvfp4Op<uint32_t>& o) { o.s_enc = encode_scale(static_scale(scale_src, sdec_out)); },
+      err, timeout_ns);
 }
 
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
@@ -1191,6 +1213,18 @@ cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const 
                                      uint64_t timeout_ns) {
   return launch_dynamic(x, (uint64_t)M * (uint64_t)K / 8, fp8_op(out), 448.0f, out.scale, sync,
                         clear, s, num_sms, timeout_ns);
+}
+
+cudaError_t launch_quant_nvfp4_after(const void* x, int64_t M, int64_t K, const float* scale_src,
+                                     const qlin_nvfp4_t& out, cudaStream_t s, int num_sms,
+                                     unsigned* err, uint64_t timeout_ns) {
+  const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
+  if (n_chunks >= (1ull << 32)) return launch_quant_nvfp4(x, M, K, scale_src, out, s, num_sms);
+  const cudaError_t e = set_smem<quant_nvfp4_ring_kernel>();
+  if (e != cudaSuccess) return e;
+  return launch_pdl(quant_nvfp4_ring_kernel, stream_grid(n_chunks, num_sms), kThreads, kSmem, s,
+                    static_cast<const uint4*>(x), n_chunks, scale_src, out.tensor_scale,
+                    nvfp4_op<uint32_t>(K, out), err, timeout_ns);
 }
 
 cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float* scale_src,

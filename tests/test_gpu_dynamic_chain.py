@@ -38,7 +38,9 @@ def _chain(x, w, label, rows=None):
     return yq
 
 
-@pytest.mark.parametrize("M,N,K", [(128, 256, 256), (130, 320, 192), (333, 512, 1088)])
+# the last: y in more 16 KB tiles than CTAs, the last tile partial
+@pytest.mark.parametrize("M,N,K", [(128, 256, 256), (130, 320, 192), (333, 512, 1088),
+                                   (4601, 2112, 128)])
 def test_dynamic_chain_ragged(M, N, K):
     x = synthetic.act_entry_outliers(M + N + K, M, K)
     (w,) = synthetic.weights(N + 1, [(N, K)], 0.02)
