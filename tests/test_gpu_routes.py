@@ -90,11 +90,13 @@ def test_grid_wait_that_expires_gives_the_same_codes(M, K):
     assert int(ws.count_nonzero()) == 0
 
 
+@pytest.mark.parametrize("M", [1, 2055, 2048 * SMS // 4, 2048 * SMS // 4 + 5])
 @pytest.mark.parametrize("shift", [0, 8])
-def test_static_nvfp4_alignment_and_partial_tile(shift):
-    # x 32-byte aligned (one 32-byte load per block) and only 16-byte aligned
-    # (two 16-byte loads); 2055 * 64 / 8 chunks end in a partial tile
-    M, K = 2055, 64
+def test_static_nvfp4_alignment_and_partial_tile(shift, M):
+    # one block per thread up to 2048 threads per SM, tiles beyond; x 32-byte
+    # aligned (there one 32-byte load per block) and only 16-byte aligned (two
+    # 16-byte loads); the last CTA's share and the last tile are partial
+    K = 64
     bits = synthetic.act_entry_outliers(9, M, K)
     buf = torch.zeros(M * K + 16, dtype=torch.bfloat16, device="cuda")
     x = buf[shift:shift + M * K].view(M, K)
