@@ -557,12 +557,14 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
       timeout_ns);
 }
 
-// FP8 weights, one scale per row: one warp per row, held in registers up to
-// K = 3072 (12288 x 3072: 21.3 -> 18.6 us), else two passes over it (the second
-// hits L1/L2).  Offline, once per layer.
-constexpr int kRowRegs = 12;   // chunks per lane
-
-__global__ void __launch_bounds__(kThreads, 2)
+// FP8 weights, one scale per row: one warp per row, held in kRegs chunks per lane
+// (kTwoPass: longer rows in two passes, the second of which hits L1/L2).  Short
+// rows take an instance of their own, with as many CTAs per SM as its registers
+// allow: through the twelve-chunk one 100003 x 64 took 42.8 us (14.6 with two
+// chunks, 18.7 in two passes) and 12288 x 1024 9.6 (7.2 with four chunks, 8.1).
+// 12288 x 3072: 18.3 us, in two passes 21.2.  Offline, once per layer.
+template <int kRegs, int kPerSm, bool kTwoPass = false>
+__global__ void __launch_bounds__(kThreads, kPerSm)
     quant_fp8_rows_kernel(const uint4* __restrict__ w, int64_t rows, int64_t K,
                           float* __restrict__ s_rows, uint2* __restrict__ codes) {
   grid_dep_wait();
@@ -574,20 +576,20 @@ __global__ void __launch_bounds__(kThreads, 2)
   for (int64_t r = warp; r < rows; r += nwarps) {
     const uint4* wr = w + r * cpr;
     uint32_t m = 0;
-    if (cpr <= 32 * kRowRegs) {
-      uint4 v[kRowRegs];
+    if (!kTwoPass || cpr <= 32 * kRegs) {
+      uint4 v[kRegs];
 #pragma unroll
-      for (int i = 0; i < kRowRegs; ++i)
+      for (int i = 0; i < kRegs; ++i)
         v[i] = lane + 32 * i < cpr ? ldg128(wr + lane + 32 * i) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int i = 0; i < kRowRegs; ++i) m = max(m, chunk_abs_max_bits(v[i]));
+      for (int i = 0; i < kRegs; ++i) m = max(m, chunk_abs_max_bits(v[i]));
       m = __reduce_max_sync(0xFFFFFFFFu, m);
       const float amax = __uint_as_float(m << 16);
       const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f);
       const float s_enc = encode_scale(s_dec);
       if (lane == 0) s_rows[r] = s_dec;
 #pragma unroll
-      for (int i = 0; i < kRowRegs; ++i) {
+      for (int i = 0; i < kRegs; ++i) {
         if (lane + 32 * i >= cpr) continue;
         float f[8];
         unpack8(v[i], f);
@@ -598,19 +600,21 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
       continue;
     }
-    for (int64_t c = lane; c < cpr; c += 32) m = max(m, chunk_abs_max_bits(__ldg(wr + c)));
-    m = __reduce_max_sync(0xFFFFFFFFu, m);
-    const float amax = __uint_as_float(m << 16);
-    const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f);
-    const float s_enc = encode_scale(s_dec);
-    if (lane == 0) s_rows[r] = s_dec;
-    for (int64_t c = lane; c < cpr; c += 32) {
-      float f[8];
-      unpack8(__ldg(wr + c), f);
+    if constexpr (kTwoPass) {
+      for (int64_t c = lane; c < cpr; c += 32) m = max(m, chunk_abs_max_bits(__ldg(wr + c)));
+      m = __reduce_max_sync(0xFFFFFFFFu, m);
+      const float amax = __uint_as_float(m << 16);
+      const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f);
+      const float s_enc = encode_scale(s_dec);
+      if (lane == 0) s_rows[r] = s_dec;
+      for (int64_t c = lane; c < cpr; c += 32) {
+        float f[8];
+        unpack8(__ldg(wr + c), f);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) f[i] = __fmul_rn(f[i], s_enc);
-      codes[r * cpr + c] =
-          make_uint2(e4m3x4(f[0], f[1], f[2], f[3]), e4m3x4(f[4], f[5], f[6], f[7]));
+        for (int i = 0; i < 8; ++i) f[i] = __fmul_rn(f[i], s_enc);
+        codes[r * cpr + c] =
+            make_uint2(e4m3x4(f[0], f[1], f[2], f[3]), e4m3x4(f[4], f[5], f[6], f[7]));
+      }
     }
   }
 }
@@ -1284,8 +1288,11 @@ cudaError_t launch_quant_fp8_rows(const void* w, int64_t N, int64_t K, const qli
                                   cudaStream_t s, int num_sms) {
   const int64_t want = (N + kThreads / 32 - 1) / (kThreads / 32);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms * 8));
-  return launch_pdl(quant_fp8_rows_kernel, grid, kThreads, 0, s, static_cast<const uint4*>(w), N, K,
-                    out.scale, reinterpret_cast<uint2*>(out.codes));
+  auto kern = K <= 2 * 256   ? quant_fp8_rows_kernel<2, 4>   // a chunk per lane: 256 of K
+              : K <= 4 * 256 ? quant_fp8_rows_kernel<4, 3>
+                             : quant_fp8_rows_kernel<12, 2, true>;
+  return launch_pdl(kern, grid, kThreads, 0, s, static_cast<const uint4*>(w), N, K, out.scale,
+                    reinterpret_cast<uint2*>(out.codes));
 }
 
 }  // namespace qlin

@@ -107,9 +107,11 @@ def test_static_nvfp4_alignment_and_partial_tile(shift, M):
     assert_nvfp4_equal(q, oracle.quant_nvfp4(bits, s), f"shift {shift}")
 
 
-@pytest.mark.parametrize("N,K", [(200, 64), (200, 3072), (33, 3136), (9, 12288)])
+@pytest.mark.parametrize("N,K", [(1, 64), (40003, 64), (200, 512), (200, 576), (3001, 1024),
+                                 (200, 1088), (200, 3072), (33, 3136), (9, 12288)])
 def test_fp8_weight_rows(N, K):
-    # rows held in registers up to K = 3072, read twice beyond
+    # rows held in registers (two, four or twelve chunks a lane) up to K = 512,
+    # 1024 and 3072, read twice beyond; more rows than warps
     (w,) = synthetic.weights(11, [(N, K)], 0.02)
     q = qlin.qlin_quantize_weight(to_dev(w), qlin.QLIN_FMT_FP8)
     codes, scales = oracle.quant_fp8_rows(w)[:2]
