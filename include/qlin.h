@@ -309,9 +309,9 @@ qlin_status qlin_sync_status(void *stream);
 qlin_status qlin_selftest_bounded_wait(uint64_t timeout_ns, void *stream);
 
 /* Wait limit used by every device-side spin (default 2 s), in ns.  The dynamic
- * quantizers wait at most 1 ms of it for the rest of their grid; a CTA whose
- * wait expires there reads all of x for the maximum itself: no error, the same
- * result. */
+ * quantizers wait at most 10 us of it for CTAs of their grid that are not
+ * running, then read x for the maximum in their place, with at most 1 ms of it
+ * for one another's last piece: no error, the same result. */
 void qlin_set_wait_timeout_ns(uint64_t ns);
 
 /* Short text for a status code (static storage). */

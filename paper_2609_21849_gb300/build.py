@@ -16,9 +16,11 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIB_DIR, "libqlin.so")
 SOURCES = ["qlin_api.cu", "qlin_quant.cu", "qlin_gemm.cu"]
-# the tensor-core rate probe of the measurement harness: a library of its own
+# the rate probes of the measurement harness and the probes of the quantizers'
+# grid-wide wait: a library of its own
 PROBE_LIB = os.path.join(LIB_DIR, "libqlin_probe.so")
-PROBE_SOURCES = ["qlin_probe.cu"]
+PROBE_SOURCES = ["qlin_probe.cu", "qlin_grid_probe.cu"]
+PROBE_SHARED = ["qlin_quant.cu"]   # the quantizer kernels, linked into both
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -71,7 +73,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     srcs = SOURCES + PROBE_SOURCES
     with cf.ThreadPoolExecutor(len(srcs)) as ex:
         objs = dict(zip(srcs, ex.map(compile_one, srcs)))
-    for lib, group in ((LIB, SOURCES), (PROBE_LIB, PROBE_SOURCES)):
+    for lib, group in ((LIB, SOURCES), (PROBE_LIB, PROBE_SOURCES + PROBE_SHARED)):
         tmp = lib + ".tmp"
         cmd = ([cc] + ARCH + ["-shared", "-cudart", "static", "-o", tmp] + [objs[f] for f in group]
                + ["-ldl", "-lpthread", "-lrt"])

@@ -119,12 +119,13 @@ qlin_status check_workspace(void* ws, size_t ws_bytes) {
   } while (0)
 
 }  // namespace
-// Workspace words: the dynamic quantizers' amax, arrival and departure counts
-// (words 0-2; zero between calls), and qlin_linear_dynamic's max |y| from the
-// GEMM epilogue and the epilogue's departure count (words 5 and 6; zero
-// between calls).
+// Workspace words: the dynamic quantizers' amax and counts (kGridSyncWords from
+// word 0; zero between calls), and qlin_linear_dynamic's max |y| from the GEMM
+// epilogue and the epilogue's departure count (words 5 and 6; zero between
+// calls).
 constexpr int kWsQuant = 0;
 constexpr int kWsChainAmax = 5;
+static_assert(kWsQuant + kGridSyncWords <= kWsChainAmax, "separate words");
 
 }  // namespace qlin
 
@@ -158,7 +159,7 @@ qlin_status qlin_quantize_act_nvfp4(const void* x_bf16, int64_t M, int64_t K,
   if (static_scale == nullptr) {
     QLIN_CUDA(launch_quant_nvfp4_dynamic(x_bf16, M, K, *out,
                                          static_cast<unsigned*>(workspace) + kWsQuant, false, s,
-                                         sms, timeout()));
+                                         sms, grid_wait(timeout())));
   } else {
     QLIN_CUDA(launch_quant_nvfp4(x_bf16, M, K, static_scale, *out, s, sms));
   }
@@ -185,7 +186,7 @@ qlin_status qlin_quantize_act_nvfp4_noalloc(const void* x_bf16, int64_t M, int64
   // the scratch words are cleared by the launch that uses them
   QLIN_CUDA(launch_quant_nvfp4_dynamic(x_bf16, M, K, *out,
                                        reinterpret_cast<unsigned*>(scratch) + kWsQuant, true, s,
-                                       sms, timeout()));
+                                       sms, grid_wait(timeout())));
   return QLIN_OK;
 }
 
@@ -205,7 +206,7 @@ qlin_status qlin_quantize_act_fp8(const void* x_bf16, int64_t M, int64_t K,
   if (static_scale == nullptr) {
     QLIN_CUDA(launch_quant_fp8_dynamic(x_bf16, M, K, *out,
                                        static_cast<unsigned*>(workspace) + kWsQuant, false, s, sms,
-                                       timeout()));
+                                       grid_wait(timeout())));
   } else {
     QLIN_CUDA(launch_quant_fp8(x_bf16, M, K, static_scale, *out, s, sms, status, timeout()));
   }

@@ -23,15 +23,27 @@ cudaError_t launch_quant_nvfp4_after(const void* x, int64_t M, int64_t K, const 
 cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* scale_src,
                              const qlin_fp8_t& out, cudaStream_t s, int num_sms, unsigned* err,
                              uint64_t timeout_ns);
-// Dynamic tensor scale.  sync: three device words of scratch, zero at launch
-// (clear = zero them first) and zero again when the kernel ends.
+// Limits of the dynamic quantizers' grid-wide wait: for CTAs that have not arrived
+// before the waiting ones read x in their place, then for the last pieces of x.
+// Ten microseconds are several times the CTAs' usual spread.
+struct GridWait {
+  uint64_t help_ns, stop_ns;
+};
+inline GridWait grid_wait(uint64_t limit_ns) {
+  return {std::min<uint64_t>(limit_ns, 10000), std::min<uint64_t>(limit_ns, 1000000)};
+}
+constexpr int kGridSyncWords = 5;
+// Dynamic tensor scale.  sync: kGridSyncWords device words of scratch, zero at
+// launch (clear = zero them first) and zero again when the kernel ends.
 cudaError_t launch_quant_nvfp4_dynamic(const void* x, int64_t M, int64_t K,
                                        const qlin_nvfp4_t& out, unsigned* sync, bool clear,
-                                       cudaStream_t s, int num_sms,
-                                       uint64_t timeout_ns);
+                                       cudaStream_t s, int num_sms, GridWait wait);
 cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
                                      unsigned* sync, bool clear, cudaStream_t s, int num_sms,
-                                     uint64_t timeout_ns);
+                                     GridWait wait);
+// How often CTAs gave that wait up since the last call (synchronises the device):
+// CTAs that helped, pieces of x they read, CTAs that read all of x alone.
+cudaError_t take_grid_counts(unsigned (&counts)[3]);
 cudaError_t launch_quant_fp8_rows(const void* w, int64_t N, int64_t K, const qlin_fp8_t& out,
                                   cudaStream_t s, int num_sms);
 

@@ -656,21 +656,36 @@ __device__ __forceinline__ void cp_async_wait_pending(int pending) {
   }
 }
 
+// How often a CTA gave up waiting for its grid: CTAs that helped, pieces they
+// read, CTAs that read all of x alone.  Counted on that path only.
+__device__ unsigned g_grid_counts[3];
+
+constexpr uint32_t kPieceChunks = 4096;       // 64 KB of x per ticket
+constexpr unsigned kAllRead = 1u << 30;       // added to the arrivals (a grid has fewer CTAs)
+constexpr uint32_t kMet = 0xFFFFFFFFu, kHelp = 0xFFFFFFFEu, kAlone = 0xFFFFFFFDu;
+
 // The maximum of the grid's warp maxima (max |x|, as bits) into *s_amax (shared
 // memory, for every thread): combine the CTA's, publish, arrive, wait for every
 // CTA, depart.  The grid is no larger than the machine, so its CTAs are resident
-// together unless other streams' kernels hold SMs for long -- or hold them
-// waiting, as another grid like this one would.  So the wait is bounded, and a
-// CTA whose wait expires reads all of x for the maximum itself: slow, but the
-// same value, and nothing waits without end.  (A cooperative launch, which
-// keeps the grid together, costs about 2 us outside a graph: 2.5 MB of FP8 6.2
-// us instead of 4.5.)
-constexpr uint64_t kGridWaitNs = 1000000;
-
+// together unless other streams' kernels hold SMs -- for long, or waiting, as
+// another grid like this one would.  So a CTA waits wait.help_ns only; then it
+// takes pieces of x by ticket, with every other CTA that waits, and when all of x
+// has been read that way the grid has met without the CTAs that are missing: they
+// find it so when they start.  Nothing then waits on a CTA that is not running,
+// and x is read once more in all.  (With 20 of 152 SMs held by another kernel,
+// 4608 x 3072 takes 50 us and 18432 x 3072 89; waiting 1 ms for the missing CTAs
+// and then reading all of x in every CTA took 1360 and 2820.  A cooperative
+// launch, which keeps the grid together, costs about 2 us outside a graph: 2.5 MB
+// of FP8 6.2 us instead of 4.5.)  The wait for the last pieces, which running CTAs
+// hold, is bounded by wait.stop_ns; a CTA whose wait expires there reads all of x
+// for itself.
+//
+// sync[0]: amax bits (fp32), sync[1]: arrivals, sync[2]: departures, sync[3]: the
+// next ticket, sync[4]: pieces read.
 template <int kThreadsPerBlock>
 __device__ __forceinline__ void grid_amax(const uint4* x, uint64_t n_chunks, uint32_t* warp_max,
-                                          unsigned* sync, float* s_amax, int* alone,
-                                          uint64_t wait_ns) {
+                                          unsigned* sync, float* s_amax, uint32_t* s_state,
+                                          GridWait wait) {
   const int tid = threadIdx.x;
   __syncthreads();   // warp_max is written
   auto combine = [&] {
@@ -679,59 +694,124 @@ __device__ __forceinline__ void grid_amax(const uint4* x, uint64_t n_chunks, uin
     for (int w = 0; w < kThreadsPerBlock / 32; ++w) b = max(b, warp_max[w]);
     return b;
   };
+  // The count and the amax are read together: a load that sees every CTA's
+  // arrival (or that all of x has been read) also sees every maximum released
+  // before it, which saves the second round trip to L2 that reading the amax
+  // afterwards took.
+  auto met = [&] {
+    const uint64_t pair = ld_acquire_gpu_pair(&sync[0]);
+    if ((uint32_t)(pair >> 32) < gridDim.x) return false;
+    *s_amax = __uint_as_float((uint32_t)pair);
+    return true;
+  };
+  // Poll until the grid has met or limit_ns have passed (0: no poll).
+  auto poll = [&](uint64_t limit_ns, uint32_t expired) {
+    if (limit_ns == 0) return expired;
+    const uint64_t t0 = global_timer_ns();
+    while (!met())
+      if (global_timer_ns() - t0 > limit_ns) return expired;
+    return kMet;
+  };
   if (tid == 0) {
     const uint32_t b = combine();
     if (b) atomicMax(&sync[0], b << 16);
     // the arrival releases the maximum above to every CTA that sees it
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&sync[1]) : "memory");
-    // The count and the amax are read together: a load that sees every
-    // CTA's arrival also sees every maximum released before it, which saves
-    // the second round trip to L2 that reading the amax afterwards took.
+    // (a loop of its own, the common case: through poll() below 0.1 us slower)
     const uint64_t t0 = global_timer_ns();
     uint64_t pair = ld_acquire_gpu_pair(&sync[0]);
     bool expired = false;
     while ((uint32_t)(pair >> 32) < gridDim.x && !expired) {
-      expired = global_timer_ns() - t0 > wait_ns;
+      expired = global_timer_ns() - t0 > wait.help_ns;
       pair = ld_acquire_gpu_pair(&sync[0]);
     }
-    *alone = (uint32_t)(pair >> 32) < gridDim.x ? 1 : 0;
+    *s_state = wait.help_ns == 0 || (uint32_t)(pair >> 32) < gridDim.x ? kHelp : kMet;
     *s_amax = __uint_as_float((uint32_t)pair);
   }
   __syncthreads();
-  if (tid == 0) {
-    // depart; the last CTA out resets the words.  The other warps do not wait
-    // for this atomic's round trip.
-    if (atomicAdd(&sync[2], 1u) == gridDim.x - 1u) {
-      sync[0] = 0u;
-      sync[1] = 0u;
-      sync[2] = 0u;
+  const uint32_t state = *s_state;
+  // Depart (by 1, a CTA that helped by 1 and 65536); the last CTA out resets the
+  // words, those of the pieces only if one helped.  The other warps do not wait
+  // for this atomic's round trip.
+  auto depart = [&](unsigned by) {
+    if (tid == 0) {
+      const unsigned before = atomicAdd(&sync[2], by);
+      if ((before & 0xFFFFu) == gridDim.x - 1u) {
+        sync[0] = 0u;
+        sync[1] = 0u;
+        sync[2] = 0u;
+        if ((before + by) >> 16) {
+          sync[3] = 0u;
+          sync[4] = 0u;
+        }
+      }
     }
-  }
-  if (*alone) {
-    uint32_t m = 0;
-    for (uint64_t c = tid; c < n_chunks; c += kThreadsPerBlock)
-      m = max(m, chunk_abs_max_bits(ldg128(x + c)));
-    m = __reduce_max_sync(0xFFFFFFFFu, m);
-    if ((tid & 31) == 0) warp_max[tid >> 5] = m;
-    __syncthreads();
-    if (tid == 0) *s_amax = __uint_as_float(combine() << 16);
-    __syncthreads();
+  };
+  if (state == kMet) depart(1u);
+  if (state == kHelp) {
+    __syncthreads();   // every thread has read s_state
+    const uint32_t pieces = (uint32_t)((n_chunks + kPieceChunks - 1) / kPieceChunks);
+    bool done = false;   // thread 0: the grid has met
+    if (tid == 0) atomicAdd(&g_grid_counts[0], 1u);
+    for (;;) {
+      if (tid == 0) {
+        uint32_t t = kMet;
+        if (!done && (t = atomicAdd(&sync[3], 1u)) >= pieces) t = poll(wait.stop_ns, kAlone);
+        *s_state = t;
+      }
+      __syncthreads();
+      const uint32_t t = *s_state;
+      if (t >= pieces) break;
+      // the last pieces first: the CTAs that are missing are mostly the last ones
+      const uint64_t c0 = (uint64_t)(pieces - 1u - t) * kPieceChunks;
+      uint32_t m = 0;
+#pragma unroll 4
+      for (uint32_t i = tid; i < kPieceChunks; i += kThreadsPerBlock)
+        if (c0 + i < n_chunks) m = max(m, chunk_abs_max_bits(ldg128(x + c0 + i)));
+      m = __reduce_max_sync(0xFFFFFFFFu, m);
+      if ((tid & 31) == 0) warp_max[tid >> 5] = m;
+      __syncthreads();
+      if (tid == 0) {
+        atomicAdd(&g_grid_counts[1], 1u);
+        const uint32_t b = combine();
+        if (b) atomicMax(&sync[0], b << 16);
+        __threadfence();
+        if (atomicAdd(&sync[4], 1u) == pieces - 1u) {
+          __threadfence();
+          asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&sync[1]), "r"(kAllRead)
+                       : "memory");
+        }
+        done = met();
+      }
+    }
+    if (*s_state == kAlone) {
+      if (tid == 0) atomicAdd(&g_grid_counts[2], 1u);
+      uint32_t m = 0;
+      for (uint64_t c = tid; c < n_chunks; c += kThreadsPerBlock)
+        m = max(m, chunk_abs_max_bits(ldg128(x + c)));
+      m = __reduce_max_sync(0xFFFFFFFFu, m);
+      if ((tid & 31) == 0) warp_max[tid >> 5] = m;
+      __syncthreads();
+      if (tid == 0) *s_amax = __uint_as_float(combine() << 16);
+      __syncthreads();
+    }
+    depart(0x10001u);
   }
 }
 
-// sync[0]: amax bits (fp32), sync[1]: arrival count, sync[2]: departure
-// count; all zero at launch, and the last CTA to depart zeroes them again, so
-// back-to-back launches (graph replays included) need no clearing between.
+// sync: the words of grid_amax, all zero at launch; the last CTA to depart zeroes
+// them again, so back-to-back launches (graph replays included) need no clearing
+// between.
 template <typename Op>
 __global__ void __launch_bounds__(kOnePassThreads, 1)
     onepass_kernel(const uint4* __restrict__ x, uint64_t n_chunks, uint32_t slice, Op op,
-                   float qmax, float* sdec_out, unsigned* sync, uint64_t wait_ns) {
+                   float qmax, float* sdec_out, unsigned* sync, GridWait wait) {
   extern __shared__ __align__(128) uint8_t qsm[];
   uint4* buf = reinterpret_cast<uint4*>(qsm);
   __shared__ uint32_t warp_max[kOnePassThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
-  __shared__ int alone;
+  __shared__ uint32_t state;
   grid_dep_wait();
   const int tid = threadIdx.x;
   const uint64_t c_begin = (uint64_t)blockIdx.x * slice;
@@ -787,7 +867,7 @@ __global__ void __launch_bounds__(kOnePassThreads, 1)
   }
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31) == 0) warp_max[tid >> 5] = m;
-  grid_amax<kOnePassThreads>(x, n_chunks, warp_max, sync, &s_amax, &alone, wait_ns);
+  grid_amax<kOnePassThreads>(x, n_chunks, warp_max, sync, &s_amax, &state, wait);
   const float amax = s_amax;
   const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
@@ -817,11 +897,11 @@ constexpr uint32_t kRegSliceMax = kRegUnits * kRegStride;       // 192 KB of x p
 template <typename Op>
 __global__ void __launch_bounds__(kRegThreads, 1)
     regpass_kernel(const uint4* __restrict__ x, uint64_t n_chunks, uint32_t slice, Op op,
-                   float qmax, float* sdec_out, unsigned* sync, uint64_t wait_ns) {
+                   float qmax, float* sdec_out, unsigned* sync, GridWait wait) {
   __shared__ uint32_t warp_max[kRegThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
-  __shared__ int alone;
+  __shared__ uint32_t state;
   grid_dep_wait();
   const uint32_t tid = threadIdx.x;
   const uint64_t c_begin = (uint64_t)blockIdx.x * slice;
@@ -850,7 +930,7 @@ __global__ void __launch_bounds__(kRegThreads, 1)
   grid_dep_launch();   // x is on chip: the next kernel may begin launching
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31u) == 0u) warp_max[tid >> 5] = m;
-  grid_amax<kRegThreads>(x, n_chunks, warp_max, sync, &s_amax, &alone, wait_ns);
+  grid_amax<kRegThreads>(x, n_chunks, warp_max, sync, &s_amax, &state, wait);
   const float amax = s_amax;
   const float s_dec = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
@@ -876,13 +956,13 @@ constexpr int kKeepSmem = kKeep * (int)kDirectTile * 16;
 template <typename Op>
 __global__ void __launch_bounds__(kThreads, kDirectPerSm)
     two_phase_kernel(const uint4* __restrict__ x, uint64_t n_chunks, Op op, float qmax,
-                     float* sdec_out, unsigned* sync, uint64_t wait_ns) {
+                     float* sdec_out, unsigned* sync, GridWait wait) {
   extern __shared__ __align__(128) uint8_t qsm[];
   uint4* const keep = reinterpret_cast<uint4*>(qsm);
   __shared__ uint32_t warp_max[kThreads / 32];
   __shared__ float op_table[128];
   __shared__ float s_amax;
-  __shared__ int alone;
+  __shared__ uint32_t state;
   l2_prefetch_first_tile(x, n_chunks);
   grid_dep_wait();
   grid_dep_launch();
@@ -948,7 +1028,7 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
   m = __reduce_max_sync(0xFFFFFFFFu, m);
   if ((tid & 31) == 0) warp_max[tid >> 5] = m;
   load(kept > 0 ? tile(kept - 1) : -1, v);   // the first tile not kept, while the grid meets
-  grid_amax<kThreads>(x, n_chunks, warp_max, sync, &s_amax, &alone, wait_ns);
+  grid_amax<kThreads>(x, n_chunks, warp_max, sync, &s_amax, &state, wait);
   const float am = s_amax;
   const float s_dec = (am == 0.0f) ? 1.0f : __fdiv_rn(am, qmax);
   if (blockIdx.x == 0 && tid == 0) *sdec_out = s_dec;
@@ -1078,16 +1158,13 @@ int stream_grid(uint64_t n_chunks, int num_sms) {
 
 }  // namespace
 
-// Limit of the grid-wide wait (the caller's wait limit, if that is shorter).
-static uint64_t grid_wait(uint64_t timeout_ns) { return std::min(timeout_ns, kGridWaitNs); }
-
 // One-pass dynamic quantization when x fits on chip: returns
 // cudaErrorNotSupported (nothing launched) when it does not, or when the
 // device cannot hold the grid resident.
 template <typename Op>
 static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                   float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                  int num_sms, uint64_t timeout_ns) {
+                                  int num_sms, GridWait wait) {
   // slices of whole 64-element groups (8 chunks), one per SM
   uint64_t slice = (n_chunks + num_sms - 1) / num_sms;
   slice = (slice + 7) / 8 * 8;
@@ -1112,18 +1189,18 @@ static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op
   }
   if (resident[reg] < 1 || grid > num_sms * resident[reg]) return cudaErrorNotSupported;
   if (clear) {
-    const cudaError_t e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s);
+    const cudaError_t e = cudaMemsetAsync(sync, 0, kGridSyncWords * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
   }
   return launch_pdl(kern, grid, threads, smem, s, static_cast<const uint4*>(x), n_chunks,
-                    (uint32_t)slice, op, qmax, sdec_out, sync, grid_wait(timeout_ns));
+                    (uint32_t)slice, op, qmax, sdec_out, sync, wait);
 }
 
 // x of any size: two phases over it in one launch.
 template <typename Op>
 static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                     float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                    int num_sms, uint64_t timeout_ns) {
+                                    int num_sms, GridWait wait) {
   static const cudaError_t attr = cudaFuncSetAttribute(
       two_phase_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKeepSmem);
   cudaError_t e = attr;
@@ -1137,11 +1214,11 @@ static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& 
     resident = r;
   }
   if (resident < 1) return cudaErrorLaunchOutOfResources;
-  if (clear && (e = cudaMemsetAsync(sync, 0, 3 * sizeof(unsigned), s)) != cudaSuccess) return e;
+  if (clear && (e = cudaMemsetAsync(sync, 0, kGridSyncWords * sizeof(unsigned), s)) != cudaSuccess) return e;
   const uint64_t tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
   const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms * std::min(resident, kDirectPerSm));
   return launch_pdl(two_phase_kernel<Op>, grid, kThreads, kKeepSmem, s, static_cast<const uint4*>(x),
-                    n_chunks, op, qmax, sdec_out, sync, grid_wait(timeout_ns));
+                    n_chunks, op, qmax, sdec_out, sync, wait);
 }
 
 // The cluster route takes x of up to 1 MB: there every CTA's eighth of x takes
@@ -1213,33 +1290,32 @@ static Fp8Op fp8_op(const qlin_fp8_t& out) {
 template <typename Op>
 static cudaError_t launch_dynamic(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                   float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                  int num_sms, uint64_t timeout_ns) {
+                                  int num_sms, GridWait wait) {
   if (n_chunks <= kClusterMaxChunks)
     return launch_cluster_quant(x, (uint32_t)n_chunks, op, qmax, sdec_out, s);
   const cudaError_t e = launch_onepass(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms,
-                                       timeout_ns);
+                                       wait);
   if (e != cudaErrorNotSupported) return e;
   return launch_two_phase(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms,
-                          timeout_ns);
+                          wait);
 }
 
 cudaError_t launch_quant_nvfp4_dynamic(const void* x, int64_t M, int64_t K,
                                        const qlin_nvfp4_t& out, unsigned* sync, bool clear,
-                                       cudaStream_t s, int num_sms,
-                                       uint64_t timeout_ns) {
+                                       cudaStream_t s, int num_sms, GridWait wait) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
   if (n_chunks < (1ull << 32))   // 32-bit index math is enough
     return launch_dynamic(x, n_chunks, nvfp4_op<uint32_t>(K, out), 2688.0f, out.tensor_scale, sync,
-                          clear, s, num_sms, timeout_ns);
+                          clear, s, num_sms, wait);
   return launch_two_phase(x, n_chunks, nvfp4_op<uint64_t>(K, out), 2688.0f, out.tensor_scale, sync,
-                          clear, s, num_sms, timeout_ns);
+                          clear, s, num_sms, wait);
 }
 
 cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
                                      unsigned* sync, bool clear, cudaStream_t s, int num_sms,
-                                     uint64_t timeout_ns) {
+                                     GridWait wait) {
   return launch_dynamic(x, (uint64_t)M * (uint64_t)K / 8, fp8_op(out), 448.0f, out.scale, sync,
-                        clear, s, num_sms, timeout_ns);
+                        clear, s, num_sms, wait);
 }
 
 cudaError_t launch_quant_nvfp4_after(const void* x, int64_t M, int64_t K, const float* scale_src,
@@ -1293,6 +1369,14 @@ cudaError_t launch_quant_fp8_rows(const void* w, int64_t N, int64_t K, const qli
                              : quant_fp8_rows_kernel<12, 2, true>;
   return launch_pdl(kern, grid, kThreads, 0, s, static_cast<const uint4*>(w), N, K, out.scale,
                     reinterpret_cast<uint2*>(out.codes));
+}
+
+cudaError_t take_grid_counts(unsigned (&counts)[3]) {
+  static const unsigned zero[3] = {};
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) e = cudaMemcpyFromSymbol(counts, g_grid_counts, sizeof counts);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_grid_counts, zero, sizeof zero);
+  return e;
 }
 
 }  // namespace qlin

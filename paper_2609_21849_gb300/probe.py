@@ -52,6 +52,13 @@ def _load():
         lib.qlin_probe_fill.restype = ctypes.c_int
         lib.qlin_probe_fill.argtypes = ([ctypes.c_int] * 5 + [ctypes.c_void_p, ctypes.c_ulonglong]
                                         + [ctypes.c_void_p] * 3)
+        u64 = ctypes.c_ulonglong
+        lib.qlin_probe_grid_max.restype = ctypes.c_int
+        lib.qlin_probe_grid_max.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_longlong,
+                                            ctypes.c_longlong, ctypes.c_char_p, ctypes.c_void_p,
+                                            u64, u64, ctypes.c_void_p, ctypes.c_void_p]
+        lib.qlin_probe_hold_sms.restype = ctypes.c_int
+        lib.qlin_probe_hold_sms.argtypes = [ctypes.c_int, u64, ctypes.c_void_p]
         _lib = lib
     return _lib
 
@@ -138,6 +145,28 @@ def fill_bytes_per_cycle(mode: int, threads: int, depth: int, iters: int = 3000,
     cyc = out.cpu().double().median().item()
     return {"mode": ("tiled_128B_box", "bulk")[mode], "threads": threads, "depth": depth,
             "bytes_per_cycle_per_sm": round(threads * iters * 16384 / cyc, 1)}
+
+
+def grid_max(x: torch.Tensor, out, sync: torch.Tensor, help_ns: int, stop_ns: int) -> tuple:
+    """The dynamic quantizer of x into `out` (NVFP4Tensor or FP8Tensor) with its
+    own wait limits (include/qlin_grid_probe.h); returns (CTAs that gave up
+    waiting for the grid, pieces of x they read, CTAs that read all of x)."""
+    from . import qlin
+    counts = (ctypes.c_uint * 3)()
+    st = _load().qlin_probe_grid_max(1 if isinstance(out, qlin.NVFP4Tensor) else 2, x.data_ptr(),
+                                     x.shape[0], x.shape[1], out.packed(), sync.data_ptr(),
+                                     help_ns, stop_ns, ctypes.addressof(counts),
+                                     torch.cuda.current_stream().cuda_stream)
+    if st != 0:
+        raise RuntimeError(f"qlin_probe_grid_max returned {st}")
+    return tuple(counts)
+
+
+def hold_sms(ctas: int, ns: int, stream) -> None:
+    """Occupy `ctas` SMs for `ns` nanoseconds (at most 5 ms)."""
+    st = _load().qlin_probe_hold_sms(ctas, ns, stream.cuda_stream)
+    if st != 0:
+        raise RuntimeError(f"qlin_probe_hold_sms({ctas}, {ns}) returned {st}")
 
 
 def copy_rates() -> dict:
