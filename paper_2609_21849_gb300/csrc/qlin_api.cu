@@ -13,7 +13,6 @@ namespace {
 // Device status word: kernels record device-side failures here.
 __device__ unsigned g_status_word;
 
-constexpr int kMaxDevices = 64;
 std::mutex g_dev_mutex;
 unsigned* g_status_ptr[kMaxDevices] = {};
 int g_num_sms[kMaxDevices] = {};
@@ -28,7 +27,7 @@ qlin_status cuda_fail(cudaError_t e) {
 
 // Per-device state, set up on the first call made on that device: the
 // address of the status word and the SM count.
-qlin_status device_state(unsigned** status, int* num_sms) {
+qlin_status device_state(unsigned** status, Device* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -51,7 +50,7 @@ qlin_status device_state(unsigned** status, int* num_sms) {
     g_num_sms[dev] = sms;
   }
   *status = g_status_ptr[dev];
-  *num_sms = g_num_sms[dev];
+  *out = {dev, g_num_sms[dev]};
   return QLIN_OK;
 }
 
@@ -153,15 +152,15 @@ qlin_status qlin_quantize_act_nvfp4(const void* x_bf16, int64_t M, int64_t K,
   if (static_scale != nullptr && !aligned(static_scale, 4)) return QLIN_ERR_MISALIGNED;
   if (static_scale == nullptr) QLIN_TRY(check_workspace(workspace, ws_bytes));
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (static_scale == nullptr) {
     QLIN_CUDA(launch_quant_nvfp4_dynamic(x_bf16, M, K, *out,
                                          static_cast<unsigned*>(workspace) + kWsQuant, false, s,
-                                         sms, grid_wait(timeout())));
+                                         dev, grid_wait(timeout())));
   } else {
-    QLIN_CUDA(launch_quant_nvfp4(x_bf16, M, K, static_scale, *out, s, sms));
+    QLIN_CUDA(launch_quant_nvfp4(x_bf16, M, K, static_scale, *out, s, dev));
   }
   return QLIN_OK;
 }
@@ -178,15 +177,15 @@ qlin_status qlin_quantize_act_nvfp4_noalloc(const void* x_bf16, int64_t M, int64
     return QLIN_ERR_WORKSPACE;
   }
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
   unsigned char* scratch = nullptr;
   QLIN_TRY(noalloc_scratch(&scratch));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // the scratch words are cleared by the launch that uses them
   QLIN_CUDA(launch_quant_nvfp4_dynamic(x_bf16, M, K, *out,
                                        reinterpret_cast<unsigned*>(scratch) + kWsQuant, true, s,
-                                       sms, grid_wait(timeout())));
+                                       dev, grid_wait(timeout())));
   return QLIN_OK;
 }
 
@@ -200,15 +199,15 @@ qlin_status qlin_quantize_act_fp8(const void* x_bf16, int64_t M, int64_t K,
   if (static_scale != nullptr && !aligned(static_scale, 4)) return QLIN_ERR_MISALIGNED;
   if (static_scale == nullptr) QLIN_TRY(check_workspace(workspace, ws_bytes));
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (static_scale == nullptr) {
     QLIN_CUDA(launch_quant_fp8_dynamic(x_bf16, M, K, *out,
-                                       static_cast<unsigned*>(workspace) + kWsQuant, false, s, sms,
+                                       static_cast<unsigned*>(workspace) + kWsQuant, false, s, dev,
                                        grid_wait(timeout())));
   } else {
-    QLIN_CUDA(launch_quant_fp8(x_bf16, M, K, static_scale, *out, s, sms, status, timeout()));
+    QLIN_CUDA(launch_quant_fp8(x_bf16, M, K, static_scale, *out, s, dev, status, timeout()));
   }
   return QLIN_OK;
 }
@@ -226,9 +225,9 @@ qlin_status qlin_quantize_weight(const void* w_bf16, int64_t N, int64_t K, qlin_
   QLIN_TRY(check_fp8(out, N, K));
   if (!out->per_channel) return QLIN_ERR_INVALID_ARG;
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
-  QLIN_CUDA(launch_quant_fp8_rows(w_bf16, N, K, *out, static_cast<cudaStream_t>(stream), sms));
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
+  QLIN_CUDA(launch_quant_fp8_rows(w_bf16, N, K, *out, static_cast<cudaStream_t>(stream), dev));
   return QLIN_OK;
 }
 
@@ -302,9 +301,9 @@ static qlin_status gemm_common(bool fp4, const void* Aany, const void* Wany, voi
     return QLIN_ERR_INVALID_ARG;  // nothing to write
   }
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
-  cudaError_t e = launch_gemm(a, static_cast<cudaStream_t>(stream), sms, status,
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
+  cudaError_t e = launch_gemm(a, static_cast<cudaStream_t>(stream), dev, status,
                               g_timeout_ns.load(std::memory_order_relaxed));
   if (e != cudaSuccess) return cuda_fail(e);
   return QLIN_OK;
@@ -347,9 +346,9 @@ static qlin_status gemm16(const void* a16, int64_t lda, const void* w16, int64_t
   a.N = N;
   a.K = K;
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
-  cudaError_t e = launch_gemm(a, static_cast<cudaStream_t>(stream), sms, status, timeout());
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
+  cudaError_t e = launch_gemm(a, static_cast<cudaStream_t>(stream), dev, status, timeout());
   if (e != cudaSuccess) return cuda_fail(e);
   return QLIN_OK;
 }
@@ -379,9 +378,9 @@ qlin_status qlin_linear_dynamic(const qlin_nvfp4_t* A, const qlin_nvfp4_t* W, vo
   QLIN_TRY(gemm_common(true, A, W, y_bf16, nullptr, nullptr, 0, stream, amax, nullptr,
                        y_q->tensor_scale));
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
-  QLIN_CUDA(launch_quant_nvfp4_after(y_bf16, A->rows, W->rows, y_q->tensor_scale, *y_q, s, sms,
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
+  QLIN_CUDA(launch_quant_nvfp4_after(y_bf16, A->rows, W->rows, y_q->tensor_scale, *y_q, s, dev,
                                      status, timeout()));
   return QLIN_OK;
 }
@@ -395,8 +394,8 @@ qlin_status qlin_linear_fused_fp8(const qlin_fp8_t* A, const qlin_fp8_t* W, void
 
 qlin_status qlin_sync_status(void* stream) {
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   QLIN_CUDA(cudaStreamSynchronize(s));
   unsigned word = 0;
@@ -411,8 +410,8 @@ qlin_status qlin_sync_status(void* stream) {
 
 qlin_status qlin_selftest_bounded_wait(uint64_t timeout_ns, void* stream) {
   unsigned* status;
-  int sms;
-  QLIN_TRY(device_state(&status, &sms));
+  Device dev;
+  QLIN_TRY(device_state(&status, &dev));
   timeout_ns = std::min<uint64_t>(std::max<uint64_t>(timeout_ns, 1000ull), 2000000000ull);
   QLIN_CUDA(launch_wait_selftest(timeout_ns, static_cast<cudaStream_t>(stream), status));
   return QLIN_OK;

@@ -1126,7 +1126,7 @@ CUresult encode_scales(CUtensorMap* map, const void* base, uint64_t rows, uint64
 }
 
 template <bool kFp4, int kBN, bool kPair, bool kRequant, bool kBf16 = false>
-cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned* err,
+cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, Device dev, unsigned* err,
                        uint64_t timeout_ns) {
   using C = Cfg<kFp4, kBN, kPair>;
   constexpr int kCM = kPair ? 2 : 1;
@@ -1185,23 +1185,26 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned*
   cfg.attrs = attr;
   cfg.numAttrs = 1;   // the occupancy query below takes the cluster attribute only
 
-  // one-time per instantiation: opt into the shared memory size and find how
-  // many clusters fit at once (a persistent grid never exceeds that)
-  static std::once_flag once;
-  static cudaError_t setup_err = cudaSuccess;
-  static int max_clusters = 0;
-  std::call_once(once, [&] {
-    setup_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     C::kSmemBytes);
-    if (setup_err != cudaSuccess) return;
-    cfg.gridDim = dim3((unsigned)(num_sms / kCM * kCM), 1, 1);
-    setup_err = cudaOccupancyMaxActiveClusters(&max_clusters, kern, &cfg);
-    if (setup_err == cudaSuccess && max_clusters < 1) setup_err = cudaErrorInvalidConfiguration;
+  // once per instantiation and device: opt into the shared memory size and find
+  // how many clusters fit at once (a persistent grid never exceeds that)
+  struct Setup {
+    cudaError_t err;
+    int max_clusters;
+  };
+  static PerDevice<Setup> per_device;
+  const Setup& setup = per_device.get(dev.index, [&] {
+    Setup t{cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes),
+            0};
+    if (t.err != cudaSuccess) return t;
+    cfg.gridDim = dim3((unsigned)(dev.num_sms / kCM * kCM), 1, 1);
+    t.err = cudaOccupancyMaxActiveClusters(&t.max_clusters, kern, &cfg);
+    if (t.err == cudaSuccess && t.max_clusters < 1) t.err = cudaErrorInvalidConfiguration;
+    return t;
   });
-  if (setup_err != cudaSuccess) return setup_err;
+  if (setup.err != cudaSuccess) return setup.err;
   const int64_t tiles_m = (a.M + kBM - 1) / kBM;
   const int64_t ctiles = ((tiles_m + kCM - 1) / kCM) * ((a.N + kBN - 1) / kBN);
-  const int clusters = (int)std::min<int64_t>(ctiles, std::min(max_clusters, num_sms / kCM));
+  const int clusters = (int)std::min<int64_t>(ctiles, std::min(setup.max_clusters, dev.num_sms / kCM));
   cfg.gridDim = dim3((unsigned)(clusters * kCM), 1, 1);
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, ta, tb, tsa, tsb, ty, p);
@@ -1216,18 +1219,18 @@ Tile tile_of(const GemmArgs& a, int num_sms) {
 }
 
 template <bool kFp4>
-cudaError_t dispatch_bn(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned* err,
+cudaError_t dispatch_bn(const GemmArgs& a, cudaStream_t s, Device dev, unsigned* err,
                         uint64_t timeout_ns) {
   const bool requant = a.next_scale != nullptr;
-  switch (tile_of(a, num_sms)) {
+  switch (tile_of(a, dev.num_sms)) {
     case Tile::kPair:
-      return requant ? launch_cfg<kFp4, 256, true, true>(a, s, num_sms, err, timeout_ns)
-                     : launch_cfg<kFp4, 256, true, false>(a, s, num_sms, err, timeout_ns);
+      return requant ? launch_cfg<kFp4, 256, true, true>(a, s, dev, err, timeout_ns)
+                     : launch_cfg<kFp4, 256, true, false>(a, s, dev, err, timeout_ns);
     case Tile::kSingle:
-      return requant ? launch_cfg<kFp4, 128, false, true>(a, s, num_sms, err, timeout_ns)
-                     : launch_cfg<kFp4, 128, false, false>(a, s, num_sms, err, timeout_ns);
+      return requant ? launch_cfg<kFp4, 128, false, true>(a, s, dev, err, timeout_ns)
+                     : launch_cfg<kFp4, 128, false, false>(a, s, dev, err, timeout_ns);
     default:
-      return launch_cfg<kFp4, 64, false, false>(a, s, num_sms, err, timeout_ns);
+      return launch_cfg<kFp4, 64, false, false>(a, s, dev, err, timeout_ns);
   }
 }
 
@@ -1262,15 +1265,15 @@ CUresult encode_tensor_map_out_bf16(CUtensorMap* map, void* base, uint64_t cols,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned* err,
+cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s, Device dev, unsigned* err,
                         uint64_t timeout_ns) {
   if (a.bf16) {
-    return tile_of(a, num_sms) == Tile::kPair
-               ? launch_cfg<false, 256, true, false, true>(a, s, num_sms, err, timeout_ns)
-               : launch_cfg<false, 128, false, false, true>(a, s, num_sms, err, timeout_ns);
+    return tile_of(a, dev.num_sms) == Tile::kPair
+               ? launch_cfg<false, 256, true, false, true>(a, s, dev, err, timeout_ns)
+               : launch_cfg<false, 128, false, false, true>(a, s, dev, err, timeout_ns);
   }
-  return a.fp4 ? dispatch_bn<true>(a, s, num_sms, err, timeout_ns)
-               : dispatch_bn<false>(a, s, num_sms, err, timeout_ns);
+  return a.fp4 ? dispatch_bn<true>(a, s, dev, err, timeout_ns)
+               : dispatch_bn<false>(a, s, dev, err, timeout_ns);
 }
 
 cudaError_t launch_wait_selftest(uint64_t timeout_ns, cudaStream_t s, unsigned* err) {

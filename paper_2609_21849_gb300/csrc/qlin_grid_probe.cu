@@ -15,12 +15,13 @@ __global__ void __launch_bounds__(32) hold_kernel(unsigned long long ns) {
   while (global_timer_ns() - t0 < ns) __nanosleep(200);
 }
 
-int num_sms() {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return 0;
-  return sms;
+// The current device (no SMs: none that can be used).
+Device device() {
+  Device d{0, 0};
+  if (cudaGetDevice(&d.index) != cudaSuccess || d.index >= kMaxDevices ||
+      cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, d.index) != cudaSuccess)
+    return {0, 0};
+  return d;
 }
 
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
@@ -45,17 +46,17 @@ extern "C" int qlin_probe_grid_max(int fmt, const void* x, long long M, long lon
     if (o.codes == nullptr || o.scales == nullptr || o.tensor_scale == nullptr || o.rows != M ||
         o.K != K || !aligned(o.codes, 16))
       return 1;
-    const int sms = num_sms();
-    if (sms == 0) return 4;
-    e = launch_quant_nvfp4_dynamic(x, M, K, o, sync, false, s, sms, wait);
+    const Device dev = device();
+    if (dev.num_sms == 0) return 4;
+    e = launch_quant_nvfp4_dynamic(x, M, K, o, sync, false, s, dev, wait);
   } else {
     const qlin_fp8_t& o = *static_cast<const qlin_fp8_t*>(out);
     if (o.codes == nullptr || o.scale == nullptr || o.per_channel || o.rows != M || o.K != K ||
         !aligned(o.codes, 16))
       return 1;
-    const int sms = num_sms();
-    if (sms == 0) return 4;
-    e = launch_quant_fp8_dynamic(x, M, K, o, sync, false, s, sms, wait);
+    const Device dev = device();
+    if (dev.num_sms == 0) return 4;
+    e = launch_quant_fp8_dynamic(x, M, K, o, sync, false, s, dev, wait);
   }
   unsigned got[3] = {};
   if (e == cudaSuccess) e = take_grid_counts(got);
@@ -65,7 +66,7 @@ extern "C" int qlin_probe_grid_max(int fmt, const void* x, long long M, long lon
 
 extern "C" int qlin_probe_hold_sms(int ctas, unsigned long long ns, void* stream) {
   if (ctas < 1 || ns > 5000000) return 1;
-  if (ctas > num_sms()) return 1;
+  if (ctas > device().num_sms) return 1;
   if (cudaFuncSetAttribute(hold_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kHoldSmem) !=
       cudaSuccess)
     return 4;

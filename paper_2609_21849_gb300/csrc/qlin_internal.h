@@ -9,19 +9,26 @@
 
 #include "qlin.h"
 #include "qlin_device.cuh"
+#include "qlin_per_device.h"
 
 namespace qlin {
+
+// The device that a launch goes to: the current one.
+struct Device {
+  int index;   // below kMaxDevices
+  int num_sms;
+};
 
 // ---- quantizers (qlin_quant.cu) ----
 // err / timeout_ns: device status word and limit of the bounded waits.
 cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float* scale_src,
-                               const qlin_nvfp4_t& out, cudaStream_t s, int num_sms);
+                               const qlin_nvfp4_t& out, cudaStream_t s, Device dev);
 // The same of an x that the kernel launched before on s writes.
 cudaError_t launch_quant_nvfp4_after(const void* x, int64_t M, int64_t K, const float* scale_src,
-                                     const qlin_nvfp4_t& out, cudaStream_t s, int num_sms,
+                                     const qlin_nvfp4_t& out, cudaStream_t s, Device dev,
                                      unsigned* err, uint64_t timeout_ns);
 cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* scale_src,
-                             const qlin_fp8_t& out, cudaStream_t s, int num_sms, unsigned* err,
+                             const qlin_fp8_t& out, cudaStream_t s, Device dev, unsigned* err,
                              uint64_t timeout_ns);
 // Limits of the dynamic quantizers' grid-wide wait: for CTAs that have not arrived
 // before the waiting ones read x in their place, then for the last pieces of x.
@@ -37,15 +44,15 @@ constexpr int kGridSyncWords = 5;
 // launch (clear = zero them first) and zero again when the kernel ends.
 cudaError_t launch_quant_nvfp4_dynamic(const void* x, int64_t M, int64_t K,
                                        const qlin_nvfp4_t& out, unsigned* sync, bool clear,
-                                       cudaStream_t s, int num_sms, GridWait wait);
+                                       cudaStream_t s, Device dev, GridWait wait);
 cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
-                                     unsigned* sync, bool clear, cudaStream_t s, int num_sms,
+                                     unsigned* sync, bool clear, cudaStream_t s, Device dev,
                                      GridWait wait);
 // How often CTAs gave that wait up since the last call (synchronises the device):
 // CTAs that helped, pieces of x they read, CTAs that read all of x alone.
 cudaError_t take_grid_counts(unsigned (&counts)[3]);
 cudaError_t launch_quant_fp8_rows(const void* w, int64_t N, int64_t K, const qlin_fp8_t& out,
-                                  cudaStream_t s, int num_sms);
+                                  cudaStream_t s, Device dev);
 
 // ---- GEMMs (qlin_gemm.cu) ----
 struct GemmArgs {
@@ -75,7 +82,7 @@ struct GemmArgs {
   unsigned* y_departures;
   float* y_sdec;
 };
-cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s, int num_sms, unsigned* err,
+cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s, Device dev, unsigned* err,
                         uint64_t timeout_ns);
 cudaError_t launch_wait_selftest(uint64_t timeout_ns, cudaStream_t s, unsigned* err);
 

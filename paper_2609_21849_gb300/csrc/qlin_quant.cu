@@ -1126,12 +1126,22 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
   op.block(v, c, own);
 }
 
-// Opt each kernel into kSmem bytes of dynamic shared memory, once.
+// Opt a kernel into `smem` bytes of dynamic shared memory and find how many of its
+// CTAs an SM holds, once per device.
+struct Setup {
+  cudaError_t err;
+  int resident;
+};
 template <auto kKern>
-cudaError_t set_smem() {
-  static const cudaError_t e =
-      cudaFuncSetAttribute(kKern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  return e;
+const Setup& setup(Device dev, int threads, int smem) {
+  static PerDevice<Setup> per_device;
+  return per_device.get(dev.index, [&] {
+    Setup t{cudaFuncSetAttribute(kKern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), 0};
+    if (t.err == cudaSuccess && cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                    &t.resident, kKern, threads, smem) != cudaSuccess)
+      t.resident = 0;
+    return t;
+  });
 }
 
 // Launch with programmatic stream serialization (see grid_dep_wait).
@@ -1164,30 +1174,26 @@ int stream_grid(uint64_t n_chunks, int num_sms) {
 template <typename Op>
 static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                   float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                  int num_sms, GridWait wait) {
+                                  Device dev, GridWait wait) {
   // slices of whole 64-element groups (8 chunks), one per SM
-  uint64_t slice = (n_chunks + num_sms - 1) / num_sms;
+  uint64_t slice = (n_chunks + dev.num_sms - 1) / dev.num_sms;
   slice = (slice + 7) / 8 * 8;
   if (slice > (uint64_t)kOnePassSliceMax || slice == 0) return cudaErrorNotSupported;
   const int grid = (int)((n_chunks + slice - 1) / slice);
   // NVFP4: held in registers where the slice fits, else in shared memory
-  bool reg = false;
-  auto kern = onepass_kernel<Op>;
-  if constexpr (Op::kBlockMax) {
-    reg = slice <= (uint64_t)kRegSliceMax;
-    if (reg) kern = regpass_kernel<Op>;
-  }
+  const bool reg = Op::kBlockMax && slice <= (uint64_t)kRegSliceMax;
   const int threads = reg ? kRegThreads : kOnePassThreads, smem = reg ? 0 : kOnePassSmem;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      onepass_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePassSmem);
-  if (attr != cudaSuccess) return attr;
-  static int resident[2] = {-1, -1};   // CTAs of each kernel one SM can hold
-  if (resident[reg] < 0) {
-    int r = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kern, threads, smem) != cudaSuccess) r = 0;
-    resident[reg] = r;
+  auto kern = onepass_kernel<Op>;
+  const Setup* st = nullptr;
+  if constexpr (Op::kBlockMax) {
+    if (reg) {
+      kern = regpass_kernel<Op>;
+      st = &setup<regpass_kernel<Op>>(dev, threads, smem);
+    }
   }
-  if (resident[reg] < 1 || grid > num_sms * resident[reg]) return cudaErrorNotSupported;
+  if (st == nullptr) st = &setup<onepass_kernel<Op>>(dev, threads, smem);
+  if (st->err != cudaSuccess) return st->err;
+  if (st->resident < 1 || grid > dev.num_sms * st->resident) return cudaErrorNotSupported;
   if (clear) {
     const cudaError_t e = cudaMemsetAsync(sync, 0, kGridSyncWords * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
@@ -1200,23 +1206,14 @@ static cudaError_t launch_onepass(const void* x, uint64_t n_chunks, const Op& op
 template <typename Op>
 static cudaError_t launch_two_phase(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                     float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                    int num_sms, GridWait wait) {
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      two_phase_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKeepSmem);
-  cudaError_t e = attr;
+                                    Device dev, GridWait wait) {
+  const Setup& st = setup<two_phase_kernel<Op>>(dev, kThreads, kKeepSmem);
+  cudaError_t e = st.err;
   if (e != cudaSuccess) return e;
-  static int resident = -1;   // CTAs one SM can hold
-  if (resident < 0) {
-    int r = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, two_phase_kernel<Op>, kThreads,
-                                                           kKeepSmem)) != cudaSuccess)
-      return e;
-    resident = r;
-  }
-  if (resident < 1) return cudaErrorLaunchOutOfResources;
+  if (st.resident < 1) return cudaErrorLaunchOutOfResources;
   if (clear && (e = cudaMemsetAsync(sync, 0, kGridSyncWords * sizeof(unsigned), s)) != cudaSuccess) return e;
   const uint64_t tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
-  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms * std::min(resident, kDirectPerSm));
+  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)dev.num_sms * std::min(st.resident, kDirectPerSm));
   return launch_pdl(two_phase_kernel<Op>, grid, kThreads, kKeepSmem, s, static_cast<const uint4*>(x),
                     n_chunks, op, qmax, sdec_out, sync, wait);
 }
@@ -1290,57 +1287,57 @@ static Fp8Op fp8_op(const qlin_fp8_t& out) {
 template <typename Op>
 static cudaError_t launch_dynamic(const void* x, uint64_t n_chunks, const Op& op, float qmax,
                                   float* sdec_out, unsigned* sync, bool clear, cudaStream_t s,
-                                  int num_sms, GridWait wait) {
+                                  Device dev, GridWait wait) {
   if (n_chunks <= kClusterMaxChunks)
     return launch_cluster_quant(x, (uint32_t)n_chunks, op, qmax, sdec_out, s);
-  const cudaError_t e = launch_onepass(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms,
+  const cudaError_t e = launch_onepass(x, n_chunks, op, qmax, sdec_out, sync, clear, s, dev,
                                        wait);
   if (e != cudaErrorNotSupported) return e;
-  return launch_two_phase(x, n_chunks, op, qmax, sdec_out, sync, clear, s, num_sms,
+  return launch_two_phase(x, n_chunks, op, qmax, sdec_out, sync, clear, s, dev,
                           wait);
 }
 
 cudaError_t launch_quant_nvfp4_dynamic(const void* x, int64_t M, int64_t K,
                                        const qlin_nvfp4_t& out, unsigned* sync, bool clear,
-                                       cudaStream_t s, int num_sms, GridWait wait) {
+                                       cudaStream_t s, Device dev, GridWait wait) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
   if (n_chunks < (1ull << 32))   // 32-bit index math is enough
     return launch_dynamic(x, n_chunks, nvfp4_op<uint32_t>(K, out), 2688.0f, out.tensor_scale, sync,
-                          clear, s, num_sms, wait);
+                          clear, s, dev, wait);
   return launch_two_phase(x, n_chunks, nvfp4_op<uint64_t>(K, out), 2688.0f, out.tensor_scale, sync,
-                          clear, s, num_sms, wait);
+                          clear, s, dev, wait);
 }
 
 cudaError_t launch_quant_fp8_dynamic(const void* x, int64_t M, int64_t K, const qlin_fp8_t& out,
-                                     unsigned* sync, bool clear, cudaStream_t s, int num_sms,
+                                     unsigned* sync, bool clear, cudaStream_t s, Device dev,
                                      GridWait wait) {
   return launch_dynamic(x, (uint64_t)M * (uint64_t)K / 8, fp8_op(out), 448.0f, out.scale, sync,
-                        clear, s, num_sms, wait);
+                        clear, s, dev, wait);
 }
 
 cudaError_t launch_quant_nvfp4_after(const void* x, int64_t M, int64_t K, const float* scale_src,
-                                     const qlin_nvfp4_t& out, cudaStream_t s, int num_sms,
+                                     const qlin_nvfp4_t& out, cudaStream_t s, Device dev,
                                      unsigned* err, uint64_t timeout_ns) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
-  if (n_chunks >= (1ull << 32)) return launch_quant_nvfp4(x, M, K, scale_src, out, s, num_sms);
-  const cudaError_t e = set_smem<quant_nvfp4_ring_kernel>();
+  if (n_chunks >= (1ull << 32)) return launch_quant_nvfp4(x, M, K, scale_src, out, s, dev);
+  const cudaError_t e = setup<quant_nvfp4_ring_kernel>(dev, kThreads, kSmem).err;
   if (e != cudaSuccess) return e;
-  return launch_pdl(quant_nvfp4_ring_kernel, stream_grid(n_chunks, num_sms), kThreads, kSmem, s,
+  return launch_pdl(quant_nvfp4_ring_kernel, stream_grid(n_chunks, dev.num_sms), kThreads, kSmem, s,
                     static_cast<const uint4*>(x), n_chunks, scale_src, out.tensor_scale,
                     nvfp4_op<uint32_t>(K, out), err, timeout_ns);
 }
 
 cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float* scale_src,
-                               const qlin_nvfp4_t& out, cudaStream_t s, int num_sms) {
+                               const qlin_nvfp4_t& out, cudaStream_t s, Device dev) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
   auto* xin = static_cast<const uint4*>(x);
-  if (n_chunks <= kSmallPerSm * (uint64_t)num_sms)
+  if (n_chunks <= kSmallPerSm * (uint64_t)dev.num_sms)
     return launch_pdl(quant_nvfp4_small_kernel,
                       (int)((n_chunks / 2 + kSmallThreads - 1) / kSmallThreads), kSmallThreads, 0,
                       s, xin, (uint32_t)n_chunks, scale_src, out.tensor_scale,
                       nvfp4_op<uint32_t>(K, out));
   const uint64_t tiles = (n_chunks + kDirectTile - 1) / kDirectTile;
-  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms * kDirectPerSm);
+  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)dev.num_sms * kDirectPerSm);
   auto* codes = reinterpret_cast<uint32_t*>(out.codes);
   const uint3 row_div = invariant_divisor((uint32_t)(K >> 3));
   auto kern = n_chunks < (1ull << 32) ? quant_nvfp4_kernel<uint32_t>   // 32-bit index math is enough
@@ -1350,20 +1347,20 @@ cudaError_t launch_quant_nvfp4(const void* x, int64_t M, int64_t K, const float*
 }
 
 cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* scale_src,
-                             const qlin_fp8_t& out, cudaStream_t s, int num_sms, unsigned* err,
+                             const qlin_fp8_t& out, cudaStream_t s, Device dev, unsigned* err,
                              uint64_t timeout_ns) {
   const uint64_t n_chunks = (uint64_t)M * (uint64_t)K / 8;
-  const cudaError_t e = set_smem<quant_fp8_kernel>();
+  const cudaError_t e = setup<quant_fp8_kernel>(dev, kThreads, kSmem).err;
   if (e != cudaSuccess) return e;
-  return launch_pdl(quant_fp8_kernel, stream_grid(n_chunks, num_sms), kThreads, kSmem, s,
+  return launch_pdl(quant_fp8_kernel, stream_grid(n_chunks, dev.num_sms), kThreads, kSmem, s,
                     static_cast<const uint4*>(x), n_chunks, scale_src, out.scale, fp8_op(out), err,
                     timeout_ns);
 }
 
 cudaError_t launch_quant_fp8_rows(const void* w, int64_t N, int64_t K, const qlin_fp8_t& out,
-                                  cudaStream_t s, int num_sms) {
+                                  cudaStream_t s, Device dev) {
   const int64_t want = (N + kThreads / 32 - 1) / (kThreads / 32);
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms * 8));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)dev.num_sms * 8));
   auto kern = K <= 2 * 256   ? quant_fp8_rows_kernel<2, 4>   // a chunk per lane: 256 of K
               : K <= 4 * 256 ? quant_fp8_rows_kernel<4, 3>
                              : quant_fp8_rows_kernel<12, 2, true>;
