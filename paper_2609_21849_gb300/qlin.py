@@ -178,8 +178,11 @@ class NVFP4Tensor:
                          self.tensor_scale.data_ptr(), self.rows, self.K)
 
     def packed(self) -> bytes:
-        return _pack_nvfp4(self.codes.data_ptr(), self.scales.data_ptr(),
-                           self.tensor_scale.data_ptr(), self.rows, self.K)
+        try:
+            return _pack_nvfp4(self.codes.data_ptr(), self.scales.data_ptr(),
+                               self.tensor_scale.data_ptr(), self.rows, self.K)
+        except struct.error:   # no integer, or out of range: as the structure takes it
+            return bytes(self.desc())
 
 
 @dataclass
@@ -197,8 +200,11 @@ class FP8Tensor:
                        self.per_channel)
 
     def packed(self) -> bytes:
-        return _pack_fp8(self.codes.data_ptr(), self.scale.data_ptr(), self.rows, self.K,
-                         self.per_channel)
+        try:
+            return _pack_fp8(self.codes.data_ptr(), self.scale.data_ptr(), self.rows, self.K,
+                             self.per_channel)
+        except struct.error:
+            return bytes(self.desc())
 
 
 def qlin_nvfp4_scale_bytes(rows: int, K: int) -> int:
