@@ -32,8 +32,7 @@ def nvcc() -> str:
 
 
 def _flags():
-    # QLIN_BUILD_DEFINES: extra -D options (the kernels' build-time layout
-    # choices, e.g. "-DQLIN_GROUP_M=4"); empty for the default build
+    # QLIN_BUILD_DEFINES: extra -D options; empty for the default build
     extra = os.environ.get("QLIN_BUILD_DEFINES", "").split()
     return ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
                    "-I" + INCLUDE, "-I" + CSRC] + extra

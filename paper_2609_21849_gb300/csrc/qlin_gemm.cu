@@ -46,12 +46,6 @@ namespace {
 constexpr int kBM = kTileM;
 constexpr int kRowBytes = kStageRowBytes;   // bytes of K per stage and row: one swizzle row
 constexpr int kStepsPerStage = 4;   // one MMA per 32 bytes of K
-// Tile order: cluster tiles are visited in groups of this many M tile groups
-// (0: all of M, i.e. M fastest within each N tile; on the 4608 x 12288 x 3072
-// NVFP4 GEMM groups of 1 to 9 measured 3-6% slower)
-#ifndef QLIN_GROUP_M
-#define QLIN_GROUP_M 0
-#endif
 constexpr int kSmemBudget = 232448 - 1536;  // opt-in shared memory minus barriers/alignment
 
 constexpr int pow2_at_least(int x) {
@@ -149,22 +143,12 @@ struct KParams {
   uint64_t timeout_ns;
 };
 
-// Coordinates of cluster tile ct: its M tile group and its N tile.  Tiles are
-// visited in groups of kGroup M tile groups (the last group may be smaller),
-// M fastest within a group.
-__device__ __forceinline__ void tile_coords(int ct, int groups_m, int tiles_n, int* mg, int* nb) {
-  constexpr int kGroup = QLIN_GROUP_M;
-  if (kGroup <= 0) {
-    *nb = ct / groups_m;
-    *mg = ct % groups_m;
-    return;
-  }
-  const int per = kGroup * tiles_n;
-  const int grp = ct / per;
-  const int within = ct - grp * per;
-  const int gm = min(kGroup, groups_m - grp * kGroup);
-  *mg = grp * kGroup + within % gm;
-  *nb = within / gm;
+// Coordinates of cluster tile ct, its M tile group and its N tile: M fastest
+// within an N tile.  (Visited in groups of 1 to 9 M tile groups the 4608 x 12288 x
+// 3072 NVFP4 GEMM measured 3-6% slower.)
+__device__ __forceinline__ void tile_coords(int ct, int groups_m, int* mg, int* nb) {
+  *nb = ct / groups_m;
+  *mg = ct % groups_m;
 }
 
 // Bounded wait that ignores the abort flag: used to drain copies and MMAs in
@@ -309,7 +293,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
   // a hundred times over (18432 x 64 x 3072 NVFP4: 12.4 us, now 9.0).
   if (warp == 0 && elect_one()) {
     int mg, nb;
-    tile_coords(cid, groups_m, tiles_n, &mg, &nb);
+    tile_coords(cid, groups_m, &mg, &nb);
     constexpr int kWRows = kBN / kCM / C::kSplit;
     const int w_row = nb * kBN + rank * (kBN / kCM);
     const int boxes = mg == 0 ? min(num_kb, C::kStages) : 0;
@@ -337,7 +321,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     bool ok = true;
     for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
       int mg, nb;
-      tile_coords(ct, groups_m, tiles_n, &mg, &nb);
+      tile_coords(ct, groups_m, &mg, &nb);
       const int a_row = (mg * kCM + rank) * kBM;
       const int w_row = nb * kBN + rank * (kBN / kCM);
       for (int kb = 0; kb < num_kb; ++kb) {
@@ -404,7 +388,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
         // 32 w + lane sit in TMEM column w, so the odd tile's half starts two
         // columns in
         int mg_, nb_;
-        tile_coords(ct, groups_m, tiles_n, &mg_, &nb_);
+        tile_coords(ct, groups_m, &mg_, &nb_);
         const uint32_t sfb_off = kBN < 128 ? 2u * (uint32_t)(nb_ & 1) : 0u;
         if (!mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1u, ctl)) break;
         if (!wait_ready(stage, phase)) break;
@@ -556,7 +540,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     bool ok = true;
     for (int ct = cid; ct < num_ctiles && ok; ct += ncl) {
       int mg, nb;
-      tile_coords(ct, groups_m, tiles_n, &mg, &nb);
+      tile_coords(ct, groups_m, &mg, &nb);
       const int a_row = mg * kCM + rank, w_row = (nb * kBN) >> 7;
       for (int kb = 0; kb < num_kb; ++kb) {
         if (!mbar_wait_warp(&sf_empty[slot], phase ^ 1u, ctl)) {
@@ -676,7 +660,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
         if (lct >= num_ctiles) return;
         if (lkb == 0) {
           int mg, nb;
-          tile_coords(lct, groups_m, tiles_n, &mg, &nb);
+          tile_coords(lct, groups_m, &mg, &nb);
           arow = p.sfa + mg * k64 * 512 + lane * 16;
           wrow = p.sfb + ((nb * kBN) >> 7) * k64 * 512 + lane * 16;
         }
@@ -772,7 +756,7 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
     uint32_t acc_phase = 0;
     for (int ct = cid; ct < num_ctiles; ct += ncl) {
       int mg, nb;
-      tile_coords(ct, groups_m, tiles_n, &mg, &nb);
+      tile_coords(ct, groups_m, &mg, &nb);
       if (!kFp4 && !kBf16 && p.w_per_channel) {
         // FP8: this tile's per-channel weight scales into L1 while the
         // accumulator is still being computed (lane i: the 128-byte line of
@@ -1235,19 +1219,6 @@ cudaError_t dispatch_bn(const GemmArgs& a, cudaStream_t s, Device dev, unsigned*
 }
 
 }  // namespace
-
-CUresult encode_tensor_map_2d_u8(CUtensorMap* map, const void* base, uint64_t inner_bytes,
-                                 uint64_t rows, uint32_t box_inner, uint32_t box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (fn == nullptr) return CUDA_ERROR_NOT_FOUND;
-  const cuuint64_t dims[2] = {inner_bytes, rows};
-  const cuuint64_t strides[1] = {inner_bytes};
-  const cuuint32_t box[2] = {box_inner, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-}
 
 // bf16 (or fp16) [rows, cols] output map: 32 x 32 boxes, 64-byte swizzle (the
 // layout of the epilogue's staging boxes).
