@@ -131,7 +131,7 @@ def test_fp8_weight_per_channel(N, K):
 @pytest.mark.parametrize("fmt", ["nvfp4", "fp8"])
 def test_dynamic_scale_x_larger_than_on_chip(fmt):
     # 9216 x 4096 bf16 (75.5 MB) exceeds what the grid can hold on chip, so
-    # the dynamic scale takes the amax pass + quantizer route; the 4608 x 3072
+    # the dynamic scale takes two phases over x in one launch; the 4608 x 3072
     # cases above take the one-read route.  Both must equal the oracle.
     M, K = 9216, 4096
     x = synthetic.act_entry_outliers(77, M, K)
@@ -148,9 +148,9 @@ def test_dynamic_scale_x_larger_than_on_chip(fmt):
 
 
 def test_dynamic_scale_two_pass_ragged_last_tile():
-    # 9217 x 4096 takes the amax pass + quantizer route and ends in a partial
-    # 16 KB tile (4 719 104 chunks of 16 bytes); the quantizer pass visits
-    # its tiles last-first, so that partial tile is the first it copies.
+    # 9217 x 4096 takes two phases over x and ends in a partial 32 KB tile
+    # (4 719 104 chunks of 16 bytes, 2048 to a tile); the second phase visits
+    # its tiles last-first, from the copies that the first one kept.
     # Rows past the last 128-row atom are a ragged scale block as well.
     M, K = 9217, 4096
     assert (M * K // 8) % 1024 != 0
@@ -161,9 +161,9 @@ def test_dynamic_scale_two_pass_ragged_last_tile():
 
 
 def test_dynamic_scale_one_read_repeated():
-    # the one-read route keeps its grid-wide amax in two scratch words that
-    # each launch clears: back-to-back calls on tensors of decreasing amax
-    # must not see a stale maximum
+    # the one-read route keeps its grid-wide amax in a scratch word that the
+    # last CTA of each launch clears: back-to-back calls on tensors of
+    # decreasing amax must not see a stale maximum
     M, K = 4608, 3072
     ws = qlin.alloc_workspace()
     for seed, gain in ((5, 8.0), (6, 1.0), (7, 0.125)):
@@ -176,15 +176,15 @@ def test_dynamic_scale_one_read_repeated():
 
 
 def test_dynamic_scale_workspace_shared_by_both_routes():
-    # one workspace serves the one-read route (words left zero after each
-    # call) and the two-pass route (its own amax word, cleared before use):
-    # alternate them and each must still equal the oracle
+    # one workspace serves the cluster route (which uses no word of it) and the
+    # two-phase route (words left zero after each call): alternate them and
+    # each must still equal the oracle (test_gpu_routes.py alternates all routes)
     ws = qlin.alloc_workspace()
-    small = synthetic.act_entry_outliers(31, 512, 1024)     # fits on chip
-    large = synthetic.act_normal(32, 9216, 4096)            # does not
+    small = synthetic.act_entry_outliers(31, 512, 1024)     # 1 MB
+    large = synthetic.act_normal(32, 9216, 4096)            # does not fit on chip
     for x in (large, small, large, small):
         M, K = x.shape
         q = qlin.qlin_quantize_act_nvfp4(to_dev(x), None, qlin.alloc_nvfp4(M, K), ws)
         assert qlin.qlin_sync_status() == 0
         assert_nvfp4_equal(q, oracle.quant_nvfp4(x), f"{M}x{K}")
-    assert int(ws[:12].sum()) == 0   # the one-read words are left zeroed
+    assert int(ws[:12].sum()) == 0   # the amax and count words are left zeroed

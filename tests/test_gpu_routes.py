@@ -21,7 +21,8 @@ if torch.cuda.is_available():
 
 # x of n chunks (8 values): 1 MB is 65536 chunks, the cluster route's last
 # size; x in registers reaches 12288 chunks per SM, in shared memory 14336.
-SMS = 152
+SMS = (torch.cuda.get_device_properties(0).multi_processor_count
+       if torch.cuda.is_available() else 152)
 ROUTES = [(1, 64), (3, 64), (17, 448), (256, 2048), (257, 2048), (1023, 512),
           (12288 * SMS // 512, 4096), (12288 * SMS // 512 + 1, 4096),
           (14336 * SMS // 512, 4096), (14336 * SMS // 512 + 1, 4096)]
@@ -47,6 +48,31 @@ def test_dynamic_routes_match_oracle(M, K):
     assert int(ws.count_nonzero()) == 0
 
 
+def test_one_workspace_for_every_route():
+    # every dynamic route and the dynamic chain in turn on one workspace, with
+    # maxima that fall: each leaves it zero for the next
+    ws = qlin.alloc_workspace()
+    shapes = [(256, 512), (1025, 512), (4608, 3072), (13000 * SMS // 512, 4096), (9217, 4096)]
+    xs = [synthetic.act_entry_outliers(50 + i, *s) for i, s in enumerate(shapes)]
+    (w,) = synthetic.weights(60, [(576, 512)], 0.02)
+    W = qlin.qlin_quantize_weight(to_dev(w), qlin.QLIN_FMT_NVFP4)
+    want4 = [oracle.quant_nvfp4(x) for x in xs]
+    want8 = [oracle.quant_fp8(x)[:2] for x in xs]
+    for order in ((4, 3, 2, 1, 0), (0, 2, 4, 1, 3)):
+        for i in order:
+            x = to_dev(xs[i])
+            q4 = qlin.qlin_quantize_act_nvfp4(x, None, None, ws)
+            q8 = qlin.qlin_quantize_act_fp8(x, None, None, ws)
+            A = qlin.qlin_quantize_act_nvfp4(to_dev(xs[1]), None, None, ws)
+            y, yq = qlin.qlin_linear_dynamic(A, W, workspace=ws)
+            assert qlin.qlin_sync_status() == 0
+            assert_nvfp4_equal(q4, want4[i], str(shapes[i]))
+            assert f32(q8.scale)[0] == np.float32(want8[i][1])
+            assert np.array_equal(u8(q8.codes), want8[i][0])
+            assert_nvfp4_equal(yq, oracle.quant_nvfp4(bf16_bits(y)), "chain")
+            assert int(ws.count_nonzero()) == 0
+
+
 @pytest.mark.parametrize("bits", [0x0001, 0x8001, 0x007F, 0x8080, 0x7F7F, 0xFF7F, 0x7F80, 0xFF80,
                                   0x7FC0, 0xFF81, 0x7FFF])
 @pytest.mark.parametrize("M,K", [(3, 64), (1000, 3072), (9217, 4096)])
@@ -69,8 +95,9 @@ def test_maximum_of_extreme_values(M, K, bits):
 @pytest.mark.parametrize("M,K", [(1025, 512), (4608, 3072), (12288 * SMS // 512 + 64, 4096),
                                  (9217, 4096)])
 def test_grid_wait_that_expires_gives_the_same_codes(M, K):
-    # with the shortest wait limit, CTAs that miss the others' arrival read all
-    # of x for the maximum themselves: same codes, no error, scratch left zero
+    # with the shortest wait limit, CTAs that miss the others' arrival read x in
+    # their place (test_gpu_grid_wait.py forces each such path and counts it):
+    # same codes, no error, scratch left zero
     bits = synthetic.act_entry_outliers(7, M, K)
     x, ws = to_dev(bits), qlin.alloc_workspace()
     want4 = qlin.qlin_quantize_act_nvfp4(x, None, None, ws)

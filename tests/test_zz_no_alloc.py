@@ -58,10 +58,10 @@ def test_noalloc_full_size_activation():
 
 
 def test_noalloc_two_pass_route_matches_oracle_twice():
-    # x [9216, 4096] (75 MB) does not fit in the grid's shared memory, so the
-    # entry point takes its two-pass route (an amax pass into the static
-    # scratch, then the quantizer).  Two calls in a row, the second with a
-    # smaller amax: a stale amax left in the scratch would change its scale.
+    # x [9216, 4096] (75 MB) does not fit on chip, so the entry point takes two
+    # phases over it in one launch, its maximum in the static scratch.  Two
+    # calls in a row, the second with a smaller amax: a stale amax left in the
+    # scratch would change its scale.
     M, K = 9216, 4096
     for bits in (synthetic.act_entry_outliers(31, M, K), synthetic.act_normal(32, M, K)):
         out = qlin.qlin_quantize_act_nvfp4_noalloc(_dev(bits), qlin.alloc_nvfp4(M, K))
