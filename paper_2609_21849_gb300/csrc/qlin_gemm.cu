@@ -22,9 +22,9 @@
 //               K = 16; NVFP4 kind::mxf4nvf4 with K = 96, 96 and 64 per 256
 //               elements) into an fp32 TMEM accumulator.
 //   warps 2-5   NVFP4: block scales into TMEM.  Pair tiles: from shared memory
-//               (tcgen05.cp), beside the MMA stream, each warp the atoms of a
-//               quarter of the stage; single-CTA tiles: from global memory
-//               through registers (tcgen05.st), each warp its lane quarter.
+//               (tcgen05.cp), beside the MMA stream, whole stages in turn;
+//               single-CTA tiles: from global memory through registers
+//               (tcgen05.st), each warp its lane quarter.
 //   warp 6      NVFP4 pair tiles: TMA producer of the scale atoms.
 //   last 8      epilogue: tcgen05.ld of the accumulator, alpha, 16-bit
 //               rounding; pair tiles store y straight from registers (the
@@ -287,7 +287,8 @@ __global__ void __launch_bounds__(Cfg<kFp4, kBN, kPair>::kThreads, 1)
 
   // The first W boxes into L2 while the previous kernel still runs: a prefetch
   // is a hint that returns no data, so it is correct even if that kernel
-  // writes W.  (4608 x 3072 x 3072 NVFP4 in a chain of launches: 19.2 -> 18.7 us.)
+  // writes W.  (512 x 1024 x 2560 NVFP4 in a chain of launches: 5.05 -> 4.97 us;
+  // larger GEMMs the same within 0.1 us.)
   // One cluster per W tile does it: the clusters of an N tile share its W, and
   // where all of them prefetched, a tall narrow GEMM asked L2 for the same lines
   // a hundred times over (18432 x 64 x 3072 NVFP4: 12.4 us, now 9.0).

@@ -26,8 +26,6 @@
 // FP8 quantizer and the dynamic chain's NVFP4 one (stream_tiles) cut x into 16 KB
 // tiles that a persistent grid (three CTAs per SM) takes through a four-deep
 // shared-memory ring filled by bulk copies, ~192 KB per SM of input in flight.
-#include <atomic>
-
 #include "qlin_internal.h"
 
 namespace qlin {
@@ -423,11 +421,10 @@ __device__ __forceinline__ float static_scale(const float* scale_src, float* sde
 // NVFP4 with a static scale: x goes straight to registers (32 bytes, one block,
 // per load where x is 32-byte aligned), each thread loading its next tile's
 // units while it quantizes this one's.  Two CTAs of 512 threads per SM keep
-// 64 KB per SM of loads in flight.  Bound by HBM: 18432 x 3072 in 22.4 us
-// (6.5 TB/s), through the shared-memory ring of the other streaming kernels
-// 24.1 us (its block reads have two-way bank conflicts); 4608 x 3072 7.5 us,
-// through the ring 7.8.  256-thread CTAs with one to three units
-// measured 22.3-23.6 us and 7.7-8.6 us.
+// 64 KB per SM of loads in flight.  Bound by HBM: 18432 x 3072 in 22.4-23.2 us
+// (6.2-6.5 TB/s), through the shared-memory ring 24.1-25.5 (its block reads have
+// two-way bank conflicts); 4608 x 3072 7.5 us, through the ring 7.8.  256-thread
+// CTAs with one to three units measured 22.3-23.6 us and 7.7-8.6 us.
 constexpr int kDirectPerSm = 2;
 constexpr int kDirectUnits = 2;                                       // per thread and tile
 constexpr uint32_t kDirectTile = 2u * kThreads * kDirectUnits;        // chunks: 32 KB
@@ -822,8 +819,8 @@ __global__ void __launch_bounds__(kOnePassThreads, 1)
   // copied itself, so waiting for its own copies suffices.  NVFP4 copies in
   // the units run_slice quantizes (two adjacent chunks, a warp covering 1 KB),
   // one copy group per step of block maxima, so that each step's maxima are
-  // taken while the later steps' copies are still landing (4608 x 3072:
-  // 12.46 -> 12.23 us)
+  // taken while the later steps' copies are still landing (4608 x 3072, which
+  // regpass_kernel takes now: 12.46 -> 12.23 us)
   const uint4* xs = x + c_begin;
   if constexpr (Op::kBlockMax) {
 #pragma unroll
@@ -1063,8 +1060,8 @@ __global__ void __launch_bounds__(kThreads, kDirectPerSm)
 // L2 after the first), combines the maxima through distributed shared memory
 // and quantizes its share, so the grid needs no grid-wide barrier.  One
 // 16-element block (two chunks) per thread, loaded first and kept in registers.
-// Bound by latency: launch, one load, one cluster barrier (128 x 256: NVFP4 4.46 -> 2.2 us, FP8 3.4 -> 2.0 us against
-// the grid-wide routes).
+// Bound by latency: launch, one load, one cluster barrier (128 x 256: NVFP4 4.46
+// -> 2.2 us, FP8 3.4 -> 2.0 us against the grid-wide routes).
 constexpr int kClusterCtas = 8;
 constexpr int kClusterThreads = 512;
 constexpr uint32_t kClusterSub = 2 * kClusterThreads;   // chunks a CTA quantizes at most
