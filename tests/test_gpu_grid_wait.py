@@ -122,3 +122,30 @@ def test_two_quantizers_and_a_gemm_on_their_own_streams(fmt):
             assert torch.equal(r.codes, q[0].codes)
     assert torch.equal(y, want)
     assert all(int(w.count_nonzero()) == 0 for w in ws)
+
+
+def test_a_waiting_quantizer_comes_before_the_next_gemm():
+    # two GEMMs on one stream, then a quantizer on another while the first runs:
+    # it starts when that one ends, not when both have
+    (w,) = synthetic.weights(47, [(12288, 3072)], 0.02)
+    W = qlin.qlin_quantize_weight(to_dev(w), qlin.QLIN_FMT_NVFP4)
+    bits = synthetic.act_normal(46, 18432, 3072)
+    A = qlin.qlin_quantize_act_nvfp4(to_dev(bits))
+    y = torch.empty((18432, 12288), dtype=torch.bfloat16, device="cuda")
+    x, q, ws = to_dev(bits[:4608]), qlin.alloc_nvfp4(4608, 3072), qlin.alloc_workspace()
+    gemms, own = torch.cuda.Stream(), torch.cuda.Stream()
+    first = []
+    for _ in range(9):
+        torch.cuda.synchronize()
+        t0, t1, t2 = (torch.cuda.Event(enable_timing=True) for _ in range(3))
+        t0.record(gemms)
+        qlin.qlin_gemm_nvfp4(A, W, y, gemms)
+        qlin.qlin_gemm_nvfp4(A, W, y, gemms)
+        t2.record(gemms)
+        qlin.qlin_quantize_act_nvfp4(x, None, q, ws, own)
+        t1.record(own)
+        torch.cuda.synchronize()
+        first.append(t0.elapsed_time(t1) < t0.elapsed_time(t2))
+    assert sum(first) >= 7, first
+    assert qlin.qlin_sync_status() == 0
+    _check("nvfp4", q, bits[:4608], "beside GEMMs")
