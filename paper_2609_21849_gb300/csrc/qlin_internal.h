@@ -32,7 +32,7 @@ cudaError_t launch_quant_fp8(const void* x, int64_t M, int64_t K, const float* s
                              uint64_t timeout_ns);
 // Limits of the dynamic quantizers' grid-wide wait: for CTAs that have not arrived
 // before the waiting ones read x in their place, then for the last pieces of x.
-// Ten microseconds are several times the CTAs' usual spread.
+// (Limits of 3 and 5 us cost mixes of streams 1-4%, 10 to 200 us nothing.)
 struct GridWait {
   uint64_t help_ns, stop_ns;
 };
